@@ -91,10 +91,9 @@ DET_API det_status_t det_linear_plan_params(int64_t M, int64_t N, int64_t K, det
  * status word and, in the prefill bucket when S > 1, the split-K partials workspace (device); the
  * decode bucket folds its segments inside the kernel and needs none.  Returns NULL on failure
  * (det_last_error(), det_last_status()).
- * A prefill plan also asks for 4 * K * roundup(M, 4) bytes in which every run
- * writes x transposed for its TMA-fed kernel (schedule only; reported as "activation_workspace_bytes"
- * by det_linear_plan_describe, not in workspace_bytes).  If that allocation fails the plan is still
- * created and runs the register-staged kernel, which computes the same bits.
+ * A prefill plan also asks for the schedule workspace of its TMA-fed kernel (a few KB of flags and, where there are more
+ * work units than SMs, 128 KiB per SM of accumulators that blocks hand over; not in workspace_bytes).  If that
+ * allocation fails the plan is still created and runs the register-staged kernel, which computes the same bits.
  * A plan may be used from one stream at a time: its workspace is not re-entrant; make one plan
  * per stream for concurrent use.  Destroy with det_linear_plan_destroy.
  */
@@ -127,8 +126,7 @@ DET_API det_linear_plan_t* det_linear_plan_shard(int64_t M, int64_t N, int64_t K
 /*
  * Enqueue the computation on `stream` (a cudaStream_t; NULL = the legacy default stream) and
  * return without synchronising.  Eq. 2 with the order above; the segment sums are folded in
- * ascending order (R3) -- inside the kernel in the decode bucket, by a second fixed-order pass in the
- * prefill bucket -- never by atomics.
+ * ascending order (R3) -- inside the kernels, or by a second fixed-order pass -- never by atomic sums.
  *   x : device, FP32, [M,K] row-major (row pitch K)
  *   W : device, BF16 bit patterns, [N,K] row-major (row pitch K): one weight row per output column
  *   b : device, FP32, [N], or NULL for no bias (then no final add happens at all)
@@ -200,8 +198,7 @@ DET_API det_status_t det_linear_plan_get_params(const det_linear_plan_t* plan, d
 
 /* Write a JSON description (bucket, V, L, P, S, seg_len, order_version, kernel, workspace_bytes, the shard
  * and, schedule only: for the decode kernel the tiling in use on the current device with its resident
- * blocks per SM, for the prefill kernel the tile, how it is fed ("tma" or "registers") and the bytes of
- * the activation workspace)
+ * blocks per SM, for the prefill kernel the tile and how it is fed ("tma" or "registers"))
  * to buf (at most n bytes including the terminator).  DET_ERR_INVALID_ARG if it does not fit. */
 DET_API det_status_t det_linear_plan_describe(const det_linear_plan_t* plan, char* buf, size_t n);
 

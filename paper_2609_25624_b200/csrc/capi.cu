@@ -69,6 +69,16 @@ static cudaError_t device_alloc(void** p, size_t bytes)
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Tile of the TMA-fed prefill kernel: height / 16 and width.  Variants 5 .. 8 force the height, 25 .. 28, 35 .. 38, 45 .. 48
+// and 55 .. 58 the width (256, 128, 64, 32) too.
+static void prefill_tile(const det_linear_plan_t* plan, int* tm, int* width)
+{
+    const det_linear_params_t& p = plan->prm;
+    const int v = plan->variant, f = v / 10;
+    *tm = v != 0 ? v % 10 : prefill_rows_per_thread(p.M);
+    *width = f >= 2 ? 256 >> (f - 2) : prefill_tile_width(p.M, plan->n_count, p.K, p.S, p.seg_len, *tm, plan->sm_count);
+}
+
 static det_status_t run_device(det_linear_plan_t* plan, const float* x, const void* W, const float* b, float* y,
                                cudaStream_t stream)
 {
@@ -82,10 +92,11 @@ static det_status_t run_device(det_linear_plan_t* plan, const float* x, const vo
     a.x = x; a.W = W; a.b = b; a.y = y;
     a.wfmt = p.weight_format;
     a.partials = plan->partials;
-    // Prefill with 2 .. 4 segments: the block that completes a tile folds it (measured 0.5 - 3 % faster than the second
-    // launch); with more segments the fold of a tile by one block is a longer serial tail than the combine launch
-    // (1 - 5 % slower), so that keeps the second pass.  Test flag 2 forces the second pass.  Same bits either way.
-    a.tile_counters = ((plan->test_flags & 2) || p.S > 4) ? nullptr : plan->tile_counters;
+    // Prefill with several segments: the warps that complete a tile fold it.  Test flag 2 forces the second pass.  Same
+    // bits either way.
+    a.tile_counters = (plan->test_flags & 2) ? nullptr : plan->tile_counters;
+    a.sync = plan->sync;
+    a.handoff = plan->handoff;
     a.M = p.M; a.N = plan->n_count; a.K = p.K;            // the kernels see the shard; the order is the layer's
     a.ldy = plan->ldy;
     a.seg_len = p.seg_len; a.S = p.S;
@@ -128,30 +139,28 @@ static det_status_t run_device(det_linear_plan_t* plan, const float* x, const vo
         }
         e = launch_decode(a, cfg, &plan->map_w, &plan->map_x);
     } else if (kernel == kKernelPrefill) {
-        // the TMA-fed kernel (variant 5 .. 8 forces its rows per thread); without the activation workspace, or with
-        // variant 15 .. 18, the register-staged kernel
+        // the TMA-fed kernel; without its workspace, or with variant 15 .. 18, the register-staged kernel
         const int v = plan->variant;
-        if (!plan->x_t || (v >= 15 && v <= 18)) {
+        if (!plan->sync || (v >= 15 && v <= 18)) {
             e = launch_prefill(a);
         } else {
-            const int tr = (v >= 5 && v <= 8) ? v : prefill_rows_per_thread(p.M);
-            const int cfg_id = 4096 + tr + 1024 * p.weight_format;
-            const int64_t ldt = (p.M + 3) / 4 * 4;
-            e = launch_transpose_x(x, plan->x_t, p.M, p.K, ldt, stream);
-            if (e != cudaSuccess) return cuda_fail("kernel launch", e);
-            if (plan->map_w_ptr != W || plan->map_cfg_id != cfg_id) {
+            int tm, width;
+            prefill_tile(plan, &tm, &width);
+            const int cfg_id = 4096 + tm + 16 * width + 8192 * p.weight_format;
+            if (plan->map_w_ptr != W || plan->map_x_ptr != x || plan->map_cfg_id != cfg_id) {
                 const CUtensorMapDataType wdt = p.weight_format == DET_WEIGHT_FP32   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                                 : p.weight_format == DET_WEIGHT_FP16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                                                                      : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
                 if (!encode_2d(&plan->map_w, wdt, p.weight_format == DET_WEIGHT_FP32 ? 4 : 2, W, (uint64_t)plan->n_count, (uint64_t)p.K,
-                               128u, 32u, CU_TENSOR_MAP_L2_PROMOTION_L2_256B))
+                               (uint32_t)width, 32u, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                               p.weight_format == DET_WEIGHT_FP32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
                     return DET_ERR_CUDA;
-                if (!encode_2d(&plan->map_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, plan->x_t, (uint64_t)p.K, (uint64_t)ldt, 32u,
-                               (uint32_t)(16 * tr), CU_TENSOR_MAP_L2_PROMOTION_L2_256B))
+                if (!encode_2d(&plan->map_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, x, (uint64_t)p.M, (uint64_t)p.K, (uint32_t)(16 * tm), 32u,
+                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_SWIZZLE_128B))
                     return DET_ERR_CUDA;
-                plan->map_w_ptr = W; plan->map_x_ptr = plan->x_t; plan->map_cfg_id = cfg_id;
+                plan->map_w_ptr = W; plan->map_x_ptr = x; plan->map_cfg_id = cfg_id;
             }
-            e = launch_prefill_tma(a, tr, &plan->map_w, &plan->map_x);
+            e = launch_prefill_tma(a, tm, width, &plan->map_w, &plan->map_x);
         }
     } else {
         e = launch_generic(a, p.bucket);
@@ -222,9 +231,10 @@ det_linear_plan_t* det_linear_plan_shard(int64_t M, int64_t N, int64_t K, int64_
     g_last_status = DET_OK;
     e = device_alloc(reinterpret_cast<void**>(&plan->status), sizeof(DeviceStatus));
     if (e == cudaSuccess) e = cudaMemset(plan->status, 0, sizeof(DeviceStatus));
-    // the partials are followed by one counter per output tile of the prefill kernel (at most ceil(M/80) ceil(N/128))
-    const uint64_t counters_at = (prm.workspace_bytes + 255) / 256 * 256;
-    const uint64_t n_counters = (uint64_t)((M + 79) / 80) * (uint64_t)((n_count + 127) / 128);
+    const PrefillWorkspace pw = prm.bucket == 1 ? prefill_workspace(M, n_count, K, prm.S, prm.seg_len, plan->sm_count) : PrefillWorkspace{};
+    // the partials are followed by the counters of the prefill kernel's in-place fold
+    const uint64_t counters_at = (4 * pw.partial_floats + 255) / 256 * 256;
+    const uint64_t n_counters = pw.counter_words;
     if (e == cudaSuccess && prm.workspace_bytes) {
         e = device_alloc(reinterpret_cast<void**>(&plan->partials), counters_at + 4 * n_counters);
         if (e == cudaSuccess) {
@@ -236,16 +246,25 @@ det_linear_plan_t* det_linear_plan_shard(int64_t M, int64_t N, int64_t K, int64_
     if (e != cudaSuccess) {
         g_last_status = DET_ERR_ALLOC;
         set_error("plan: device allocation (status word, %llu bytes of split-K workspace) failed: %s",
-                  (unsigned long long)prm.workspace_bytes, cudaGetErrorString(e));
+                  (unsigned long long)(4 * pw.partial_floats), cudaGetErrorString(e));
         cudaGetLastError();
         det_linear_plan_destroy(plan);              // frees whatever was allocated before the failure
         return nullptr;
     }
-    // Activation workspace of the TMA-fed prefill kernel: x transposed, 4 K roundup(M, 4) bytes.
-    // Without it the plan still works: it uses the register-staged kernel, which computes the same bits.
+    // Schedule workspace of the TMA-fed prefill kernel: a ticket, hand-over flags and, where blocks take equal stretches, the
+    // accumulators handed over.  Without it the plan still works: it uses the register-staged kernel, which computes the same bits.
     if (prm.kernel == kKernelPrefill) {
-        e = device_alloc(reinterpret_cast<void**>(&plan->x_t), 4ull * (uint64_t)((M + 3) / 4 * 4) * (uint64_t)K);
-        if (e != cudaSuccess) { plan->x_t = nullptr; cudaGetLastError(); }
+        const uint64_t handoff_at = (4 * pw.sync_words + 255) / 256 * 256;
+        e = device_alloc(reinterpret_cast<void**>(&plan->sync), handoff_at + 4 * pw.handoff_floats);
+        if (e == cudaSuccess) e = cudaMemset(plan->sync, 0, 4 * pw.sync_words);
+        if (e == cudaSuccess) {
+            plan->n_sync = pw.sync_words;
+            if (pw.handoff_floats) plan->handoff = reinterpret_cast<float*>(reinterpret_cast<char*>(plan->sync) + handoff_at);
+        } else {
+            cudaGetLastError();
+            if (plan->sync) cudaFree(plan->sync);
+            plan->sync = nullptr;
+        }
     }
     return plan;
 }
@@ -434,12 +453,11 @@ det_status_t det_linear_plan_check(det_linear_plan_t* plan, void* stream)
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail("check", e);
     if (h.timeout_flag) {
-        // a block that gave up did not count itself in: bring the tile counters of the in-kernel fold back to zero
-        if (plan->tile_counters) {
-            e = cudaMemsetAsync(plan->tile_counters, 0, 4 * plan->n_tile_counters, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            if (e != cudaSuccess) return cuda_fail("check", e);
-        }
+        // a block that gave up neither counted itself in nor handed its work over: back to zero
+        if (plan->tile_counters) e = cudaMemsetAsync(plan->tile_counters, 0, 4 * plan->n_tile_counters, st);
+        if (e == cudaSuccess && plan->sync) e = cudaMemsetAsync(plan->sync, 0, 4 * plan->n_sync, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return cuda_fail("check", e);
         set_error("check: a kernel gave up a bounded wait (site %u)", h.where);
         return DET_ERR_DEVICE_TIMEOUT;
     }
@@ -469,11 +487,11 @@ det_status_t det_linear_plan_describe(const det_linear_plan_t* plan, char* buf, 
     char ptile[160] = "null";
     if (p.kernel == kKernelPrefill) {
         const int v = plan->variant;
-        const bool staged = !plan->x_t || (v >= 15 && v <= 18);
-        const int tr = (v >= 5 && v <= 8) ? v : (v >= 15 && v <= 18) ? v - 10 : prefill_rows_per_thread(p.M);
-        snprintf(ptile, sizeof ptile, "{\"bm\": %d, \"bn\": 128, \"bk\": 32, \"feed\": \"%s\", \"activation_workspace_bytes\": %llu}",
-                 16 * tr, staged ? "registers" : "tma",
-                 plan->x_t ? 4ull * (unsigned long long)((p.M + 3) / 4 * 4) * (unsigned long long)p.K : 0ull);
+        const bool staged = !plan->sync || (v >= 15 && v <= 18);
+        int tm, width = 128;
+        if (staged) tm = (v >= 15 && v <= 18) ? v - 10 : prefill_rows_per_thread(p.M);
+        else prefill_tile(plan, &tm, &width);
+        snprintf(ptile, sizeof ptile, "{\"bm\": %d, \"bn\": %d, \"bk\": 32, \"feed\": \"%s\"}", 16 * tm, width, staged ? "registers" : "tma");
     }
     int w = snprintf(buf, n,
                      "{\"M\": %lld, \"N\": %lld, \"K\": %lld, \"bucket\": \"%s\", \"V\": %d, \"L\": %d, \"P\": %d, "
@@ -492,7 +510,7 @@ void det_linear_plan_destroy(det_linear_plan_t* plan)
 {
     if (!plan) return;
     if (plan->partials) cudaFree(plan->partials);
-    if (plan->x_t) cudaFree(plan->x_t);
+    if (plan->sync) cudaFree(plan->sync);
     if (plan->status) cudaFree(plan->status);
     if (plan->x_stage) cudaFree(plan->x_stage);
     if (plan->y_stage) cudaFree(plan->y_stage);
@@ -545,9 +563,9 @@ det_status_t det_test_plan_set_variant(det_linear_plan_t* plan, int variant)
             set_error("set_variant: the decode kernel has fewer than %d tilings for this batch size", variant);
             return DET_ERR_INVALID_ARG;
         }
-    } else if (variant != 0 && (variant < 5 || variant > 8) && (variant < 15 || variant > 18)) {
-        set_error("set_variant: the prefill bucket takes 0 (automatic), 5 .. 8 (rows per thread) or 15 .. 18 (the same with "
-                  "the register-staged kernel)");
+    } else if (variant != 0 && (variant >= 60 || variant % 10 < 5 || variant % 10 > 8)) {
+        set_error("set_variant: the prefill bucket takes 0 (automatic), 5 .. 8 (tile height / 16), 15 .. 18 (the same with "
+                  "the register-staged kernel) or 25 .. 28, 35 .. 38, 45 .. 48, 55 .. 58 (tiles 256, 128, 64, 32 wide)");
         return DET_ERR_INVALID_ARG;
     }
     plan->variant = variant;

@@ -37,7 +37,9 @@ struct LaunchArgs {
     float* y;             // final output [M,N], row pitch ldy
     int64_t ldy;          // floats between consecutive rows of y (N unless the plan is a column shard)
     float* partials;      // [S,M,N] when S > 1, else nullptr
-    unsigned* tile_counters;   // prefill with S > 1: one zeroed counter per output tile (the TMA-fed kernel folds in place), or nullptr
+    unsigned* tile_counters;   // prefill with S > 1: zeroed counters per output tile and warp (the TMA-fed kernel folds in place), or nullptr
+    unsigned* sync;       // TMA-fed prefill kernel: zeroed ticket and hand-over flags
+    float* handoff;       // prefill in equal stretches: accumulators on their way from one block to the next, or nullptr
     int64_t M, N, K;
     int64_t seg_len;
     int S;
@@ -57,12 +59,15 @@ cudaError_t launch_combine(const LaunchArgs& a);
 // Register-staged prefill kernel (the fallback without an activation workspace; a.variant 15 .. 18 forces 5 .. 8 rows
 // per thread).
 cudaError_t launch_prefill(const LaunchArgs& a);
-// Prefill kernel with both tiles fed by TMA (prefill_tma.cu).  It reads the
-// activations from a workspace xT [K][ldt] (x transposed, ldt = M rounded up to a multiple of 4; launch_transpose_x
-// writes it).  Tensor maps without swizzle: map_x: xT, box [32][16 tr]; map_w: W [N][K] in its format, box [128][32].
-cudaError_t launch_transpose_x(const float* x, float* xT, int64_t M, int64_t K, int64_t ldt, cudaStream_t stream);
-cudaError_t launch_prefill_tma(const LaunchArgs& a, int tr, const CUtensorMap* map_w, const CUtensorMap* map_x);
-// rows per thread (tile height = 16 x this) the prefill kernel uses for batch size M; schedule only
+// Prefill kernel with both tiles fed by TMA (prefill_tma_kernel.cuh); block tile 16 tm rows x width columns.  Tensor maps,
+// swizzled over the width of the box: map_x: x [M][K], box [16 tm][32]; map_w: W [N][K] in its format, box [width][32].
+cudaError_t launch_prefill_tma(const LaunchArgs& a, int tm, int width, const CUtensorMap* map_w, const CUtensorMap* map_x);
+int prefill_tile_width(int64_t M, int64_t N, int64_t K, int S, int64_t seg_len, int tm, int sm_count);
+// Device memory the TMA-fed kernel wants: split-K partials by tile with their counters; ticket, flags and accumulators of
+// the hand-over between blocks (no accumulators when every unit of work gets a block of its own).
+struct PrefillWorkspace { uint64_t partial_floats, counter_words, sync_words, handoff_floats; };
+PrefillWorkspace prefill_workspace(int64_t M, int64_t N, int64_t K, int S, int64_t seg_len, int sm_count);
+// tile height / 16 the prefill kernels use for batch size M (the register-staged kernel: rows per thread); schedule only
 int prefill_rows_per_thread(int64_t M);
 // Fixed-order RMSNorm of M rows of H elements (rmsnorm.cu).
 cudaError_t launch_rmsnorm(const float* x, const float* g, float eps, int64_t M, int64_t H, float* y, cudaStream_t stream);
@@ -102,7 +107,9 @@ struct det_linear_plan {
     float* partials;                 // device, S*M*n_count floats or nullptr
     unsigned* tile_counters;         // device, inside the partials allocation (prefill, S > 1) or nullptr
     uint64_t n_tile_counters;
-    float* x_t;                      // device, K * roundup(M, 4) floats: x transposed (prefill bucket) or nullptr
+    unsigned* sync;                  // device, prefill: ticket and hand-over flags of the TMA-fed kernel, or nullptr
+    uint64_t n_sync;
+    float* handoff;                  // device, in the same allocation: accumulators handed over from block to block, or nullptr
     int64_t n_begin, n_count, ldy;   // column shard computed by this plan (0, N, N for a whole layer)
     detlin::DeviceStatus* status;    // device
     float* x_stage;                  // device staging for det_linear_run_host

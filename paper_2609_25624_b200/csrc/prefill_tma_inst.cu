@@ -1,0 +1,92 @@
+// Launchers of the TMA-fed prefill kernel for one weight format (compiled once per format, DET_WF = 0 BF16, 1 FP16, 2 FP32)
+// and every tile: heights 80, 96, 112 and 128, widths 256, 128, 64 and 32.
+#include "prefill_tma_kernel.cuh"
+
+namespace detlin {
+
+namespace {
+
+using namespace prefill_detail;
+
+template <int WF, int TR, int TC, int LX, int LY>
+cudaError_t launch_t(const LaunchArgs& la, const CUtensorMap* map_w, const CUtensorMap* map_x)
+{
+    typedef Tile<WF, TR, TC, LX, LY> T;
+    static bool configured[kMaxDevices];             // function attributes belong to a device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    auto kern = prefill_tma_kernel<WF, TR, TC, LX, LY>;
+    if (!configured[dev]) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kSmemBytes);
+        if (e != cudaSuccess) return e;
+        configured[dev] = true;
+    }
+    const long long tiles_m = (la.M + T::BM - 1) / T::BM, tiles_n = (la.N + T::BN - 1) / T::BN;
+    const long long units = tiles_m * tiles_n * la.S;
+    if (units > 0x7fffffffLL) return cudaErrorInvalidValue;
+    Args a{};
+    a.bias = la.b; a.y = la.y; a.partials = la.partials; a.handoff = la.handoff; a.sync = la.sync;
+    a.tile_counters = la.tile_counters; a.status = la.status;
+    a.ldy = la.ldy;
+    a.M = (int)la.M; a.N = (int)la.N; a.K = (int)la.K;
+    a.seg_slabs = (int)(la.seg_len / BK);
+    a.tile_slabs = (int)((la.K + BK - 1) / BK);
+    a.S = la.S; a.tiles_m = (int)tiles_m;
+    a.total = tiles_m * tiles_n * a.tile_slabs;
+    a.wait_limit_ns = la.wait_limit_ns;
+    a.test_flags = la.test_flags;
+    // Equal stretches as soon as the units need more than one wave.  A unit may be cut once only, so a stretch is at least
+    // a segment long.
+    long long grid = units;
+    if (units > la.sm_count && la.handoff) {
+        a.cut = 1;
+        const long long most = a.total / (a.seg_slabs < a.tile_slabs ? a.seg_slabs : a.tile_slabs);
+        grid = most < la.sm_count ? most : la.sm_count;
+    }
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(T::kThreads);
+    cfg.dynamicSmemBytes = T::kSmemBytes;
+    cfg.stream = la.stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kern, *map_x, *map_w, a);
+    if (e != cudaSuccess) return e;
+    if (la.S > 1 && !la.tile_counters) return launch_combine(la);
+    return cudaSuccess;
+}
+
+// tile height 16 TM
+template <int WF, int TM>
+cudaError_t launch_h(const LaunchArgs& a, int width, const CUtensorMap* map_w, const CUtensorMap* map_x)
+{
+    switch (width) {
+    case 256: return launch_t<WF, 2 * TM, 8, 32, 8>(a, map_w, map_x);
+    case 128: return launch_t<WF, 8, 8, 16, 2 * TM>(a, map_w, map_x);
+    case 64: return launch_t<WF, 4, 8, 8, 4 * TM>(a, map_w, map_x);
+    case 32: return launch_t<WF, 4, 4, 8, 4 * TM>(a, map_w, map_x);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace
+
+#define DET_CAT2(a, b) a##b
+#define DET_PREFILL_NAME(wf) DET_CAT2(launch_prefill_tma_wf, wf)
+cudaError_t DET_PREFILL_NAME(DET_WF)(const LaunchArgs& a, int tm, int width, const CUtensorMap* map_w, const CUtensorMap* map_x)
+{
+    switch (tm) {
+    case 5: return launch_h<DET_WF, 5>(a, width, map_w, map_x);
+    case 6: return launch_h<DET_WF, 6>(a, width, map_w, map_x);
+    case 7: return launch_h<DET_WF, 7>(a, width, map_w, map_x);
+    case 8: return launch_h<DET_WF, 8>(a, width, map_w, map_x);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace detlin
