@@ -206,13 +206,14 @@ det_linear_plan_t* det_linear_plan_shard(int64_t M, int64_t N, int64_t K, int64_
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) { g_last_status = cuda_fail("cudaGetDevice", e); return nullptr; }
-    cudaDeviceProp prop;
-    e = cudaGetDeviceProperties(&prop, dev);
-    if (e != cudaSuccess) { g_last_status = cuda_fail("cudaGetDeviceProperties", e); return nullptr; }
-    if (prop.major != 10) {
+    int major = 0, minor = 0, sms = 0;                // (single attributes: cudaGetDeviceProperties takes milliseconds)
+    e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) { g_last_status = cuda_fail("plan: device query", e); return nullptr; }
+    if (major != 10) {
         g_last_status = DET_ERR_ARCH;
-        set_error("plan: device %d is sm_%d%d; this library is built for sm_100a only (no fallback)", dev, prop.major,
-                  prop.minor);
+        set_error("plan: device %d is sm_%d%d; this library is built for sm_100a only (no fallback)", dev, major, minor);
         return nullptr;
     }
     det_linear_plan_t* plan = new (std::nothrow) det_linear_plan_t();
@@ -223,7 +224,7 @@ det_linear_plan_t* det_linear_plan_shard(int64_t M, int64_t N, int64_t K, int64_
     plan->n_count = n_count;
     plan->ldy = ldy;
     plan->device = dev;
-    plan->sm_count = prop.multiProcessorCount;
+    plan->sm_count = sms;
     plan->forced_kernel = -1;
     plan->map_cfg_id = -1;
     plan->decode_cfg_variant = -1;
