@@ -276,8 +276,10 @@ DET_API det_status_t det_attention_decode(const float* q, const float* k, const 
  *
  * The first call on each device looks up the array's device address (with that device current);
  * make that first call before starting any stream capture.  The address is kept for the life of the
- * process: after a cudaDeviceReset the library must be reloaded before this entry point is used again.  The kernels are the library's generic
- * ones (any shape and alignment, not tuned for speed).  Enqueues on `stream`, no synchronisation.
+ * process: after a cudaDeviceReset the library must be reloaded before this entry point is used again.  The kernels are
+ * those of det_linear_run (the prefill bucket without cutting work units across thread blocks, which needs a
+ * workspace); W and b may be written by the kernel before this call in the stream.  There is no plan to ask about an
+ * expired wait.  Enqueues on `stream`, no synchronisation.
  */
 DET_API det_status_t det_linear_run_noalloc(int64_t M, int64_t N, int64_t K, const float* x, const uint16_t* W,
                                             const float* b, float* y, void* stream);

@@ -79,8 +79,7 @@ static void prefill_tile(const det_linear_plan_t* plan, int* tm, int* width)
     *width = f >= 2 ? 256 >> (f - 2) : prefill_tile_width(p.M, plan->n_count, p.K, p.S, p.seg_len, *tm, plan->sm_count);
 }
 
-static det_status_t run_device(det_linear_plan_t* plan, const float* x, const void* W, const float* b, float* y,
-                               cudaStream_t stream)
+det_status_t run_device(det_linear_plan_t* plan, const float* x, const void* W, const float* b, float* y, cudaStream_t stream)
 {
     const det_linear_params_t& p = plan->prm;
     int dev = -1;

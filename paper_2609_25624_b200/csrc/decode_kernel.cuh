@@ -135,8 +135,9 @@ __device__ __forceinline__ void consumer_barrier(int threads)
     asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
 }
 
-// Test hook bits (LaunchArgs::test_flags): never set outside the tests.
+// LaunchArgs::test_flags: bit 0 is a test hook, never set outside the tests.
 constexpr int kTestWithholdFirstX = 1;   // block 0 never requests the activations of its first stage
+constexpr int kLateWeights = kFlagLateWeights;   // weights and bias too are touched only after the previous kernel in the stream
 
 
 template <int MT, int WM, int RT, int WR, int SK, int KC, int STAGES, int WF>
@@ -257,7 +258,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
         // once, activation requests wait for that kernel to finish.  A thread that requests both sends the
         // first ring of weight requests ahead of the wait.
         int pre = 0;
-        if (do_w && do_x) {
+        if (do_w && do_x && !(test_flags & kLateWeights)) {
             const Cursor c0 = c;
             const bool live0 = live;
             while (live && pre < STAGES) {
@@ -268,7 +269,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
             c = c0;
             live = live0;
         }
-        if (do_x) pdl_wait();
+        if (do_x || (test_flags & kLateWeights)) pdl_wait();
         int st = 0;
         unsigned phase = 0, n_issued = 0;
         bool ok = true;
@@ -297,6 +298,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
 
     // ---------------- consumer warps ----------------
     if (C::kMoveRegs) reg_inc<C::kConsumerRegs>();
+    if (test_flags & kLateWeights) pdl_wait();                // (the bias is read ahead of the output's wait)
     const int g = warp / C::kGroupWarps;
     const int gw = warp % C::kGroupWarps;
     const int wm = gw % WM;

@@ -23,6 +23,10 @@ struct DeviceStatus {
     unsigned int where;          // which wait (diagnostic)
 };
 
+// LaunchArgs::test_flags beyond the test hooks: the decode kernel also waits for the previous kernel in the stream before it
+// touches W and b (callers for whom they are not parameters that were complete long before)
+constexpr int kFlagLateWeights = 4;
+
 constexpr int kMaxDevices = 64;     // per-device caches (function attributes, symbol addresses)
 
 void set_error(const char* fmt, ...);
@@ -129,3 +133,10 @@ struct det_linear_plan {
     CUtensorMap map_w;
     CUtensorMap map_x;
 };
+
+namespace detlin {
+
+// One run on the plan's device buffers (capi.cu): alignment checks, choice of the kernel, tensor maps, launch.
+det_status_t run_device(det_linear_plan_t* plan, const float* x, const void* W, const float* b, float* y, cudaStream_t stream);
+
+}  // namespace detlin

@@ -8,7 +8,8 @@
 // on the host: the split-K partials live in a fixed array that is part of the library image.
 //
 // The paper has no counterpart for this entry point; it computes exactly the same thing (same
-// order, same bits) as det_linear_plan + det_linear_run.
+// order, same bits, same kernels) as det_linear_plan + det_linear_run.  With the generic kernels that it used before,
+// M = 3, N = K = 4096 took 44.8 us a call.
 #include "internal.h"
 #include <mutex>
 
@@ -19,27 +20,41 @@ namespace detlin {
 constexpr size_t kNoallocScratchFloats = (size_t)1 << 20;
 static __device__ __align__(256) float g_noalloc_scratch[kNoallocScratchFloats];
 
-static float* g_scratch_addr[kMaxDevices];      // device address of the array, per device
+// Status word (first two words) and the schedule words that the prefill kernel expects beside it (all zero, not written
+// here: they only matter to blocks that hand work over, which needs a workspace this entry point does not have).
+static __device__ __align__(256) unsigned g_noalloc_words[64];
+
+struct NoallocAddresses {
+    float* scratch;
+    unsigned* words;
+};
+static NoallocAddresses g_addr[kMaxDevices];    // device addresses of the arrays, per device
 static std::mutex g_scratch_mutex;
 
-// In host code `g_noalloc_scratch` is only a handle for the runtime, not a device address; the
+// In host code the arrays are only handles for the runtime, not device addresses; the
 // address a kernel can use has to be asked for, once per device, with that device current.
-static cudaError_t scratch_address(float** out)
+static cudaError_t static_addresses(int dev, NoallocAddresses* out)
 {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(g_scratch_mutex);
-    if (!g_scratch_addr[dev]) {
-        void* p = nullptr;
-        e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
+    if (!g_addr[dev].words) {
+        void *p = nullptr, *q = nullptr;
+        cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
+        if (e == cudaSuccess) e = cudaGetSymbolAddress(&q, g_noalloc_words);
         if (e != cudaSuccess) return e;
-        g_scratch_addr[dev] = static_cast<float*>(p);
+        g_addr[dev].scratch = static_cast<float*>(p);
+        g_addr[dev].words = static_cast<unsigned*>(q);
     }
-    *out = g_scratch_addr[dev];
+    *out = g_addr[dev];
     return cudaSuccess;
 }
+
+// The decode tiling depends on the shape and the device only; a loop that repeats a shape does not search again.
+static thread_local struct {
+    int64_t M, N, K;
+    int dev;
+    DecodeConfig cfg;
+} g_last_tiling;
 
 }  // namespace detlin
 
@@ -59,28 +74,48 @@ extern "C" det_status_t det_linear_run_noalloc(int64_t M, int64_t N, int64_t K, 
                   p.S, (unsigned long long)(need * 4), (unsigned long long)(kNoallocScratchFloats * 4));
         return DET_ERR_UNSUPPORTED_SHAPE;
     }
-    int dev = 0, major = 0;
+    int dev = 0, major = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) { set_error("run_noalloc: device query: %s", cudaGetErrorString(e)); return DET_ERR_CUDA; }
     if (major != 10) {
         set_error("run_noalloc: device %d is sm_%dx; this library is built for sm_100a only (no fallback)", dev, major);
         return DET_ERR_ARCH;
     }
-    float* scratch = nullptr;
-    e = scratch_address(&scratch);
+    NoallocAddresses at{};
+    e = static_addresses(dev, &at);
     if (e != cudaSuccess) {
         set_error("run_noalloc: cudaGetSymbolAddress failed: %s", cudaGetErrorString(e));
         return DET_ERR_CUDA;
     }
-    LaunchArgs a{};
-    a.x = x; a.W = W; a.b = b; a.y = y;
-    a.wfmt = DET_WEIGHT_BF16;
-    a.partials = need ? scratch : nullptr;       // every partial is written by the first pass before the
-    a.M = M; a.N = N; a.K = K; a.ldy = N;                   // second pass reads it: nothing has to start at zero
-    a.seg_len = p.seg_len; a.S = p.S;
-    a.stream = static_cast<cudaStream_t>(stream);
-    e = launch_generic(a, p.bucket);
-    if (e != cudaSuccess) { set_error("run_noalloc: kernel launch: %s", cudaGetErrorString(e)); return DET_ERR_CUDA; }
-    return DET_OK;
+    // A plan on the stack, without memory of its own: the same kernels as det_linear_run.  No in-kernel fold of prefill
+    // segments (its counters would be shared by calls of different shapes) and no stretches cut across blocks.
+    det_linear_plan_t plan{};
+    plan.prm = p;
+    plan.device = dev;
+    plan.sm_count = sms;
+    plan.partials = need ? at.scratch : nullptr;            // every partial is written by the first pass before the
+                                                            // second pass reads it: nothing has to start at zero
+    plan.status = reinterpret_cast<DeviceStatus*>(at.words);
+    plan.sync = at.words + 8;
+    plan.n_count = N;
+    plan.ldy = N;
+    plan.forced_kernel = -1;
+    plan.wait_limit_ns = kDefaultWaitLimitNs;
+    plan.test_flags = kFlagLateWeights;                     // nothing was said here about W and b being older than the stream's last kernel
+    plan.decode_cfg_variant = -1;
+    plan.map_cfg_id = -1;
+    auto& t = g_last_tiling;
+    const bool decode = p.kernel == kKernelDecode;
+    if (decode && t.M == M && t.N == N && t.K == K && t.dev == dev) {
+        plan.decode_cfg = t.cfg;
+        plan.decode_cfg_variant = 0;
+    }
+    st = run_device(&plan, x, W, b, y, static_cast<cudaStream_t>(stream));
+    if (st == DET_OK && decode && plan.decode_cfg_variant == 0) {
+        t.M = M; t.N = N; t.K = K; t.dev = dev;
+        t.cfg = plan.decode_cfg;
+    }
+    return st;
 }

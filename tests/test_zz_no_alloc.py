@@ -68,3 +68,21 @@ def test_noalloc_rejects_shapes_beyond_the_builtin_scratch():
     assert str(prm.workspace_bytes) in msg and str(4 << 20) in msg
     rc = B.lib().det_linear_run_noalloc(1, 8, 8, None, None, None, None, None)
     assert rc == 1
+
+
+@pytest.mark.parametrize("M,N,K", [(64, 520, 1024), (1, 20000, 264), (65, 300, 40), (100, 1000, 1000), (3000, 9000, 256)])
+def test_noalloc_fast_kernels_with_weights_written_just_before(M, N, K):
+    """The kernels of the planned path, on aligned buffers: decode with and without a split, prefill with one unit per
+    thread block (more units than SMs too) and a second pass.  The weights are written by the stream's previous kernel."""
+    x, W, b = inputs.make_case(M, N, K)
+    xd, Wd, bd = x.cuda(), W.cuda(), b.cuda()
+    assert B.det_linear_plan_params(M, N, K).workspace_bytes <= (4 << 20)
+    want = run_gpu(x, W, b) if M * N * K > 2e9 else oracle_y(x, W, b)
+    W2, b2 = torch.empty_like(Wd), torch.empty_like(bd)
+    y = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    b2.copy_(bd)
+    W2.copy_(Wd)
+    B.det_linear_run_noalloc(xd, W2, b2, y)
+    torch.cuda.synchronize()
+    assert_bits_equal(y.cpu().numpy(), want, f"{M},{N},{K}")
