@@ -116,7 +116,7 @@ def lib() -> ctypes.CDLL:
 
 
 def _check(status):
-    if status != DET_OK:
+    if status:
         raise DetLinearError(status, det_last_error())
 
 
@@ -139,8 +139,18 @@ def det_linear_plan_params(M: int, N: int, K: int) -> Params:
     return out
 
 
+# The raw handle of the current stream, without building a torch.cuda.Stream object around it: 0.2 us instead of 3.3 us,
+# a third of what a small layer took.
+try:
+    _raw_current_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+except AttributeError:                           # a torch without CUDA
+    _raw_current_stream = None
+
+
 def _stream_ptr(stream):
     if stream is None:
+        if _raw_current_stream is not None:
+            return _raw_current_stream(_current_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -170,6 +180,9 @@ class Plan:
             self._h = lib().det_linear_plan_w(self.M, self.N, self.K, self.wfmt)
         if not self._h:
             raise DetLinearError(det_last_status(), det_last_error())
+        # what a run looks up on every call
+        self._x_shape, self._w_shape, self._b_shape, self._y_shape = (self.M, self.K), (self.N, self.K), (self.N,), (self.M, self.N)
+        self._run = lib().det_linear_run if self.wfmt == DET_WEIGHT_BF16 else lib().det_linear_run_w
 
     def close(self):
         if getattr(self, "_h", None):
@@ -236,22 +249,26 @@ def det_linear_plan_describe(plan: Plan) -> dict:
     return json.loads(buf.value.decode())
 
 
+_F32 = torch.float32
+
+
 def _expect(t, dtype, shape, name):
-    if not t.is_cuda or t.dtype != dtype or tuple(t.shape) != tuple(shape) or not t.is_contiguous():
+    if t.dtype is not dtype or t.shape != shape or not t.is_cuda or not t.is_contiguous():
         raise ValueError(f"{name}: need a contiguous CUDA tensor of dtype {dtype} and shape {tuple(shape)}, "
                          f"got {t.dtype} {tuple(t.shape)} cuda={t.is_cuda}")
 
 
 def det_linear_run(plan: Plan, x, W, b, y, stream=None) -> None:
     """Enqueue y = x . up(W)^T (+ b) on `stream` (default: torch's current stream)."""
-    _expect(x, torch.float32, (plan.M, plan.K), "x")
-    _expect(W, plan.w_dtype, (plan.N, plan.K), "W")
-    _expect(y, torch.float32, (plan.M, plan.N), "y")
+    _expect(x, _F32, plan._x_shape, "x")
+    _expect(W, plan.w_dtype, plan._w_shape, "W")
+    _expect(y, _F32, plan._y_shape, "y")
     if b is not None:
-        _expect(b, torch.float32, (plan.N,), "b")
-    fn = lib().det_linear_run if plan.wfmt == DET_WEIGHT_BF16 else lib().det_linear_run_w
-    _check(fn(plan.handle, x.data_ptr(), W.data_ptr(), b.data_ptr() if b is not None else None,
-              y.data_ptr(), _stream_ptr(stream)))
+        _expect(b, _F32, plan._b_shape, "b")
+        b = b.data_ptr()
+    status = plan._run(plan._h, x.data_ptr(), W.data_ptr(), b, y.data_ptr(), _stream_ptr(stream))
+    if status:
+        _check(status)
 
 
 def det_linear_run_w(plan: Plan, x, W, b, y, stream=None) -> None:
