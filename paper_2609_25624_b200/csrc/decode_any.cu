@@ -1,0 +1,299 @@
+// Decode order (V=4, L=32, P=1, S segments) for any K and any alignment (K % 8 != 0, misaligned buffers); compiled once per
+// weight format (DET_WF = 0 BF16, 1 FP16, 2 FP32).
+//
+// A warp owns RT weight rows and MT batch rows: lane l owns k = c + 4l + j in every 128-element chunk of a segment and
+// accumulates them in ascending order into one chain per output; the 32 lane sums of an output are added adjacent-first;
+// segment sums are added in ascending order as the warp goes (rule R3).
+//
+// What bounds it: with rows that start anywhere, TMA and vector loads are out, and a warp that walks its row chunk by
+// chunk waits for memory every time (the kernel before this one did, and read the row again for every batch row).
+//   * weights go from memory to registers, a group of UC chunks of every row loaded ahead of the group that is
+//     being multiplied.  16-bit rows start on any 2-byte boundary: a lane loads the two or three aligned words that hold
+//     its four weights, two byte permutations line them up (rows at the very ends of W, where such a word would reach
+//     outside of W, and the last partial chunk of a row are loaded element by element);
+//   * activations sit in shared memory, rows padded to whole chunks; the warps of a block share them.  The padding is
+//     -0.0 and weights beyond K count as +0: the product is -0.0, and adding -0.0 changes no accumulator (not even a
+//     -0.0 one), so elements beyond K are skipped in effect without a test in the loop;
+//   * two rows' chains advance in one packed FMA (RT > 1), the lane sums of all outputs fold in one butterfly.
+// Measured on B200, us a call in a chain, before -> now: M = 6, N = 1333, K = 1001 15.8 -> 7.4; M = 3, N = K = 4097 49.6 -> 16.4;
+// M = 64, N = 8192, K = 4097 1705 -> 218 (27 % of the FP32 peak: line-up and widening of every weight in every batch
+// block, one-word loads); M = 64, N = 300, K = 333 68 -> 6; 20 x 2000 x 2001 with FP16 weights 92 -> 21.
+#include "internal.h"
+#include "device_utils.cuh"
+
+namespace detlin {
+
+namespace {
+
+constexpr int kAnySmemBytes = 110 * 1024;            // activations of one window of K with two blocks of 8 warps per SM ...
+constexpr int kAnySmemBytes1 = 220 * 1024;           // ... or one block of 16
+
+template <int WF, int MT, int RT>
+__global__ void __launch_bounds__(512, 1)
+decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::type* __restrict__ W, const float* __restrict__ b,
+                  float* __restrict__ y, int M, int N, unsigned K, unsigned seg_len, long long ldy, unsigned win, int groups)
+{
+    typedef typename WeightElem<WF>::type WT;
+    constexpr int UC = 8 / RT;                       // chunks of a row loaded together
+    constexpr int NW = WF == 2 ? 4 : 3;              // words a lane loads of a chunk
+    extern __shared__ __align__(16) float xs[];      // [MT][win]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, threads = blockDim.x;
+    const int m0 = blockIdx.y * MT;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    // activations of the window [w_lo, w_lo + win) into shared memory
+    auto stage = [&](unsigned w_lo) {
+        const unsigned len = min(win, K - w_lo);
+        const uint32_t base = (uint32_t)__cvta_generic_to_shared(xs);
+#pragma unroll 1
+        for (int m = 0; m < MT; ++m) {
+            const float* src = x + (size_t)min(m0 + m, M - 1) * K + w_lo;     // rows beyond M repeat the last one
+#pragma unroll 4
+            for (unsigned i = threadIdx.x; i < len; i += threads)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(base + (m * win + i) * 4u), "l"(src + i) : "memory");
+            for (unsigned i = len + threadIdx.x; i < win; i += threads) xs[m * win + i] = -0.0f;
+        }
+        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    };
+
+    const bool one_window = K <= win;
+    for (int grp = (int)blockIdx.x; grp < groups; grp += (int)gridDim.x) {
+        const int n0 = (grp * (threads >> 5) + warp) * RT;
+
+        // The warp's rows, as the word that holds the lane's first weight, and how the lane's words are lined up: bytes
+        // 0 .. 3 of two words for rows that start on a word, bytes 2 .. 5 for the others.  A warp with a row at
+        // which such a word could reach outside of W loads by elements.
+        const uint32_t* pw[RT];
+        uint32_t sel[RT];
+        bool by_word = true;
+#pragma unroll
+        for (int r = 0; r < RT; ++r) {
+            const int n = min(n0 + r, N - 1);        // rows beyond N repeat the last one; their sums are not stored
+            const uintptr_t at = reinterpret_cast<uintptr_t>(W + (size_t)n * K + 4 * lane);
+            const bool odd = WF != 2 && (at & 2u) != 0;
+            pw[r] = reinterpret_cast<const uint32_t*>(at & ~(uintptr_t)3);
+            sel[r] = odd ? 0x5432u : 0x3210u;
+            if (odd && (n == 0 || n == N - 1)) by_word = false;
+        }
+        uint32_t raw[2][UC][RT][NW];
+        // one chunk of every row, `u` chunks behind the words' position, by words
+        auto load_words = [&](uint32_t (&v)[RT][NW], int u) {
+#pragma unroll
+            for (int r = 0; r < RT; ++r) {
+                if constexpr (WF == 2) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) v[r][j] = __ldg(pw[r] + 128 * u + j);
+                } else {
+                    v[r][0] = __ldg(pw[r] + 64 * u);
+                    v[r][1] = __ldg(pw[r] + 64 * u + 1);
+                    if (sel[r] == 0x5432u) v[r][2] = __ldg(pw[r] + 64 * u + 2);
+                }
+            }
+        };
+        // the chunks of [c, end): whole ones by words, a partial one by elements; the words advance
+        auto load = [&](uint32_t (&v)[UC][RT][NW], unsigned c, unsigned end) {
+            if (by_word && end - c == 128 * UC) {
+#pragma unroll
+                for (int u = 0; u < UC; ++u) load_words(v[u], u);
+            } else {
+#pragma unroll
+                for (int u = 0; u < UC; ++u) {
+                    if (by_word && c + 128 * u + 128 <= end) load_words(v[u], u);
+                    else if (c + 128 * u < end) {
+                        const unsigned k = c + 128 * u + 4 * lane;
+#pragma unroll
+                        for (int r = 0; r < RT; ++r) {
+                            const WT* p = W + (size_t)min(n0 + r, N - 1) * K + k;
+                            uint32_t e[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                if constexpr (WF == 2) e[j] = k + j < end ? __float_as_uint(__ldg(p + j)) : 0u;
+                                else e[j] = k + j < end ? (uint32_t)__ldg(p + j) : 0u;
+                            }
+                            if constexpr (WF == 2) {
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) v[u][r][j] = e[j];
+                            } else {
+                                v[u][r][0] = e[0] | (e[1] << 16);
+                                v[u][r][1] = e[2] | (e[3] << 16);
+                            }
+                        }
+                    }
+                }
+            }
+            const unsigned step = (end - c) * sizeof(WT) / 4;        // (a partial chunk is the row's last: not used after it)
+#pragma unroll
+            for (int r = 0; r < RT; ++r) pw[r] += step;
+        };
+        float acc[MT][RT];
+        float tot[Scatter<MT * RT>::kKeep];
+        auto multiply = [&](const uint32_t (&v)[RT][NW], const float* xl, bool words) {
+            float w[RT][4];
+#pragma unroll
+            for (int r = 0; r < RT; ++r) {
+                if constexpr (WF == 2) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) w[r][j] = __uint_as_float(v[r][j]);
+                } else {
+                    const uint32_t sl = words ? sel[r] : 0x3210u;
+                    const uint32_t lo = __byte_perm(v[r][0], v[r][1], sl), hi = __byte_perm(v[r][1], v[r][2], sl);
+                    w[r][0] = up16_lo<WF>(lo); w[r][1] = up16_hi<WF>(lo);
+                    w[r][2] = up16_lo<WF>(hi); w[r][3] = up16_hi<WF>(hi);
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < MT; ++m) {
+                const float4 xv = *reinterpret_cast<const float4*>(xl + m * win);
+                const float xk[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if constexpr (RT == 1) {
+                        acc[m][0] = __fmaf_rn(xk[j], w[0][j], acc[m][0]);
+                    } else {
+#pragma unroll
+                        for (int r = 0; r < RT; r += 2) {
+                            const float2 t = __ffma2_rn(make_float2(xk[j], xk[j]), make_float2(w[r][j], w[r + 1][j]), make_float2(acc[m][r], acc[m][r + 1]));
+                            acc[m][r] = t.x;
+                            acc[m][r + 1] = t.y;
+                        }
+                    }
+                }
+            }
+        };
+
+        // groups of up to UC chunks, never across the end of a segment or of a window
+        auto group_end = [&](unsigned c, unsigned s_hi, unsigned w_hi) { return min(min(K, s_hi), min(w_hi, c + 128 * UC)); };
+        bool first = true;                           // no segment has ended yet
+        unsigned w_hi = win, w_lo = ~0u;             // end of the window of the group loaded last; start of the one in shared memory
+        unsigned s_hi = seg_len;                     // end of the segment of the group being multiplied
+        unsigned c = 0, c_end = group_end(0, s_hi, w_hi);
+        load(raw[0], c, c_end);
+#pragma unroll
+        for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int r = 0; r < RT; ++r) acc[m][r] = 0.0f;
+        int buf = 0;
+#pragma unroll 1
+        while (c < K) {
+            if (one_window ? (w_lo != 0 && grp == (int)blockIdx.x) : (w_lo == ~0u || c - w_lo >= win)) {
+                w_lo = one_window ? 0 : c;
+                __syncthreads();                     // everybody has finished with the window before
+                stage(w_lo);
+                __syncthreads();
+            }
+            const bool seg_done = c_end == min(K, s_hi);
+            if (seg_done) s_hi += seg_len;
+            if (c_end == w_hi) w_hi += win;
+            const unsigned nc_end = c_end < K ? group_end(c_end, s_hi, w_hi) : c_end;
+            const float* xl = xs + (one_window ? c : c - w_lo) + 4 * lane;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {   // (the buffers are registers: their index has to be a constant)
+                if (buf == half) {
+                    if (nc_end != c_end) load(raw[half ^ 1], c_end, nc_end);
+                    if (c_end - c == 128 * UC) {
+#pragma unroll
+                        for (int u = 0; u < UC; ++u) multiply(raw[half][u], xl + 128 * u, by_word);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < UC; ++u)
+                            if (c + 128 * u < c_end) multiply(raw[half][u], xl + 128 * u, by_word && c + 128 * u + 128 <= c_end);
+                    }
+                }
+            }
+            buf ^= 1;
+            if (seg_done) {
+                float v[MT * RT];
+#pragma unroll
+                for (int m = 0; m < MT; ++m)
+#pragma unroll
+                    for (int r = 0; r < RT; ++r) { v[m * RT + r] = acc[m][r]; acc[m][r] = 0.0f; }
+                lane_tree_scatter<MT * RT>(v, lane);
+#pragma unroll
+                for (int t = 0; t < Scatter<MT * RT>::kKeep; ++t) tot[t] = first ? v[t] : __fadd_rn(tot[t], v[t]);
+                first = false;
+            }
+            c = c_end;
+            c_end = nc_end;
+        }
+        constexpr int kSteps = Scatter<MT * RT>::kSteps;
+        if ((lane >> kSteps) == 0) {
+            int base = 0, cnt = MT * RT;
+#pragma unroll
+            for (int i = 0; i < kSteps; ++i) { cnt >>= 1; base += ((lane >> i) & 1) * cnt; }
+#pragma unroll
+            for (int t = 0; t < Scatter<MT * RT>::kKeep; ++t) {
+                const int idx = base + t;
+                const int m = m0 + idx / RT, n = n0 + idx % RT;
+                if (m < M && n < N) y[m * ldy + n] = b ? __fadd_rn(tot[t], __ldg(b + n)) : tot[t];
+            }
+        }
+    }
+}
+
+template <int WF, int MT, int RT>
+cudaError_t launch_t(const LaunchArgs& a, long long mblocks, int sms)
+{
+    static bool configured[kMaxDevices];             // function attributes belong to a device
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    auto kern = decode_any_kernel<WF, MT, RT>;
+    if (!configured[dev]) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kAnySmemBytes1);
+        if (e != cudaSuccess) return e;
+        configured[dev] = true;
+    }
+    // Two blocks of 8 warps per SM, or one of 16 where only that keeps all activations of a batch block in shared memory; the
+    // window holds whole chunks of 128.
+    const long long padded = (a.K + 127) / 128 * 128, cap = kAnySmemBytes / 4 / MT / 256 * 256, cap1 = kAnySmemBytes1 / 4 / MT / 256 * 256;
+    const bool big = padded > cap;
+    const int warps = big ? 16 : 8;
+    const unsigned win = (unsigned)(!big ? padded : padded < cap1 ? padded : cap1);
+    const long long groups = (a.N + warps * RT - 1) / (warps * RT);
+    long long grid = (big ? 1ll : 2ll) * sms / mblocks;
+    if (grid < 1) grid = 1;
+    if (a.max_blocks > 0 && grid > a.max_blocks) grid = a.max_blocks;
+    if (grid > groups) grid = groups;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3((unsigned)grid, (unsigned)mblocks);
+    cfg.blockDim = dim3(32 * warps);
+    cfg.dynamicSmemBytes = (size_t)MT * win * 4;
+    cfg.stream = a.stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, a.x, static_cast<const typename WeightElem<WF>::type*>(a.W), a.b, a.y, (int)a.M, (int)a.N,
+                              (unsigned)a.K, (unsigned)a.seg_len, (long long)a.ldy, win, (int)groups);
+}
+
+template <int WF, int MT>
+cudaError_t launch_m(const LaunchArgs& a)
+{
+    const long long mblocks = (a.M + MT - 1) / MT;
+    const int sms = a.sm_count > 0 ? a.sm_count : 148;
+    // Rows per warp: four from 8 warps' worth of work per SM on, two from 4, one for smaller layers (they need the warps).
+    // Measured, us with four / two rows against the next smaller number: M = 3, N = K = 4097 22.8 (four) 16.4 (two) 28.7 (one);
+    // M = 1, N = 1333, K = 1001 3.3 (two) 6.9 (one); M = 6 likewise 7.4 (two) 8.7 (one).
+    const long long rows = a.N * mblocks;
+    if (rows >= 4ll * 8 * sms) return launch_t<WF, MT, 4>(a, mblocks, sms);
+    if (rows >= 2ll * 4 * sms) return launch_t<WF, MT, 2>(a, mblocks, sms);
+    return launch_t<WF, MT, 1>(a, mblocks, sms);
+}
+
+}  // namespace
+
+#define DET_CAT2(a, b) a##b
+#define DET_CAT(a, b) DET_CAT2(a, b)
+cudaError_t DET_CAT(launch_decode_any_wf, DET_WF)(const LaunchArgs& a)
+{
+    if (a.M <= 1) return launch_m<DET_WF, 1>(a);
+    if (a.M <= 2) return launch_m<DET_WF, 2>(a);
+    if (a.M <= 4) return launch_m<DET_WF, 4>(a);
+    return launch_m<DET_WF, 8>(a);
+}
+
+}  // namespace detlin

@@ -42,4 +42,50 @@ __device__ __forceinline__ float lane_tree_sum(float a)
     return a;
 }
 
+// Butterfly reduce-scatter that realises the adjacent-first lane tree for NV values per lane at once.  At
+// step i (i = 0..4) lanes l and l ^ (1 << i) are partners.  While the number of values a lane holds is
+// even, the partners exchange halves and add (the lane with bit i set keeps the upper half), so the work
+// per step halves; afterwards the remaining steps add whole arrays.  kSteps = number of halving steps,
+// kKeep = values a lane holds at the end (v[0 .. kKeep)); they are the sums of the values with index
+// base + t, base = sum over halving steps i of bit_i(lane) * (NV >> (i + 1)); lanes whose bits
+// kSteps .. 4 are zero hold distinct results.
+template <int NV>
+struct Scatter {
+    static constexpr int steps()
+    {
+        int n = NV, h = 0;
+        while (h < 5 && n % 2 == 0) { n /= 2; ++h; }
+        return h;
+    }
+    static constexpr int kSteps = steps();
+    static constexpr int kKeep = NV >> kSteps;
+};
+
+template <int NV>
+__device__ __forceinline__ void lane_tree_scatter(float (&v)[NV], int lane)
+{
+    constexpr int H = Scatter<NV>::kSteps;
+    int n = NV;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const int d = 1 << i;
+        if (i < H) {
+            const int half = n >> 1;
+            const bool hi = (lane >> i) & 1;
+#pragma unroll
+            for (int t = 0; t < NV / 2; ++t) {
+                if (t < half) {
+                    const float send = hi ? v[t] : v[t + half];
+                    const float keep = hi ? v[t + half] : v[t];
+                    v[t] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, d));
+                }
+            }
+            n = half;
+        } else {
+#pragma unroll
+            for (int t = 0; t < Scatter<NV>::kKeep; ++t) v[t] = __fadd_rn(v[t], __shfl_xor_sync(0xffffffffu, v[t], d));
+        }
+    }
+}
+
 }  // namespace detlin

@@ -1,0 +1,52 @@
+"""The decode kernel for any K and alignment against the oracle, bit for bit: chunk, group and segment edges, activations
+that need several windows of shared memory, weight rows on every 2- or 4-byte offset, special values at a ragged end."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_25624_b200 import binding as B
+from paper_2609_25624_b200 import inputs
+from tests.gpu_util import KERNEL_GENERIC, assert_bits_equal, oracle_y, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+# one, two and four rows a warp; batches on both sides of 1, 2, 4, 8; K around 128, 256 (segment), 1024 and beyond one window
+@pytest.mark.parametrize("M,N,K", [(1, 1, 1), (1, 9, 129), (2, 1300, 255), (3, 700, 257), (5, 5000, 127), (9, 2400, 385), (64, 700, 131),
+                                   (1, 4800, 1025), (8, 33, 7169), (4, 70, 14211), (1, 17, 57001), (17, 40, 2049)])
+@pytest.mark.parametrize("wfmt", ["bf16", "fp32"])
+def test_ragged_sizes(M, N, K, wfmt):
+    x, W, b = inputs.make_case_w(M, N, K, wfmt)
+    assert_bits_equal(run_gpu(x, W, b, kernel=KERNEL_GENERIC), oracle_y(x, W, b), f"{M},{N},{K} {wfmt}")
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3, 5])
+@pytest.mark.parametrize("wfmt", ["bf16", "fp16", "fp32"])
+def test_misaligned_weights_and_activations(offset, wfmt):
+    M, N, K = 6, 1300, 640                           # whole chunks: the rows differ in alignment by the offset only
+    x, W, b = inputs.make_case_w(M, N, K, wfmt)
+    Wd = torch.empty(N * K + offset, dtype=W.dtype, device="cuda")[offset:].view(N, K)
+    xd = torch.empty(M * K + offset, dtype=x.dtype, device="cuda")[offset:].view(M, K)
+    Wd.copy_(W)
+    xd.copy_(x)
+    y = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+    plan = B.det_linear_plan_w(M, N, K, wfmt)
+    B.det_linear_run(plan, xd, Wd, b.cuda(), y)
+    B.det_linear_plan_check(plan)
+    plan.close()
+    assert_bits_equal(y.cpu().numpy(), oracle_y(x, W, b), f"offset {offset} {wfmt}")
+
+
+def test_padding_changes_no_accumulator():
+    """A chain that ends on -0.0 (an underflowing negative product) keeps its sign, infinities and NaN stay what they are:
+    the elements beyond K are skipped, not added."""
+    M, N, K = 3, 20, 133
+    x = torch.zeros(M, K)
+    x[0, :] = -1e-30
+    x[1, 5] = float("inf")
+    x[2, :] = torch.randn(K, generator=torch.Generator().manual_seed(1))
+    W = torch.full((N, K), 1e-30).to(torch.bfloat16)
+    W[1::2] = 1.0
+    want, got = oracle_y(x, W, None), run_gpu(x, W, None, kernel=KERNEL_GENERIC)
+    assert np.array_equal(np.isnan(got), np.isnan(want))
+    assert_bits_equal(np.nan_to_num(got, nan=0.0, posinf=1.0), np.nan_to_num(want, nan=0.0, posinf=1.0), "special values")
