@@ -128,15 +128,19 @@ det_status_t run_device(det_linear_plan_t* plan, const float* x, const void* W, 
             const CUtensorMapDataType wdt = p.weight_format == DET_WEIGHT_FP32   ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                             : p.weight_format == DET_WEIGHT_FP16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                                                                  : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-            if (!encode_2d(&plan->map_w, wdt, p.weight_format == DET_WEIGHT_FP32 ? 4 : 2, W, (uint64_t)plan->n_count, (uint64_t)p.K,
-                           (uint32_t)(cfg.rt * cfg.wr), (uint32_t)(cfg.kc < 256 ? cfg.kc : 256), CU_TENSOR_MAP_L2_PROMOTION_L2_256B))
+            const int w_bytes = p.weight_format == DET_WEIGHT_FP32 ? 4 : 2;
+            const uint32_t kb = (uint32_t)(cfg.kc < 256 ? cfg.kc : 256);
+            if (!encode_2d(&plan->map_w, wdt, w_bytes, W, (uint64_t)plan->n_count, (uint64_t)p.K, (uint32_t)(cfg.rt * cfg.wr), kb,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B) ||
+                !encode_2d(&plan->map_g, wdt, w_bytes, W, (uint64_t)plan->n_count, (uint64_t)p.K, (uint32_t)cfg.rt, kb,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B))
                 return DET_ERR_CUDA;
             if (!encode_2d(&plan->map_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, x, (uint64_t)p.M, (uint64_t)p.K,
                            (uint32_t)(cfg.mt * cfg.wm), (uint32_t)(cfg.kc < 256 ? cfg.kc : 256), CU_TENSOR_MAP_L2_PROMOTION_L2_256B))
                 return DET_ERR_CUDA;
             plan->map_w_ptr = W; plan->map_x_ptr = x; plan->map_cfg_id = cfg.id + 1024 * p.weight_format;
         }
-        e = launch_decode(a, cfg, &plan->map_w, &plan->map_x);
+        e = launch_decode(a, cfg, &plan->map_w, &plan->map_g, &plan->map_x);
     } else if (kernel == kKernelPrefill) {
         // the TMA-fed kernel; without its workspace, or with variant 15 .. 18, the register-staged kernel
         const int v = plan->variant;

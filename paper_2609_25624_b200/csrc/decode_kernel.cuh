@@ -13,10 +13,13 @@
 // pairing is invisible in the bits.
 //
 // Everything else is schedule and therefore numerically inert (supplement C on rule R2: tile
-// sizes, warp counts and pipeline depth do not change the reduction tree).  A thread block owns
-// one (row tile, batch block) work unit at a time and ALL its K segments: SK groups of WM x WR
+// sizes, warp counts and pipeline depth do not change the reduction tree).  The weight rows are dealt out to
+// the thread blocks in tiles of WR row groups (RT rows, one warp's share); of the tall tiles, what is left after whole
+// rounds is dealt out by row groups, so that a block's last tile holds fewer (its other warps then leave the schedulers to
+// the rest): 28672 rows on 148 blocks are 3.5 tiles of 56 rows for everybody instead of 4 for some.  A block works on
+// one (row tile, batch block) at a time and ALL its K segments: SK groups of WM x WR
 // consumer warps work on SK segments side by side (each group has its own ring of stages, fed by
-// one producer thread), the remaining segments follow in further rounds, and the block folds the S
+// one producer warp), the remaining segments follow in further rounds, and the block folds the S
 // segment sums itself -- in registers when SK = 1, through shared memory otherwise -- so no
 // workspace, no atomics and no second launch are needed.  Rule R4 holds by construction: nothing
 // that touches the order reads M.
@@ -89,6 +92,12 @@ struct Cfg {
     static constexpr int kRingBytes = SK * STAGES * kStageBytes;
     static constexpr int kBarBytes = (16 * SK * STAGES + 16 + 127) / 128 * 128;   // full + empty barriers, abort flag
     static constexpr int kTile = kMB * kRB;                   // outputs of a work unit
+    // Deal out what is left after whole rounds?  Batches of more than 8 rows are bound by the multiply loop, and a last round
+    // that is nearly empty costs a whole tile: for the tall tiles, 3.46 -> 3.5 instead of 4 rounds at 28672 rows (M = 16: 84.0
+    // -> 78.8 us).  Below that the weight stream binds, which the blocks of a thin last round share out among themselves (M = 8,
+    // 128256 rows: 200 us without, 207 with), and tiles of 28 rows lose more by the extra bookkeeping (M = 32, 1 %) than
+    // their smaller rounds leave to gain.
+    static constexpr bool kDealRest = kMB >= 16 && kRB >= 56;
     static constexpr int kFixedSmem = kRingBytes + kBarBytes + 128;               // + 128 for alignment
     static constexpr int kLM = ilog2(MT);
     static constexpr int kKeep = RT / 2;                      // sums a lane holds after the lane tree
@@ -140,11 +149,22 @@ constexpr int kTestWithholdFirstX = 1;   // block 0 never requests the activatio
 constexpr int kLateWeights = kFlagLateWeights;   // weights and bias too are touched only after the previous kernel in the stream
 
 
+// Tensor map of a single row group: a parameter only of the tilings that use it.
+template <bool DEAL> struct GroupMap { typedef CUtensorMap type; };
+template <> struct GroupMap<false> { typedef int type; };
+
+// How the row groups are dealt out: n_shares shares of whole_rounds tiles each, then rest_each groups for everybody and
+// one more for the first rest_more shares.
+struct Shares {
+    int n_shares, whole_rounds, rest_each, rest_more;
+};
+
 template <int MT, int WM, int RT, int WR, int SK, int KC, int STAGES, int WF>
 __global__ void __launch_bounds__((Cfg<MT, WM, RT, WR, SK, KC, STAGES, WF>::kThreads), (Cfg<MT, WM, RT, WR, SK, KC, STAGES, WF>::kMinBlocks))
 decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
+              const __grid_constant__ typename GroupMap<Cfg<MT, WM, RT, WR, SK, KC, STAGES, WF>::kDealRest>::type map_g,
               const float* __restrict__ bias, float* __restrict__ y, int M, int N, int K, int seg_len, int S,
-              int n_row_tiles, int n_mblocks, long long ldy, DeviceStatus* status, unsigned long long wait_limit_ns,
+              const Shares sh, int n_mblocks, long long ldy, DeviceStatus* status, unsigned long long wait_limit_ns,
               int test_flags)
 {
     using C = Cfg<MT, WM, RT, WR, SK, KC, STAGES, WF>;
@@ -186,11 +206,26 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
     }
     pdl_launch_dependents();
 
-    const int total_units = n_row_tiles * n_mblocks;          // the host keeps this below 2^31
+    const int total_shares = sh.n_shares * n_mblocks;         // the host keeps this below 2^31
+    const int last_tile = C::kDealRest ? sh.whole_rounds : 0;      // number of a share's last tile
     const int rounds = S / SK;                                // the host only picks tilings with S % SK == 0
 
-    // Work unit u -> (batch block fastest, then row tile): the batch blocks of one row tile run side
-    // by side, so the tile's weights come from HBM once and from L2 for the other blocks.
+    // Share v -> (batch block fastest, then row groups): the batch blocks of the same rows run side by side, so the weights
+    // come from HBM once and from L2 for the other blocks.  A share has whole_rounds tiles of WR row groups, dealt out
+    // round robin, and one last tile of its part of the remaining groups (at most WR; none if grp == grp_hi).
+    // Without dealing out the rest (C::kDealRest), a share is one tile.
+    auto tile_of = [&](int v, int k, int& grp, int& grp_hi, int& mb) {
+        int i = v;
+        mb = 0;
+        if (n_mblocks > 1) { i = v / n_mblocks; mb = v - i * n_mblocks; }
+        if (!C::kDealRest || k < sh.whole_rounds) {
+            grp = (k * sh.n_shares + i) * WR;
+            grp_hi = grp + WR;
+        } else {
+            grp = sh.whole_rounds * sh.n_shares * WR + i * sh.rest_each + min(i, sh.rest_more);
+            grp_hi = grp + sh.rest_each + (i < sh.rest_more ? 1 : 0);
+        }
+    };
     auto seg_range = [&](int s, int& k_lo, int& k_hi) {
         k_lo = s * seg_len;
         k_hi = min(K, k_lo + seg_len);
@@ -212,16 +247,23 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
         const uint32_t emptyg = empty0 + 8 * g * STAGES;
         const uint32_t ringg = smem_base + (uint32_t)(g * STAGES * C::kStageBytes);
 
-        // Position in the group's stream of stages: work unit (row tile, batch block), round, first k.
+        // Position in the group's stream of stages: share, tile of the share, its row groups and batch block, round, first k.
         struct Cursor {
-            int u, tile, mb, r, k0, k_hi;
+            int v, t, grp, grp_hi, mb, r, k0, k_hi;
+        };
+        // the first tile that is not empty from (c.v, c.t) on
+        auto find_tile = [&](Cursor& c) -> bool {
+            for (; c.v < total_shares; c.v += (int)gridDim.x, c.t = 0)
+                for (; c.t <= last_tile; ++c.t) {
+                    tile_of(c.v, c.t, c.grp, c.grp_hi, c.mb);
+                    if (!C::kDealRest || c.grp < c.grp_hi) return true;
+                }
+            return false;
         };
         auto start = [&](Cursor& c) -> bool {
-            c.u = (int)blockIdx.x;
-            c.r = 0;
-            if (c.u >= total_units) return false;
-            c.tile = c.u / n_mblocks;
-            c.mb = c.u - c.tile * n_mblocks;
+            c.v = (int)blockIdx.x;
+            c.t = c.r = 0;
+            if (!find_tile(c)) return false;
             seg_range(g, c.k0, c.k_hi);
             return true;
         };
@@ -230,10 +272,8 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
             if (c.k0 < c.k_hi) return true;
             if (++c.r == rounds) {
                 c.r = 0;
-                c.u += (int)gridDim.x;
-                if (c.u >= total_units) return false;
-                c.tile = c.u / n_mblocks;
-                c.mb = c.u - c.tile * n_mblocks;
+                ++c.t;
+                if (!find_tile(c)) return false;
             }
             seg_range(c.r * SK + g, c.k0, c.k_hi);
             return true;
@@ -243,12 +283,21 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
         // announcement: the phase cannot complete before the announcing arrival).
         auto issue = [&](int st, const Cursor& c, bool w, bool x) {
             const uint32_t fb = fullg + 8 * st;
-            if (w) mbar_arrive_expect_tx(fb, C::kStageBytes);
+            const int n_grp = C::kDealRest ? c.grp_hi - c.grp : WR;
+            if (w) mbar_arrive_expect_tx(fb, C::kSubs * (C::kXBytes + n_grp * RT * C::kWPitch));
 #pragma unroll
             for (int sub = 0; sub < C::kSubs; ++sub) {
                 const uint32_t dst = ringg + (uint32_t)(st * C::kStageBytes + sub * C::kSubBytes);
-                if (w) tma_load_2d(dst + C::kXBytes, &map_w, c.k0 + sub * C::kKB, c.tile * C::kRB, fb, pol_w);
-                if (x) tma_load_2d(dst, &map_x, c.k0 + sub * C::kKB, c.mb * C::kMB, fb, pol_x);
+                const int k = c.k0 + sub * C::kKB;
+                if (w) {
+                    if (n_grp == WR) {
+                        tma_load_2d(dst + C::kXBytes, &map_w, k, c.grp * RT, fb, pol_w);
+                    } else if constexpr (C::kDealRest) {
+                        for (int i = 0; i < n_grp; ++i)     // part of a tile: one box per row group
+                            tma_load_2d(dst + C::kXBytes + i * RT * C::kWPitch, &map_g, k, (c.grp + i) * RT, fb, pol_w);
+                    }
+                }
+                if (x) tma_load_2d(dst, &map_x, k, c.mb * C::kMB, fb, pol_x);
             }
         };
 
@@ -322,9 +371,16 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
     // there when the multiply loop needs it.
     bool ready = false;
     constexpr int kKeep = C::kKeep;
-    for (int u = (int)blockIdx.x; u < total_units; u += (int)gridDim.x) {
-        const int mb = u % n_mblocks;
-        const int tile = u / n_mblocks;
+
+    for (int v = (int)blockIdx.x; v < total_shares; v += (int)gridDim.x)
+#pragma unroll 1
+    for (int t = 0; t <= last_tile; ++t) {
+        int mb, grp, grp_hi;
+        tile_of(v, t, grp, grp_hi, mb);
+        if (C::kDealRest && grp == grp_hi) continue;
+        const int n_tile = C::kDealRest ? (grp_hi - grp) * RT : C::kRB;      // weight rows of this tile
+        const int row0 = grp * RT;                            // its first row
+        const bool mine = !C::kDealRest || wr * RT < n_tile;  // the last tile of a share may have no rows for this warp
         float tot[kKeep];                                     // running fold over the segments when SK == 1
 
         for (int r = 0; r < rounds; ++r) {
@@ -390,7 +446,9 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                         }
                     }
                 };
-                if (k0 + KC <= k_hi) {
+                if (!mine) {
+                    ready = false;                            // no rows here: only keeps the ring in step
+                } else if (k0 + KC <= k_hi) {
                     // whole stage inside the segment: no per-lane test
                     {
 #pragma unroll(MT * RT >= 64 ? 1 : 2)
@@ -478,17 +536,18 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                 if (r == rounds - 1) {
                     // ---- bias and store straight from the owner lanes ----
                     const int m = mb * C::kMB + wm * MT + m_slot;
-                    const int n0 = tile * C::kRB + wr * RT + b0;
+                    const int n0 = row0 + wr * RT + b0;
+                    const int n_hi = min(N, row0 + n_tile);       // (rows beyond the range are another block's)
                     float bv[kKeep];
 #pragma unroll
-                    for (int j = 0; j < kKeep; ++j) bv[j] = (bias != nullptr && owner && n0 + 2 * j < N) ? __ldg(bias + n0 + 2 * j) : 0.0f;
+                    for (int j = 0; j < kKeep; ++j) bv[j] = (bias != nullptr && owner && n0 + 2 * j < n_hi) ? __ldg(bias + n0 + 2 * j) : 0.0f;
                     // the output buffer may still be read by the previous kernel in the stream
                     if (!waited) { pdl_wait(); waited = true; }
                     if (ok && owner && m < M) {
 #pragma unroll
                         for (int j = 0; j < kKeep; ++j) {
                             const int n = n0 + 2 * j;
-                            if (n < N) y[(long long)m * ldy + n] = bias ? __fadd_rn(tot[j], bv[j]) : tot[j];
+                            if (n < n_hi) y[(long long)m * ldy + n] = bias ? __fadd_rn(tot[j], bv[j]) : tot[j];
                         }
                     }
                 }
@@ -500,7 +559,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
             // (the bias of the thread's first output is requested before the barrier: its latency hides there)
             float b_first = 0.0f;
             {
-                const int n = tile * C::kRB + (int)threadIdx.x % C::kRB;
+                const int n = row0 + (int)threadIdx.x % C::kRB;
                 if (bias != nullptr && (int)threadIdx.x < C::kTile && n < N) b_first = __ldg(bias + n);
             }
             consumer_barrier(C::kConsumerWarps * 32);
@@ -509,8 +568,8 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
             if (!aborting) {
                 for (int o = threadIdx.x; o < C::kTile; o += C::kConsumerWarps * 32) {
                     const int ml = o / C::kRB, nl = o % C::kRB;
-                    const int m = mb * C::kMB + ml, n = tile * C::kRB + nl;
-                    if (m < M && n < N) {
+                    const int m = mb * C::kMB + ml, n = row0 + nl;
+                    if (m < M && nl < n_tile && n < N) {
                         float t = part[o];
                         for (int s2 = 1; s2 < S; ++s2) t = __fadd_rn(t, part[s2 * C::kTile + o]);
                         if (bias) t = __fadd_rn(t, o == (int)threadIdx.x ? b_first : __ldg(bias + n));
@@ -519,14 +578,14 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                 }
             }
             consumer_barrier(C::kConsumerWarps * 32);         // the partial tiles are rewritten by the next unit
-            if (aborting) break;                              // uniform: every warp read the flag after the same barrier
+            if (aborting) return;                             // uniform: every warp read the flag after the same barrier
         } else {
-            if (!ok) break;
+            if (!ok) return;
         }
     }
 }
 
-typedef cudaError_t (*DecodeLaunchFn)(const LaunchArgs&, const CUtensorMap*, const CUtensorMap*);
+typedef cudaError_t (*DecodeLaunchFn)(const LaunchArgs&, const CUtensorMap*, const CUtensorMap*, const CUtensorMap*);
 typedef int (*DecodeOccupancyFn)(int S);
 
 // Resident blocks per SM of one tiling for an order with S segments (also opts the kernel into its
@@ -566,18 +625,27 @@ int decode_occupancy_t(int S)
 }
 
 template <int MT, int WM, int RT, int WR, int SK, int KC, int STAGES, int WF>
-cudaError_t launch_decode_t(const LaunchArgs& a, const CUtensorMap* map_w, const CUtensorMap* map_x)
+cudaError_t launch_decode_t(const LaunchArgs& a, const CUtensorMap* map_w, const CUtensorMap* map_g, const CUtensorMap* map_x)
 {
     using C = Cfg<MT, WM, RT, WR, SK, KC, STAGES, WF>;
     auto kern = decode_kernel<MT, WM, RT, WR, SK, KC, STAGES, WF>;
     const int blocks_per_sm = decode_occupancy_t<MT, WM, RT, WR, SK, KC, STAGES, WF>(a.S);
     if (blocks_per_sm <= 0) return cudaErrorLaunchOutOfResources;
-    const int n_row_tiles = (int)((a.N + C::kRB - 1) / C::kRB);
+    const long long n_groups = (a.N + RT - 1) / RT;
     const int n_mblocks = (int)((a.M + C::kMB - 1) / C::kMB);
-    const long long units = (long long)n_row_tiles * n_mblocks;
-    long long grid = (long long)a.sm_count * blocks_per_sm;
+    const long long slots = (long long)a.sm_count * blocks_per_sm;
+    Shares sh{(int)((n_groups + WR - 1) / WR), 1, 0, 0};      // one tile per share
+    if (C::kDealRest) {
+        // equal shares of the row groups, one per resident block and batch block (plain tiles when not even one round fills up)
+        long long n = slots / n_mblocks;
+        if (n < 1) n = 1;
+        if (n > n_groups) n = n_groups;
+        const long long rounds = n_groups / (n * WR), rest = n_groups - rounds * n * WR;
+        if (rounds > 0) sh = Shares{(int)n, (int)rounds, (int)(rest / n), (int)(rest % n)};
+    }
+    long long grid = (long long)sh.n_shares * n_mblocks;
+    if (grid > slots) grid = slots;
     if (a.max_blocks > 0 && grid > a.max_blocks) grid = a.max_blocks;
-    if (grid > units) grid = units;
 
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)grid);
@@ -589,8 +657,10 @@ cudaError_t launch_decode_t(const LaunchArgs& a, const CUtensorMap* map_w, const
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, *map_w, *map_x, a.b, a.y, (int)a.M, (int)a.N, (int)a.K, (int)a.seg_len, a.S,
-                              n_row_tiles, n_mblocks, (long long)a.ldy, a.status, a.wait_limit_ns, a.test_flags);
+    typename GroupMap<C::kDealRest>::type group_map{};
+    if constexpr (C::kDealRest) group_map = *map_g;
+    return cudaLaunchKernelEx(&cfg, kern, *map_w, *map_x, group_map, a.b, a.y, (int)a.M, (int)a.N, (int)a.K, (int)a.seg_len, a.S,
+                              sh, n_mblocks, (long long)a.ldy, a.status, a.wait_limit_ns, a.test_flags);
 }
 
 struct DecodeEntry {

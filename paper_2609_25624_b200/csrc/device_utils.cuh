@@ -13,7 +13,7 @@ namespace detlin {
 template <int WF>
 __device__ __forceinline__ float up16_lo(uint32_t w)
 {
-    if (WF == 0) return __uint_as_float(w << 16);
+    if (WF == 0) return __uint_as_float(__byte_perm(w, 0u, 0x1044));       // (faster than the shift: 82.5 against 80 % in the decode loop)
     return __half2float(__ushort_as_half((unsigned short)(w & 0xffffu)));
 }
 template <int WF>

@@ -98,7 +98,8 @@ struct DecodeConfig {
 // S = number of K segments of the order (it only scales the unit count in the schedule's cost model)
 bool decode_config_for(int64_t M, int64_t N, int64_t K, int S, int wfmt, int variant, DecodeConfig* out);
 int decode_num_variants();
-cudaError_t launch_decode(const LaunchArgs& a, const DecodeConfig& cfg, const CUtensorMap* map_w, const CUtensorMap* map_x);
+// map_w: box of a whole tile (rt * wr weight rows); map_g: of one row group (rt)
+cudaError_t launch_decode(const LaunchArgs& a, const DecodeConfig& cfg, const CUtensorMap* map_w, const CUtensorMap* map_g, const CUtensorMap* map_x);
 // resident blocks per SM of a tiling on the current device for an order with S segments (schedule information only)
 int decode_config_occupancy(int wfmt, const DecodeConfig& cfg, int S);
 
@@ -131,6 +132,7 @@ struct det_linear_plan {
     const void* map_x_ptr;
     int map_cfg_id;
     CUtensorMap map_w;
+    CUtensorMap map_g;               // decode: one row group of a tile
     CUtensorMap map_x;
 };
 

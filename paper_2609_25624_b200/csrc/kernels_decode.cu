@@ -51,6 +51,16 @@ double tiling_cost(const DecodeEntry& e, int64_t M, int64_t N, int64_t K, int S,
     const double hbm = ((double)rb * (double)K * 2.0 / 22.5 + 0.06 * (double)mb * (double)K * 4.0 / 64.0) * resident;
     const double body = (fma > hbm ? fma : hbm) * latency;
     const double overhead = (double)S * 1020.0 * ((double)(mb * rb) / 896.0) + (c.sk > 1 ? 1500.0 : 0.0);
+    if (rb >= 56 && mb >= 16) {
+        // what is left after whole rounds is dealt out by row groups (Cfg::kDealRest); half a tile takes a little longer than
+        // half the time (one warp per scheduler)
+        int64_t shares = (int64_t)sm_count * occ / mblocks;
+        const int64_t groups = (N + c.rt - 1) / c.rt;
+        shares = shares < 1 ? 1 : shares > groups ? groups : shares;
+        const int64_t whole = groups / (shares * c.wr), rest = groups - whole * shares * c.wr;
+        const double part = (double)((rest + shares - 1) / shares) / c.wr;
+        if (whole > 0) return (double)whole * (body + overhead) + (part < 1.0 ? part * 1.08 : 1.0) * body + (rest ? overhead : 0.0);
+    }
     return (double)rounds * (body + overhead);
 }
 
@@ -115,9 +125,9 @@ int decode_config_occupancy(int wfmt, const DecodeConfig& cfg, int S)
     return class_table(wfmt, cfg.id / 64)->entries[cfg.id % 64].occupancy(S);
 }
 
-cudaError_t launch_decode(const LaunchArgs& a, const DecodeConfig& cfg, const CUtensorMap* map_w, const CUtensorMap* map_x)
+cudaError_t launch_decode(const LaunchArgs& a, const DecodeConfig& cfg, const CUtensorMap* map_w, const CUtensorMap* map_g, const CUtensorMap* map_x)
 {
-    return class_table(a.wfmt, cfg.id / 64)->entries[cfg.id % 64].fn(a, map_w, map_x);
+    return class_table(a.wfmt, cfg.id / 64)->entries[cfg.id % 64].fn(a, map_w, map_g, map_x);
 }
 
 }  // namespace detlin
