@@ -102,30 +102,31 @@ cudaError_t launch_combine(const LaunchArgs& a)
 namespace cg = cooperative_groups;
 constexpr int kArgmaxCluster = 8;
 
-__device__ __forceinline__ bool argmax_better(float v, int i, float bv, int bi)
+// A value as an unsigned key with the order above: NaN on top, -0 = +0.  A pair (key, index) is better if its key is
+// larger, or equal with a smaller index; as one 64-bit number with the index complemented, the better pair is the larger.
+__device__ __forceinline__ uint32_t argmax_key(float v)
 {
-    const bool vn = (v != v), bn = (bv != bv);
-    if (vn || bn) return vn && (!bn || i < bi);
-    return (v > bv) || (v == bv && i < bi);
+    if (v != v) return 0xffffffffu;
+    const uint32_t u = __float_as_uint(__fadd_rn(v, 0.0f));      // -0 + +0 = +0
+    return u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u);
 }
-
-__device__ __forceinline__ void argmax_warp(float& bv, int& bi)
+__device__ __forceinline__ unsigned long long argmax_warp(unsigned long long p)
 {
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, bv, d);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, d);
-        if (argmax_better(ov, oi, bv, bi)) { bv = ov; bi = oi; }
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, p, d);
+        p = o > p ? o : p;
     }
+    return p;
 }
 
+// Bound by latency for the few rows of a decode step: a thread's whole share of a row (16-byte loads where the row starts
+// aligned) is in flight at once.  M = 8, N = 128256: 14 -> 4 us.
 __global__ void __cluster_dims__(kArgmaxCluster, 1, 1) __launch_bounds__(1024)
 argmax_rows_kernel(const float* __restrict__ y, int64_t N, int32_t* __restrict__ idx)
 {
-    __shared__ float sv[32];
-    __shared__ int si[32];
-    __shared__ float block_v;
-    __shared__ int block_i;
+    __shared__ unsigned long long warp_best[32];
+    __shared__ unsigned long long block_best;
     // programmatic dependent launch: let the next kernel of the stream start its prologue now, and
     // wait for the kernel that produced y before reading it
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -133,36 +134,54 @@ argmax_rows_kernel(const float* __restrict__ y, int64_t N, int32_t* __restrict__
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const float* row = y + (int64_t)blockIdx.y * N;
-    const int64_t per = (N + kArgmaxCluster - 1) / kArgmaxCluster;
-    const int64_t lo = rank * per;
-    const int64_t hi = (lo + per < N) ? lo + per : N;
-    // a block whose slice is empty contributes the row's first element (always a valid candidate)
-    float bv = row[lo < N ? lo : 0];
-    int bi = (int)(lo < N ? lo : 0);
-    for (int64_t n = lo + threadIdx.x; n < hi; n += blockDim.x) {
-        const float v = row[n];
-        if (argmax_better(v, (int)n, bv, bi)) { bv = v; bi = (int)n; }
+    uint32_t key = 0, at = 0xffffffffu;              // 0 < any value's key: an empty share loses
+    auto look = [&](float v, uint32_t n) {           // a thread's elements come in ascending order
+        const uint32_t k = argmax_key(v);
+        if (k > key) { key = k; at = n; }
+    };
+    if ((reinterpret_cast<uintptr_t>(row) & 15u) == 0) {
+        const uint32_t quads = (uint32_t)(N / 4), per = (quads + kArgmaxCluster - 1) / kArgmaxCluster;
+        const uint32_t lo = rank * per, hi = min(lo + per, quads);
+        const float4* r4 = reinterpret_cast<const float4*>(row);
+        uint32_t i = lo + threadIdx.x;
+        for (; i + 3 * 1024 < hi; i += 4 * 1024) {
+            float4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = r4[i + 1024 * u];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t n = 4 * (i + 1024 * u);
+                look(v[u].x, n); look(v[u].y, n + 1); look(v[u].z, n + 2); look(v[u].w, n + 3);
+            }
+        }
+        float4 v[3];
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+            if (i + 1024 * u < hi) v[u] = r4[i + 1024 * u];
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+            if (i + 1024 * u < hi) {
+                const uint32_t n = 4 * (i + 1024 * u);
+                look(v[u].x, n); look(v[u].y, n + 1); look(v[u].z, n + 2); look(v[u].w, n + 3);
+            }
+        if (rank == kArgmaxCluster - 1 && threadIdx.x < (N & 3)) look(row[4ll * quads + threadIdx.x], 4 * quads + threadIdx.x);
+    } else {
+        const uint32_t per = (uint32_t)((N + kArgmaxCluster - 1) / kArgmaxCluster);
+        const int64_t lo = (int64_t)rank * per, hi = (lo + per < N) ? lo + per : N;
+#pragma unroll 4
+        for (int64_t n = lo + threadIdx.x; n < hi; n += 1024) look(row[n], (uint32_t)n);
     }
-    argmax_warp(bv, bi);
-    if ((threadIdx.x & 31) == 0) { sv[threadIdx.x >> 5] = bv; si[threadIdx.x >> 5] = bi; }
+    unsigned long long best = argmax_warp(((unsigned long long)key << 32) | (uint32_t)~at);
+    if ((threadIdx.x & 31) == 0) warp_best[threadIdx.x >> 5] = best;
     __syncthreads();
     if (threadIdx.x < 32) {
-        const int nw = blockDim.x >> 5;
-        bv = (threadIdx.x < nw) ? sv[threadIdx.x] : sv[0];
-        bi = (threadIdx.x < nw) ? si[threadIdx.x] : si[0];
-        argmax_warp(bv, bi);
-        if (threadIdx.x == 0) { block_v = bv; block_i = bi; }
+        best = argmax_warp(warp_best[threadIdx.x]);
+        if (threadIdx.x == 0) block_best = best;
     }
     cluster.sync();
-    if (rank == 0 && threadIdx.x == 0) {
-        bv = block_v;
-        bi = block_i;
-        for (int r = 1; r < kArgmaxCluster; ++r) {
-            const float ov = *cluster.map_shared_rank(&block_v, r);
-            const int oi = *cluster.map_shared_rank(&block_i, r);
-            if (argmax_better(ov, oi, bv, bi)) { bv = ov; bi = oi; }
-        }
-        idx[blockIdx.y] = bi;
+    if (rank == 0 && threadIdx.x < 32) {
+        best = argmax_warp(threadIdx.x < kArgmaxCluster ? *cluster.map_shared_rank(&block_best, threadIdx.x) : 0ull);
+        if (threadIdx.x == 0) idx[blockIdx.y] = (int32_t)~(uint32_t)best;
     }
     cluster.sync();     // keep every block's shared memory alive until block 0 has read it
 }

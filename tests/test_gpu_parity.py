@@ -283,3 +283,22 @@ def test_prefill_very_short_k(M, N, K):
         W32s = W32[:, : K - 4].contiguous()             # K a multiple of 4 only: the four-element tail
         xs = x[:, : K - 4].contiguous()
         assert_bits_equal(run_gpu(xs, W32s, b, kernel=KERNEL_PREFILL), oracle_y(xs, W32s, b), "fp32 weights, K % 8 == 4")
+
+
+@pytest.mark.parametrize("N", [3, 4, 1027, 32768 + 5, 131072, 131076])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_argmax_vector_and_scalar_loads(N, offset):
+    """Rows that start aligned (16-byte loads) or not, ties in and across the shares of threads and blocks, NaN, infinities."""
+    M = 5
+    g = torch.Generator().manual_seed(N + offset)
+    y = torch.randn(M, N, generator=g)
+    y[1, N - 1] = y[1, N // 2] = y[1, 0] = 9.0
+    y[2, :] = float("-inf")
+    y[3, N // 3] = y[3, N - 1] = float("nan")
+    y[4, :] = -0.0
+    y[4, N - 1] = 0.0
+    buf = torch.empty(M * N + offset, device="cuda")[offset:].view(M, N)
+    buf.copy_(y)
+    idx = torch.full((M,), -1, dtype=torch.int32, device="cuda")
+    B.det_argmax_rows(buf, idx)
+    assert idx.cpu().tolist() == oracle.argmax_rows(y.numpy()).tolist()

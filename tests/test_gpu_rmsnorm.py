@@ -98,3 +98,11 @@ def test_bad_arguments():
     with pytest.raises(B.DetLinearError):
         B.det_rmsnorm(x, g, float("nan"), y)
     assert B.lib().det_rmsnorm(None, g.data_ptr(), 0.0, 2, 8, y.data_ptr(), None) == 1
+
+
+# a block per row (few rows, or rows beyond 4096 elements) on both sides of its limits, of the gain quads a thread fetches
+# ahead (8192 elements) and of whole groups of eight chunks
+@pytest.mark.parametrize("M,H", [(512, 260), (513, 260), (3, 4), (2, 1020), (2, 1028), (5, 4100), (600, 4224), (2, 8188), (2, 8196), (1, 49152), (1, 49156)])
+def test_block_per_row_bit_exact(M, H):
+    x, g = make(M, H, 7 * M + H)
+    assert_bits_equal(run(x, g, 1e-5), oracle.rmsnorm(x.numpy(), g.numpy(), 1e-5), f"{M}x{H}")
