@@ -407,7 +407,8 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                 // One 128-element chunk: the lane's four elements of every row / batch row of the warp tile.
                 // Row pairs are processed in passes of at most four pairs so that only a few widened
                 // weights are live at a time (the accumulators already take most of the registers).
-                auto chunk = [&](int cc) {
+                // `look`: ask whether the stage after this one has landed, once the loads are out (they would wait for the answer)
+                auto chunk = [&](int cc, bool look) {
                     // chunk cc lies in box cc / (kKB / 128) of the stage, at element (cc * 128) % kKB of its rows
                     const uint32_t box = (uint32_t)((cc * 128) / C::kKB) * C::kSubBytes;
                     const uint32_t kin = (uint32_t)((cc * 128) % C::kKB);
@@ -428,6 +429,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                         for (int q = 0; q < 2 * kMaxPass; ++q)
                             if (q < 2 * np)
                                 w[q] = wload<WF>(((q & 1) ? ws_odd : ws_even) + (2 * p0 + q) * C::kWPitch);
+                        if (look && p0 == 0) ready = mbar_test_wait(fullg + 8 * st, phase);
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {          // the lane's four elements, ascending
                             float2 wp[kMaxPass];
@@ -452,9 +454,8 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     // whole stage inside the segment: no per-lane test
                     {
 #pragma unroll(MT * RT >= 64 ? 1 : 2)
-                        for (int cc = 0; cc < KC / 128 - 1; ++cc) chunk(cc);
-                        ready = mbar_test_wait(fullg + 8 * st, phase);          // look ahead: the stage after this one
-                        chunk(KC / 128 - 1);
+                        for (int cc = 0; cc < KC / 128 - 1; ++cc) chunk(cc, false);
+                        chunk(KC / 128 - 1, true);
                     }
                 } else {
                     ready = false;
@@ -462,7 +463,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     // (K % 4 == 0 here, so a lane's four elements are all inside or all outside).
 #pragma unroll 1
                     for (int cc = 0; cc < KC / 128; ++cc)
-                        if (k0 + cc * 128 + 4 * lane < k_hi) chunk(cc);
+                        if (k0 + cc * 128 + 4 * lane < k_hi) chunk(cc, false);
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(emptyg + 8 * st_cur);
