@@ -132,3 +132,16 @@ def test_attention_argument_checks():
         B.det_attention_decode(q.cuda(), k.cuda(), v.cuda(), 1.0, o)
     assert ei.value.status == 2 and "shared memory" in B.det_last_error()
     assert B.lib().det_attention_decode(None, None, None, 1.0, 1, 1, 1, 1, 4, None, None) == 1
+
+
+# the ring of asynchronous copies: five and three slots and none, P.V slices of 1, 2 and 4 consecutive d, one and two chunks of
+# the head dimension (lanes idle in the last), a last block with a partial segment, a partial group, no keys at all
+@pytest.mark.parametrize("B_,Hq,Hkv,T,D", [(20, 8, 8, 130, 128), (24, 16, 8, 255, 64), (10, 64, 8, 300, 132), (5, 32, 16, 1025, 256), (20, 8, 8, 2049, 36),
+                                           (40, 4, 4, 2300, 128), (40, 16, 4, 4099, 128), (80, 16, 2, 1290, 128), (19, 8, 4, 2050, 4), (3, 8, 8, 5121, 128)])
+def test_attention_streaming_schedules(B_, Hq, Hkv, T, D):
+    q, k, v = make_qkv(B_, Hq, Hkv, T, D, seed=T + B_)
+    scale = float(np.float32(1.0 / math.sqrt(D)))
+    want = oracle.attention_decode(q.numpy(), k.numpy(), v.numpy(), scale)
+    got = run_gpu_attention(q, k, v, scale)
+    assert not np.isnan(got).any()
+    assert_bits_equal(got, want, f"attention {B_},{Hq},{Hkv},{T},{D}")
