@@ -94,6 +94,30 @@ cudaError_t launch_combine(const LaunchArgs& a)
     return cudaLaunchKernelEx(&cfg, combine_kernel, (const float*)a.partials, a.b, a.y, MN, a.N, a.S, a.ldy);
 }
 
+// Small activations from (mapped) pinned host memory to device memory: 16-byte loads across the bus, all of them on their way at
+// once, and the kernel after this one may start its prologue and its weight stream meanwhile.
+__global__ void __launch_bounds__(256) copy_from_host_kernel(const float4* __restrict__ src, float4* __restrict__ dst, unsigned n)
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) dst[i] = __ldcv(src + i);
+}
+
+cudaError_t launch_copy_from_host(const void* src, void* dst, size_t bytes, cudaStream_t stream)
+{
+    const unsigned n = (unsigned)(bytes / 16), blocks = (n + 255) / 256;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3(blocks < 256 ? blocks : 256);
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, copy_from_host_kernel, static_cast<const float4*>(src), static_cast<float4*>(dst), n);
+}
+
 // Row argmax, lowest index on ties (the paper's stated tie rule for greedy decoding).  Ordering
 // key: NaN beats everything (first NaN wins), otherwise larger value, then smaller index.
 // Comparisons only, so the result is exact and order-free.  A cluster of kArgmaxCluster blocks

@@ -302,3 +302,31 @@ def test_argmax_vector_and_scalar_loads(N, offset):
     idx = torch.full((M,), -1, dtype=torch.int32, device="cuda")
     B.det_argmax_rows(buf, idx)
     assert idx.cpu().tolist() == oracle.argmax_rows(y.numpy()).tolist()
+
+
+# activations and results that cross the bus by a kernel (pinned, aligned, up to a MiB) or by the copy engines
+@pytest.mark.parametrize("M,N,K", [(3, 40, 520), (8, 4097, 1000), (64, 5000, 264), (5, 64, 60000), (64, 80, 4608), (130, 72, 136), (2, 9, 7)])
+@pytest.mark.parametrize("where", ["pinned", "pinned, off by 4 bytes", "pageable"])
+def test_run_host_by_kernel_and_by_copy(M, N, K, where):
+    x, W, b = inputs.make_case(M, N, K)
+    want = oracle_y(x, W, b)
+    off = 1 if "off" in where else 0
+
+    def host(rows, cols):
+        t = torch.empty(rows * cols + off)
+        return (t if where == "pageable" else t.pin_memory())[off:].view(rows, cols)
+
+    xh, yh = host(M, K), host(M, N)
+    plan = B.det_linear_plan(M, N, K)
+    Wd, bd = W.cuda(), b.cuda()
+    for rep in range(2):
+        xh.copy_(x if rep else -x)
+        yh.fill_(float("nan"))
+        B.det_linear_run_host(plan, xh, Wd, bd, yh)
+    assert_bits_equal(yh.numpy(), want, where)
+    if where != "pageable":
+        yh.fill_(float("nan"))
+        B.det_linear_run_host_async(plan, xh, Wd, bd, yh)
+        torch.cuda.current_stream().synchronize()
+        assert_bits_equal(yh.numpy(), want, where + ", asynchronous")
+    plan.close()
