@@ -18,7 +18,8 @@ OBJ_DIR = os.path.join(HERE, "csrc", "obj")
 SOURCES = [("plan.cpp", ()), ("capi.cu", ()), ("kernels_generic.cu", ()), ("kernels_decode.cu", ()),
            ("kernels_prefill.cu", ()), ("prefill_tma.cu", ()), ("bench_kernels.cu", ()), ("noalloc.cu", ()), ("ablation.cu", ()), ("rmsnorm.cu", ()), ("attention.cu", ())]
 SOURCES += [(f"decode_inst_{i}.cu", (f"-DDET_WF={wf}",)) for wf in (0, 1, 2) for i in range(4)]
-SOURCES += [(src, (f"-DDET_WF={wf}",)) for wf in (0, 1, 2) for src in ("prefill_tma_inst.cu", "decode_any.cu")]
+SOURCES += [("decode_any.cu", (f"-DDET_WF={wf}",)) for wf in (0, 1, 2)]
+SOURCES += [("prefill_tma_inst.cu", (f"-DDET_WF={wf}", f"-DDET_PLAIN={plain}")) for wf in (0, 1, 2) for plain in (0, 1)]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

@@ -255,9 +255,9 @@ det_linear_plan_t* det_linear_plan_shard(int64_t M, int64_t N, int64_t K, int64_
         det_linear_plan_destroy(plan);              // frees whatever was allocated before the failure
         return nullptr;
     }
-    // Schedule workspace of the TMA-fed prefill kernel: a ticket, hand-over flags and, where blocks take equal stretches, the
+    // Schedule workspace of the prefill kernel: a ticket, hand-over flags and, where blocks take equal stretches, the
     // accumulators handed over.  Without it the plan still works: it uses the register-staged kernel, which computes the same bits.
-    if (prm.kernel == kKernelPrefill) {
+    if (prm.bucket == 1) {
         const uint64_t handoff_at = (4 * pw.sync_words + 255) / 256 * 256;
         e = device_alloc(reinterpret_cast<void**>(&plan->sync), handoff_at + 4 * pw.handoff_floats);
         if (e == cudaSuccess) e = cudaMemset(plan->sync, 0, 4 * pw.sync_words);

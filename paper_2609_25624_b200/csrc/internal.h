@@ -66,6 +66,9 @@ cudaError_t launch_prefill(const LaunchArgs& a);
 // Prefill kernel with both tiles fed by TMA (prefill_tma_kernel.cuh); block tile 16 tm rows x width columns.  Tensor maps,
 // swizzled over the width of the box: map_x: x [M][K], box [16 tm][32]; map_w: W [N][K] in its format, box [width][32].
 cudaError_t launch_prefill_tma(const LaunchArgs& a, int tm, int width, const CUtensorMap* map_w, const CUtensorMap* map_x);
+// The same kernel fed by plain loads: any K, any alignment (x and W themselves, no tensor maps).  Without the hand-over
+// workspace every unit of work gets a block of its own.
+cudaError_t launch_prefill_plain(const LaunchArgs& a);
 int prefill_tile_width(int64_t M, int64_t N, int64_t K, int S, int64_t seg_len, int tm, int sm_count);
 // Device memory the TMA-fed kernel wants: split-K partials by tile with their counters; ticket, flags and accumulators of
 // the hand-over between blocks (no accumulators when every unit of work gets a block of its own).

@@ -1,6 +1,5 @@
-// Generic kernels: any shape, any alignment, scalar bounds-checked loads.  They execute exactly the
-// frozen order and serve ragged shapes (K % 8 != 0, misaligned buffers: what the
-// paper's ragged 100 x 1000 x 1000 probe exercises), the split-K second pass and the row argmax.  They are not tuned.
+// The dispatch for shapes and buffers that TMA cannot read (K % 8 != 0 or FP32 weights with K % 4 != 0, misaligned buffers),
+// the split-K second pass, the copy of small activations from the host and the row argmax.
 #include "internal.h"
 #include "device_utils.cuh"
 #include <cooperative_groups.h>
@@ -10,26 +9,6 @@ namespace detlin {
 cudaError_t launch_decode_any_wf0(const LaunchArgs& a);        // decode_any.cu
 cudaError_t launch_decode_any_wf1(const LaunchArgs& a);
 cudaError_t launch_decode_any_wf2(const LaunchArgs& a);
-
-// Prefill order (V=1, L=1, P=1): one thread per (m, n, segment), one chain, strictly ascending k.
-template <int WF>
-__global__ void __launch_bounds__(256)
-generic_prefill_kernel(const float* __restrict__ x, const typename WeightElem<WF>::type* __restrict__ W, const float* __restrict__ b,
-                       float* __restrict__ out, int64_t M, int64_t N, int64_t K, int64_t seg_len, int S, int direct, int64_t ldy)
-{
-    const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t m = blockIdx.y;
-    const int s = blockIdx.z;
-    if (n >= N) return;
-    const int64_t k_lo = (int64_t)s * seg_len;
-    const int64_t k_hi = (k_lo + seg_len < K) ? k_lo + seg_len : K;
-    const float* xrow = x + m * K;
-    const typename WeightElem<WF>::type* wrow = W + n * K;
-    float t = 0.0f;
-    for (int64_t k = k_lo; k < k_hi; ++k) t = __fmaf_rn(xrow[k], up_elem<WF>(wrow[k]), t);
-    if (direct) out[m * ldy + n] = b ? __fadd_rn(t, b[n]) : t;
-    else        out[((int64_t)s * M + m) * N + n] = t;
-}
 
 // Split-K second pass (rule R3): the S partials of every output are added in ascending segment
 // order by one thread, then the bias; no atomics anywhere.
@@ -49,34 +28,11 @@ combine_kernel(const float* __restrict__ partials, const float* __restrict__ b, 
     y[m * ldy + n] = b ? __fadd_rn(t, b[n]) : t;
 }
 
-template <int WF>
-static cudaError_t launch_generic_prefill_t(const LaunchArgs& a)
-{
-    typedef typename WeightElem<WF>::type WT;
-    const WT* W = static_cast<const WT*>(a.W);
-    const int direct = (a.S == 1);
-    float* out = direct ? a.y : a.partials;
-    {
-        // grid.y carries M (< 65536 per launch); larger M is cut into slabs of rows
-        const int64_t max_y = 32768;
-        for (int64_t m0 = 0; m0 < a.M; m0 += max_y) {
-            const int64_t mm = (a.M - m0 < max_y) ? a.M - m0 : max_y;
-            dim3 grid((unsigned)((a.N + 255) / 256), (unsigned)mm, (unsigned)a.S);
-            float* o = out + m0 * (direct ? a.ldy : a.N);   // both layouts ([M][ldy] and [s][M][N]) advance by whole rows
-            generic_prefill_kernel<WF><<<grid, 256, 0, a.stream>>>(a.x + m0 * a.K, W, a.b, o, a.M, a.N, a.K, a.seg_len, a.S, direct, a.ldy);
-        }
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (!direct) return launch_combine(a);
-    return cudaSuccess;
-}
-
+// Any shape, any alignment: the same orders, the same bits.
 cudaError_t launch_generic(const LaunchArgs& a, int bucket)
 {
-    if (a.wfmt == 1) return bucket == 0 ? launch_decode_any_wf1(a) : launch_generic_prefill_t<1>(a);
-    if (a.wfmt == 2) return bucket == 0 ? launch_decode_any_wf2(a) : launch_generic_prefill_t<2>(a);
-    return bucket == 0 ? launch_decode_any_wf0(a) : launch_generic_prefill_t<0>(a);
+    if (bucket != 0) return launch_prefill_plain(a);
+    return a.wfmt == 1 ? launch_decode_any_wf1(a) : a.wfmt == 2 ? launch_decode_any_wf2(a) : launch_decode_any_wf0(a);
 }
 
 cudaError_t launch_combine(const LaunchArgs& a)

@@ -3,9 +3,12 @@
 
 namespace detlin {
 
-cudaError_t launch_prefill_tma_wf0(const LaunchArgs& a, int tm, int width, const CUtensorMap* map_w, const CUtensorMap* map_x);
-cudaError_t launch_prefill_tma_wf1(const LaunchArgs& a, int tm, int width, const CUtensorMap* map_w, const CUtensorMap* map_x);
-cudaError_t launch_prefill_tma_wf2(const LaunchArgs& a, int tm, int width, const CUtensorMap* map_w, const CUtensorMap* map_x);
+#define DET_DECLARE(wf) \
+    cudaError_t launch_prefill_wf##wf##_0(const LaunchArgs& a, int tm, int width, const CUtensorMap* map_w, const CUtensorMap* map_x); \
+    cudaError_t launch_prefill_wf##wf##_1(const LaunchArgs& a, int tm, int width, const CUtensorMap* map_w, const CUtensorMap* map_x);
+DET_DECLARE(0)
+DET_DECLARE(1)
+DET_DECLARE(2)
 
 // Tile width (schedule only: every width gives the same bits).  Wide tiles multiply fastest, narrow ones make more units:
 // with more units than SMs the work is dealt out in equal stretches and the width's rate decides, with fewer the call
@@ -53,9 +56,35 @@ cudaError_t launch_prefill_tma(const LaunchArgs& a, int tm, int width, const CUt
 {
     if (!a.status || !a.sync) return cudaErrorInvalidValue;
     switch (a.wfmt) {
-    case DET_WEIGHT_BF16: return launch_prefill_tma_wf0(a, tm, width, map_w, map_x);
-    case DET_WEIGHT_FP16: return launch_prefill_tma_wf1(a, tm, width, map_w, map_x);
-    case DET_WEIGHT_FP32: return launch_prefill_tma_wf2(a, tm, width, map_w, map_x);
+    case DET_WEIGHT_BF16: return launch_prefill_wf0_0(a, tm, width, map_w, map_x);
+    case DET_WEIGHT_FP16: return launch_prefill_wf1_0(a, tm, width, map_w, map_x);
+    case DET_WEIGHT_FP32: return launch_prefill_wf2_0(a, tm, width, map_w, map_x);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_prefill_plain(const LaunchArgs& a)
+{
+    if (!a.status) return cudaErrorInvalidValue;
+    const int64_t most = (int64_t)1 << 30;           // rows are counted in 32 bits; no memory holds that many of several segments
+    if (a.M > most) {
+        if (a.S > 1) return cudaErrorInvalidValue;
+        for (int64_t m = 0; m < a.M; m += most) {
+            LaunchArgs part = a;
+            part.x += m * a.K;
+            part.y += m * a.ldy;
+            part.M = a.M - m < most ? a.M - m : most;
+            const cudaError_t e = launch_prefill_plain(part);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    }
+    const int tm = prefill_rows_per_thread(a.M);
+    const int width = prefill_tile_width(a.M, a.N, a.K, a.S, a.seg_len, tm, a.sm_count);
+    switch (a.wfmt) {
+    case DET_WEIGHT_BF16: return launch_prefill_wf0_1(a, tm, width, nullptr, nullptr);
+    case DET_WEIGHT_FP16: return launch_prefill_wf1_1(a, tm, width, nullptr, nullptr);
+    case DET_WEIGHT_FP32: return launch_prefill_wf2_1(a, tm, width, nullptr, nullptr);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -1,5 +1,6 @@
-// Launchers of the TMA-fed prefill kernel for one weight format (compiled once per format, DET_WF = 0 BF16, 1 FP16, 2 FP32)
-// and every tile: heights 80, 96, 112 and 128, widths 256, 128, 64 and 32.
+// Launchers of the prefill kernel for one weight format (DET_WF = 0 BF16, 1 FP16, 2 FP32), fed by TMA or (DET_PLAIN = 1) by plain
+// loads for any K and alignment, and every tile: heights 80, 96, 112 and 128, widths 256, 128, 64 and 32.  Compiled once
+// per format and feed.
 #include "prefill_tma_kernel.cuh"
 
 namespace detlin {
@@ -8,16 +9,16 @@ namespace {
 
 using namespace prefill_detail;
 
-template <int WF, int TR, int TC, int LX, int LY>
+template <int WF, int TR, int TC, int LX, int LY, bool PLAIN>
 cudaError_t launch_t(const LaunchArgs& la, const CUtensorMap* map_w, const CUtensorMap* map_x)
 {
-    typedef Tile<WF, TR, TC, LX, LY> T;
+    typedef Tile<WF, TR, TC, LX, LY, PLAIN> T;
     static bool configured[kMaxDevices];             // function attributes belong to a device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    auto kern = prefill_tma_kernel<WF, TR, TC, LX, LY>;
+    auto kern = prefill_tma_kernel<WF, TR, TC, LX, LY, PLAIN>;
     if (!configured[dev]) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::kSmemBytes);
         if (e != cudaSuccess) return e;
@@ -27,6 +28,7 @@ cudaError_t launch_t(const LaunchArgs& la, const CUtensorMap* map_w, const CUten
     const long long units = tiles_m * tiles_n * la.S;
     if (units > 0x7fffffffLL) return cudaErrorInvalidValue;
     Args a{};
+    a.x = la.x; a.w = la.W;
     a.bias = la.b; a.y = la.y; a.partials = la.partials; a.handoff = la.handoff; a.sync = la.sync;
     a.tile_counters = la.tile_counters; a.status = la.status;
     a.ldy = la.ldy;
@@ -55,7 +57,8 @@ cudaError_t launch_t(const LaunchArgs& la, const CUtensorMap* map_w, const CUten
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, kern, *map_x, *map_w, a);
+    const CUtensorMap none{};
+    e = cudaLaunchKernelEx(&cfg, kern, PLAIN ? none : *map_x, PLAIN ? none : *map_w, a);
     if (e != cudaSuccess) return e;
     if (la.S > 1 && !la.tile_counters) return launch_combine(la);
     return cudaSuccess;
@@ -66,19 +69,19 @@ template <int WF, int TM>
 cudaError_t launch_h(const LaunchArgs& a, int width, const CUtensorMap* map_w, const CUtensorMap* map_x)
 {
     switch (width) {
-    case 256: return launch_t<WF, 2 * TM, 8, 32, 8>(a, map_w, map_x);
-    case 128: return launch_t<WF, 8, 8, 16, 2 * TM>(a, map_w, map_x);
-    case 64: return launch_t<WF, 4, 8, 8, 4 * TM>(a, map_w, map_x);
-    case 32: return launch_t<WF, 4, 4, 8, 4 * TM>(a, map_w, map_x);
+    case 256: return launch_t<WF, 2 * TM, 8, 32, 8, DET_PLAIN>(a, map_w, map_x);
+    case 128: return launch_t<WF, 8, 8, 16, 2 * TM, DET_PLAIN>(a, map_w, map_x);
+    case 64: return launch_t<WF, 4, 8, 8, 4 * TM, DET_PLAIN>(a, map_w, map_x);
+    case 32: return launch_t<WF, 4, 4, 8, 4 * TM, DET_PLAIN>(a, map_w, map_x);
     default: return cudaErrorInvalidValue;
     }
 }
 
 }  // namespace
 
-#define DET_CAT2(a, b) a##b
-#define DET_PREFILL_NAME(wf) DET_CAT2(launch_prefill_tma_wf, wf)
-cudaError_t DET_PREFILL_NAME(DET_WF)(const LaunchArgs& a, int tm, int width, const CUtensorMap* map_w, const CUtensorMap* map_x)
+#define DET_CAT3(a, b, c) a##b##_##c
+#define DET_PREFILL_NAME(wf, plain) DET_CAT3(launch_prefill_wf, wf, plain)
+cudaError_t DET_PREFILL_NAME(DET_WF, DET_PLAIN)(const LaunchArgs& a, int tm, int width, const CUtensorMap* map_w, const CUtensorMap* map_x)
 {
     switch (tm) {
     case 5: return launch_h<DET_WF, 5>(a, width, map_w, map_x);

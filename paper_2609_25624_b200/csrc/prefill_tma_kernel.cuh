@@ -36,6 +36,15 @@
 // TFLOP/s); M = 2048, N = 4096, K = 14336 3916 -> 3622 us (89.2 %); M = 72, N = 28672, K = 4096 391 -> 311 us; M = 128,
 // N = 4096, K = 14336 299 -> 254 us; 100 x 1000 x 1000 with FP32 weights 41 -> 13 us.
 //
+// Any K, any alignment (PLAIN): rows that start anywhere are out of TMA's reach, so the preparing warps load them themselves,
+// a slab ahead (a block of 4 rows x 4 k ahead for the 256 columns wide tile, whose register split leaves no more: 56 registers
+// spilled, so they get 88 here and the multiplying warps 208); a 16-bit row's weights are two or three aligned words, lined up
+// by byte permutations (element by element where such a word would reach outside of W).  Beyond K they store -0.0 for
+// activations and +0 for weights: the product is -0.0, and adding -0.0 changes no accumulator (not even a -0.0 one), so the
+// multiply loop may run on to a whole octet.  Everything else is the same kernel.  Against one thread per output before: M =
+// 300, N = 8192, K = 4097 13362 -> 379 us (71 % of 74.45 TFLOP/s; the scalar loads hold it up); 100 x 1001 x 1001 156 -> 18 us,
+// with FP32 weights 157 -> 17 us; 130 x 500 x 333 48 -> 13 us.
+//
 // Every wait is bounded: one that expires records the fact in the device status word and the block returns without
 // storing.
 #pragma once
@@ -56,7 +65,7 @@ constexpr int kMaxMulWarps = 8;
 constexpr int kPrepBarrier = 1;                      // named barrier of the preparing warps
 
 // Thread tile TR x TC on LX x LY multiplying threads (columns x rows).
-template <int WF, int TR, int TC, int LX, int LY> struct Tile {
+template <int WF, int TR, int TC, int LX, int LY, bool PLAIN = false> struct Tile {
     static constexpr int BM = TR * LY, BN = TC * LX;
     static constexpr int kMulThreads = LX * LY, kMulWarps = kMulThreads / 32, kThreads = kMulThreads + kPrepThreads;
     static constexpr int kXGroups = BM / 4, kWGroups = BN / 4;            // 16-byte groups of a k row
@@ -67,20 +76,22 @@ template <int WF, int TR, int TC, int LX, int LY> struct Tile {
     static constexpr int kRawBytes = kRawXBytes + kRawWBytes;
     static constexpr bool kWide = TR * TC > 64;
     // Raw stages cover the latency of memory: a slab of the wide tile takes 4 us, of the narrow ones down to 0.3 us.
-    static constexpr int kRawStages = kWide ? 2 : (BN > 64 ? 3 : 4);
+    static constexpr int kRawStages = PLAIN ? 0 : kWide ? 2 : (BN > 64 ? 3 : 4);
     static constexpr int kBudget = 227 * 1024 - 1024 - 256;
     static constexpr int kStages = 3 * (kXBytes + kWBytes) + kRawStages * kRawBytes <= kBudget ? 3 : 2;
     static constexpr int kSmemBytes = kStages * (kXBytes + kWBytes) + kRawStages * kRawBytes + 256 + 1024;   // + barriers, + alignment
     static_assert(kSmemBytes <= 227 * 1024, "shared memory");
     // A block of twelve warps is launched with 168 registers a thread; a 16 x 8 tile wants more, the preparing warps less:
-    // 256 x 224 + 128 x 56 = 384 x 168.
-    static constexpr int kMulRegs = 224, kPrepRegs = 56;
+    // 256 x 224 + 128 x 56 = 384 x 168 = 256 x 208 + 128 x 88.
+    static constexpr int kMulRegs = PLAIN ? 208 : 224, kPrepRegs = PLAIN ? 88 : 56;
     static_assert(!kWide || kMulThreads * kMulRegs + kPrepThreads * kPrepRegs <= kThreads * 168, "the block's own registers");
     static_assert(!kWide || kMulWarps % 4 == 0, "registers move between whole warpgroups");
     static_assert(kMulWarps <= kMaxMulWarps && kMulThreads % 32 == 0, "warps");
 };
 
 struct Args {
+    const float* x;              // PLAIN: the operands themselves
+    const void* w;
     const float* bias;
     float* y;
     float* partials;             // S > 1: segment sums, [tile][segment][piece][thread] in 8-byte pieces with counters, else [segment][M][N]
@@ -171,11 +182,11 @@ struct Cursor {
     int j, left, k, m0, n0;
 };
 
-template <int WF, int TR, int TC, int LX, int LY>
-__global__ void __launch_bounds__((Tile<WF, TR, TC, LX, LY>::kThreads), 1)
+template <int WF, int TR, int TC, int LX, int LY, bool PLAIN>
+__global__ void __launch_bounds__((Tile<WF, TR, TC, LX, LY, PLAIN>::kThreads), 1)
 prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, const __grid_constant__ Args a)
 {
-    typedef Tile<WF, TR, TC, LX, LY> T;
+    typedef Tile<WF, TR, TC, LX, LY, PLAIN> T;
     constexpr int BM = T::BM, BN = T::BN, ST = T::kStages, RS = T::kRawStages;
     constexpr int kMulThreads = T::kMulThreads, kMulWarps = T::kMulWarps;
     constexpr int XG = TR / 4, XR = TR % 4;          // a thread's rows: XG groups of four, then XR (0 or 2)
@@ -222,6 +233,152 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         // ---------------- preparing warps ----------------
         if constexpr (T::kWide) reg_dec<T::kPrepRegs>();
         const int t = threadIdx.x - kMulThreads;
+        if constexpr (PLAIN) {
+            typedef typename WeightElem<WF>::type WT;
+            constexpr int NHW = (NGW + 15) / 16, NHX = (NGX + 15) / 16, NB = NHW + NHX;      // blocks of a slab per thread
+            const int g0 = (t & 7) + 8 * (t >> 6), q = (t >> 3) & 7;
+            const WT* wg = static_cast<const WT*>(a.w);
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            struct Block { uint32_t v[4][4]; unsigned odd; };
+            int j = 0, k = 0, left = 0, m0 = 0, n0 = 0;
+            auto open = [&]() {
+                if (j >= n_pieces) return;
+                const Piece p = piece_of(a, w, j);
+                left = p.n_slabs;
+                k = p.k0;
+                m0 = (p.tile % a.tiles_m) * BM;
+                n0 = (p.tile / a.tiles_m) * BN;
+            };
+            open();
+            // block b of the slab at the cursor: weights first, then activations.  Rows beyond the matrices repeat the last one.
+            auto load = [&](Block& r, int b) {
+                const int kq = k + 4 * q;
+                r.odd = 0u;
+                if (b < NHW) {
+                    if (NGW % 16 != 0 && g0 + 16 * b >= NGW) return;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int n = min(n0 + g0 + 16 * b + NGW * i, a.N - 1);
+                        const WT* src = wg + (long long)n * a.K + kq;
+                        const bool odd = WF != 2 && (reinterpret_cast<uintptr_t>(src) & 2u) != 0;
+                        if (kq + 4 <= a.K && !(odd && ((n == 0 && kq == 0) || (n == a.N - 1 && kq + 4 == a.K)))) {
+                            if constexpr (WF == 2) {
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) r.v[i][e] = __float_as_uint(__ldg(src + e));
+                            } else {
+                                const uint32_t* p = reinterpret_cast<const uint32_t*>(reinterpret_cast<uintptr_t>(src) & ~(uintptr_t)3);
+                                r.v[i][0] = __ldg(p);
+                                r.v[i][1] = __ldg(p + 1);
+                                r.v[i][2] = odd ? __ldg(p + 2) : 0u;
+                                r.odd |= (odd ? 1u : 0u) << i;
+                            }
+                        } else {
+                            uint32_t e[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                if constexpr (WF == 2) e[u] = kq + u < a.K ? __float_as_uint(__ldg(src + u)) : 0u;
+                                else e[u] = kq + u < a.K ? (uint32_t)__ldg(src + u) : 0u;
+                            }
+                            if constexpr (WF == 2) {
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) r.v[i][u] = e[u];
+                            } else {
+                                r.v[i][0] = e[0] | (e[1] << 16);
+                                r.v[i][1] = e[2] | (e[3] << 16);
+                                r.v[i][2] = 0u;
+                            }
+                        }
+                    }
+                } else {
+                    const int h = b - NHW;
+                    if (NGX % 16 != 0 && g0 + 16 * h >= NGX) return;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int m = min(m0 + g0 + 16 * h + NGX * i, a.M - 1);
+                        const float* src = a.x + (long long)m * a.K + kq;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) r.v[i][e] = kq + e < a.K ? __float_as_uint(__ldg(src + e)) : 0x80000000u;
+                    }
+                }
+            };
+            auto store = [&](const Block& r, int b, uint32_t stage) {
+                float f[4][4];                       // [row][k]
+                uint32_t dst;
+                uint32_t pitch;
+                if (b < NHW) {
+                    if (NGW % 16 != 0 && g0 + 16 * b >= NGW) return;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if constexpr (WF == 2) {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) f[i][e] = __uint_as_float(r.v[i][e]);
+                        } else {
+                            const uint32_t sel = ((r.odd >> i) & 1u) ? 0x5432u : 0x3210u;
+                            const uint32_t lo = __byte_perm(r.v[i][0], r.v[i][1], sel), hi = __byte_perm(r.v[i][1], r.v[i][2], sel);
+                            f[i][0] = up16_lo<WF>(lo); f[i][1] = up16_hi<WF>(lo);
+                            f[i][2] = up16_lo<WF>(hi); f[i][3] = up16_hi<WF>(hi);
+                        }
+                    }
+                    pitch = T::kWPitch;
+                    dst = stage + (uint32_t)(4 * q * T::kWPitch + ((g0 + 16 * b) << 4));
+                } else {
+                    const int h = b - NHW;
+                    if (NGX % 16 != 0 && g0 + 16 * h >= NGX) return;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) f[i][e] = __uint_as_float(r.v[i][e]);
+                    pitch = T::kXPitch;
+                    dst = stage + T::kWBytes + (uint32_t)(4 * q * T::kXPitch + ((g0 + 16 * h) << 4));
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sts128(dst + (uint32_t)e * pitch, f[0][e], f[1][e], f[2][e], f[3][e]);
+            };
+            auto advance = [&]() {
+                k += BK;
+                if (--left == 0) { ++j; open(); }
+            };
+            // narrow tiles leave the registers to have a whole slab on its way, wide ones a block
+            constexpr bool kSlabAhead = !T::kWide;
+            Block r[kSlabAhead ? NB : 2];
+#pragma unroll
+            for (int b = 0; b < (kSlabAhead ? NB : 1); ++b) load(r[b], b);
+            int st = 0;
+            unsigned phase = 0;
+#pragma unroll 1
+            for (int it = 0; it < n_it; ++it) {
+                if (it >= ST) {
+                    const bool ok = mbar_wait(empty0 + 8 * st, phase ^ 1u, abort_flag, a.status, a.wait_limit_ns, 3);
+                    if (!__all_sync(0xffffffffu, ok)) return;
+                }
+                const uint32_t stage = ring + (uint32_t)(st * kStageBytes);
+                if constexpr (kSlabAhead) {
+                    advance();
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) {
+                        store(r[b], b, stage);
+                        if (it + 1 < n_it) load(r[b], b);
+                    }
+                } else {
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) {
+                        if (b + 1 < NB) {
+                            load(r[(b + 1) & 1], b + 1);
+                        } else {
+                            advance();
+                            if (it + 1 < n_it) load(r[NB & 1], 0);
+                        }
+                        store(r[b & 1], b, stage);
+                    }
+                    if constexpr (NB & 1) r[0] = r[1];
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(full0 + 8 * st);
+                if (++st == ST) { st = 0; phase ^= 1u; }
+            }
+            return;
+        }
+        constexpr int RSN = RS > 0 ? RS : 1;         // (nothing below is reached without raw stages)
         Cursor c{};
         auto cursor_at = [&](int j) {
             c.j = j;
@@ -325,7 +482,7 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             // aborting: wait (bounded) for the requests still in flight
             const unsigned long long t0 = global_timer_ns();
             for (int i = requested > RS ? requested - RS : 0; i < requested; ++i)
-                while (!(withhold && i == 0) && !mbar_try_wait(rawfull0 + 8 * (i % RS), (uint32_t)(i / RS) & 1u))
+                while (!(withhold && i == 0) && !mbar_try_wait(rawfull0 + 8 * (i % RSN), (uint32_t)(i / RSN) & 1u))
                     if (global_timer_ns() - t0 > a.wait_limit_ns) return;
         }
         return;
@@ -518,6 +675,7 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             using Eight = std::integral_constant<int, 8>;
             using Four = std::integral_constant<int, 4>;
             int n = min(BK, k_left);
+            if constexpr (PLAIN) n = (n + 7) & ~7;   // the operands beyond K change nothing
             k_left -= BK;
 #pragma unroll 1
             for (; n > 8; n -= 8) {
@@ -529,7 +687,7 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             // the last k of the slab are followed by the first ones of the next slab, if that has been prepared already
             loaded = __all_sync(0xffffffffu, mbar_test_wait(full0 + 8 * st, phase));
             const uint32_t off_n = loaded ? (uint32_t)(st * kStageBytes) : off;
-            if (WF != 2 || n == 8) steps(wp, xp, rp, w_thr + off_n, x_thr + off_n, x_rem + off_n, Eight());
+            if (WF != 2 || PLAIN || n == 8) steps(wp, xp, rp, w_thr + off_n, x_thr + off_n, x_rem + off_n, Eight());
             else steps(wp, xp, rp, w_thr + off_n, x_thr + off_n, x_rem + off_n, Four());
             __syncwarp();
             if (lane == 0) mbar_arrive(empty0 + 8 * st_cur);
