@@ -136,7 +136,11 @@ DET_API det_linear_plan_t* det_linear_plan_shard(int64_t M, int64_t N, int64_t K
  * the stream STARTS (the decode kernel is launched with programmatic dependent launch and requests
  * its first weight tiles, and reads b, before it waits for that kernel to finish; only x and y are
  * touched after the wait).  If W or b were just written on the same stream -- a dequantise or copy
- * kernel, a device-side random fill -- put another kernel or a synchronisation in between.  The fast kernels need K % 8 == 0 and 16-byte aligned x, W, y; anything else runs a
+ * kernel, a device-side random fill -- put another kernel or a synchronisation in between.  Of this library's own kernels, those of
+ * det_rmsnorm, det_attention_decode, det_linear_run_noalloc, the prefill bucket and the generic decode kernel count as such:
+ * they let the next kernel start only once everything before them is complete.  The fast decode kernel and det_argmax_rows
+ * do not count: they start, and let the next kernel start, while the kernel before them may still be running.
+ * The fast kernels need K % 8 == 0 and 16-byte aligned x, W, y; anything else runs a
  * slower generic kernel that produces the same bits.  Errors: DET_ERR_INVALID_ARG for NULL
  * arguments, DET_ERR_CUDA if a launch fails.  Nothing is launched when an error is returned.
  */

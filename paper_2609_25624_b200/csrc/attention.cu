@@ -414,8 +414,9 @@ attention_decode_kernel(const float* __restrict__ q, const float* __restrict__ k
     float* l_s = part + (size_t)segs_per_block * G * D;        // [16] denominators of the heads of this block
     float* red = l_s + 16;                                     // [8][kAttnWarps] the warps' row maxima, by head
     const uint32_t ring0 = ((uint32_t)__cvta_generic_to_shared(red + 8 * kAttnWarps) + kGroupBytes - 1) & ~(uint32_t)(kGroupBytes - 1);   // [kAttnWarps][NS] groups
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // The next kernel may start, and request its weights, only once what precedes this kernel is complete.
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int b = blockIdx.y / Hkv, hk = blockIdx.y % Hkv;

@@ -39,8 +39,9 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
     extern __shared__ __align__(16) float xs[];      // [MT][win]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, threads = blockDim.x;
     const int m0 = blockIdx.y * MT;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // The next kernel may start, and request its weights, only once what precedes this kernel is complete.
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     // activations of the window [w_lo, w_lo + win) into shared memory
     auto stage = [&](unsigned w_lo) {

@@ -139,6 +139,15 @@ __device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.al
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Launches with late weights (kFlagLateWeights) are told from others by an explicit cluster size, of one block: the kernel asks
+// a special register.  A kernel parameter, read before the next kernel is let go, costs every call 0.1 us (3 % of a small layer).
+__device__ __forceinline__ bool launched_as_cluster()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\tmov.pred p, %%is_explicit_cluster;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
+
 __device__ __forceinline__ void consumer_barrier(int threads)
 {
     asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
@@ -146,8 +155,6 @@ __device__ __forceinline__ void consumer_barrier(int threads)
 
 // LaunchArgs::test_flags: bit 0 is a test hook, never set outside the tests.
 constexpr int kTestWithholdFirstX = 1;   // block 0 never requests the activations of its first stage
-constexpr int kLateWeights = kFlagLateWeights;   // weights and bias too are touched only after the previous kernel in the stream
-
 
 // Tensor map of a single row group: a parameter only of the tilings that use it.
 template <bool DEAL> struct GroupMap { typedef CUtensorMap type; };
@@ -204,6 +211,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
     } else {
         asm volatile("bar.sync 2, %0;" ::"r"(C::kThreads) : "memory");
     }
+    if (launched_as_cluster()) pdl_wait();                    // late weights: nothing of this or the next kernel starts earlier
     pdl_launch_dependents();
 
     const int total_shares = sh.n_shares * n_mblocks;         // the host keeps this below 2^31
@@ -307,7 +315,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
         // once, activation requests wait for that kernel to finish.  A thread that requests both sends the
         // first ring of weight requests ahead of the wait.
         int pre = 0;
-        if (do_w && do_x && !(test_flags & kLateWeights)) {
+        if (do_w && do_x) {
             const Cursor c0 = c;
             const bool live0 = live;
             while (live && pre < STAGES) {
@@ -318,7 +326,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
             c = c0;
             live = live0;
         }
-        if (do_x || (test_flags & kLateWeights)) pdl_wait();
+        if (do_x) pdl_wait();
         int st = 0;
         unsigned phase = 0, n_issued = 0;
         bool ok = true;
@@ -347,7 +355,6 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
 
     // ---------------- consumer warps ----------------
     if (C::kMoveRegs) reg_inc<C::kConsumerRegs>();
-    if (test_flags & kLateWeights) pdl_wait();                // (the bias is read ahead of the output's wait)
     const int g = warp / C::kGroupWarps;
     const int gw = warp % C::kGroupWarps;
     const int wm = gw % WM;
@@ -653,11 +660,13 @@ cudaError_t launch_decode_t(const LaunchArgs& a, const CUtensorMap* map_w, const
     cfg.blockDim = dim3(C::kThreads);
     cfg.dynamicSmemBytes = C::smem_bytes(a.S);
     cfg.stream = a.stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = (a.test_flags & kFlagLateWeights) ? 2 : 1;
     typename GroupMap<C::kDealRest>::type group_map{};
     if constexpr (C::kDealRest) group_map = *map_g;
     return cudaLaunchKernelEx(&cfg, kern, *map_w, *map_x, group_map, a.b, a.y, (int)a.M, (int)a.N, (int)a.K, (int)a.seg_len, a.S,

@@ -24,7 +24,8 @@ struct DeviceStatus {
 };
 
 // LaunchArgs::test_flags beyond the test hooks: the decode kernel also waits for the previous kernel in the stream before it
-// touches W and b (callers for whom they are not parameters that were complete long before)
+// touches W and b, and before it lets the next kernel start (callers for whom W and b are not parameters that were complete long
+// before)
 constexpr int kFlagLateWeights = 4;
 
 constexpr int kMaxDevices = 64;     // per-device caches (function attributes, symbol addresses)

@@ -212,9 +212,6 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
     __syncthreads();
     const int blk = shared_ticket;
-    // (after the ticket: the next kernel of the stream may draw tickets of the same plan from here on)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
     Walk w;
     if (a.cut) {
         w.lo = a.total * blk / (int)gridDim.x;
@@ -228,7 +225,6 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     w.u_last = unit_at(a, w.hi - 1);
     const int n_it = (int)(w.hi - w.lo);             // slabs of this block
     const int n_pieces = w.count();
-
     if (warp >= kMulWarps) {
         // ---------------- preparing warps ----------------
         if constexpr (T::kWide) reg_dec<T::kPrepRegs>();
@@ -625,7 +621,10 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     };
 
     constexpr size_t kTileFloats = (size_t)BM * BN;
-    asm volatile("griddepcontrol.wait;" ::: "memory");       // workspaces and y belong to the kernel before this one until it ends
+    // Workspaces and y belong to the kernels before this one until they end.  Then the next kernel may start: not before, since it
+    // may request its weights at once, and not ahead of this block's ticket, since it may draw tickets of the same plan.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     int st = 0;
     unsigned phase = 0;
     bool loaded = false;                             // the first operands of the next slab are in registers already

@@ -161,8 +161,9 @@ rmsnorm_block_per_row_kernel(const float* __restrict__ x, const float* __restric
 {
     extern __shared__ __align__(16) float4 row[];
     __shared__ float r_shared;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // The next kernel may start, and request its weights, only once what precedes this kernel is complete.
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tid = threadIdx.x, lane = tid & 31, quads = H / 4;
     const float4* xr = reinterpret_cast<const float4*>(x + (size_t)blockIdx.x * H);
     const float4* gr = reinterpret_cast<const float4*>(g);
