@@ -137,8 +137,8 @@ DET_API det_linear_plan_t* det_linear_plan_shard(int64_t M, int64_t N, int64_t K
  * its first weight tiles, and reads b, before it waits for that kernel to finish; only x and y are
  * touched after the wait).  If W or b were just written on the same stream -- a dequantise or copy
  * kernel, a device-side random fill -- put another kernel or a synchronisation in between.  Of this library's own kernels, those of
- * det_rmsnorm, det_attention_decode, det_linear_run_noalloc, the prefill bucket and the generic decode kernel count as such:
- * they let the next kernel start only once everything before them is complete.  The fast decode kernel and det_argmax_rows
+ * det_rmsnorm, det_attention_decode, det_linear_run_noalloc, det_linear_run_host*, the prefill bucket and the generic decode
+ * kernel count as such: they let the next kernel start only once everything before them is complete.  The fast decode kernel and det_argmax_rows
  * do not count: they start, and let the next kernel start, while the kernel before them may still be running.
  * The fast kernels need K % 8 == 0 and 16-byte aligned x, W, y; anything else runs a
  * slower generic kernel that produces the same bits.  Errors: DET_ERR_INVALID_ARG for NULL
@@ -157,8 +157,9 @@ DET_API det_status_t det_linear_run_w(const det_linear_plan_t* plan, const float
 /*
  * End-to-end variant with HOST activations: copies x (host, [M,K]) to a plan-owned device buffer,
  * runs the same kernels, copies y back to y_host (host, [M,N]) and waits for the stream.  W (in the
- * plan's weight format) and b stay device-resident (they are the model's parameters).  The staging buffers are allocated on
- * first use.  Synchronises `stream` before returning.
+ * plan's weight format) and b stay device-resident (they are the model's parameters); they may be written by the kernel before
+ * this call in the stream: nothing of them is read before the copy of x has begun, which waits for that kernel.
+ * The staging buffers are allocated on first use.  Synchronises `stream` before returning.
  */
 DET_API det_status_t det_linear_run_host(det_linear_plan_t* plan, const float* x_host, const void* W,
                                  const float* b, float* y_host, void* stream);

@@ -51,11 +51,12 @@ cudaError_t launch_combine(const LaunchArgs& a)
 }
 
 // Small activations from (mapped) pinned host memory to device memory: 16-byte loads across the bus, all of them on their way at
-// once, and the kernel after this one may start its prologue and its weight stream meanwhile.
+// once, and the kernel after this one may start its prologue and its weight stream meanwhile.  Not before this kernel's own
+// wait: W and b may have been written by the kernel before it.
 __global__ void __launch_bounds__(256) copy_from_host_kernel(const float4* __restrict__ src, float4* __restrict__ dst, unsigned n)
 {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) dst[i] = __ldcv(src + i);
 }
 

@@ -92,3 +92,22 @@ def test_weights_written_before_the_kernel_in_between(between):
     plan = B.det_linear_plan_w(2, 64, 256, "fp32")
     _check(_writer(64, 256, 16384), W, BETWEEN[between](), lambda: B.det_linear_run(plan, x, W, None, y), y)
     plan.close()
+
+
+# activations that come over by a kernel (pinned and small) and by a copy
+@pytest.mark.parametrize("M,N,pinned", [(3, 256, True), (30, 256, True), (3, 256, False), (70, 256, True)])
+def test_bias_written_before_a_run_on_host_activations(M, N, pinned):
+    W, b = _normal(22, N, 512).to(torch.bfloat16), torch.empty(1, N, device="cuda")
+    x, y = _normal(21, M, 512).cpu(), torch.empty(M, N)
+    if pinned:
+        x, y = x.pin_memory(), y.pin_memory()
+    plan = B.det_linear_plan(M, N, 512)
+    _check(_writer(1, N, 65536), b, lambda: None, lambda: B.det_linear_run_host(plan, x, W, b[0], y), y)
+    plan.close()
+
+
+def test_weights_written_before_a_run_on_host_activations():
+    W, x, y = torch.empty(64, 256, device="cuda"), _normal(21, 2, 256).cpu().pin_memory(), torch.empty(2, 64).pin_memory()
+    plan = B.det_linear_plan_w(2, 64, 256, "fp32")
+    _check(_writer(64, 256, 16384), W, lambda: None, lambda: B.det_linear_run_host(plan, x, W, None, y), y)
+    plan.close()
