@@ -48,13 +48,14 @@ __device__ __forceinline__ typename WVec<WF>::type wload(uint32_t addr)
     if constexpr (WF == 2) return lds128(addr);
     else return lds64(addr);
 }
-template <int WF>
+template <int WF, bool SHIFT>
 __device__ __forceinline__ float wget(const typename WVec<WF>::type& v, int kk)
 {
     if constexpr (WF == 2) {
         return kk == 0 ? v.x : kk == 1 ? v.y : kk == 2 ? v.z : v.w;
     } else {
         const uint32_t w = (kk < 2) ? v.x : v.y;
+        if (WF == 0 && SHIFT && !(kk & 1)) return __uint_as_float(w << 16);
         return (kk & 1) ? up16_hi<WF>(w) : up16_lo<WF>(w);
     }
 }
@@ -98,6 +99,14 @@ struct Cfg {
     // 128256 rows: 200 us without, 207 with), and tiles of 28 rows lose more by the extra bookkeeping (M = 32, 1 %) than
     // their smaller rounds leave to gain.
     static constexpr bool kDealRest = kMB >= 16 && kRB >= 56;
+    // BF16: the lower half of a word is widened by a byte permutation, or by a shift in the 4-row tilings of two segment groups
+    // that run two blocks to an SM at the full 128 registers: M = 24, N = 6144, K = 4096 35.5 us by shift, 39.4 by permutation (M =
+    // 8, N = K = 4096 9.86 and 9.72).  Elsewhere the permutation is up to 3 % faster: M = 48, N = 28672, K = 4096 274.8 and 282.6.
+    static constexpr bool kShift = MT == 4 && SK == 2 && kConsumerWarps == 4;
+    // Ask whether the next stage has landed after the last chunk's loads, which then do not wait for the answer, or before them:
+    // M = 16, N = 4096, K = 14336 44.8 us after, 46.1 before with BF16 weights, but 53.1 and 51.6 with FP16 weights, whose
+    // conversions fill the 4-row tiles' registers.
+    static constexpr bool kLookEarly = WF == 1 && MT == 4;
     static constexpr int kFixedSmem = kRingBytes + kBarBytes + 128;               // + 128 for alignment
     static constexpr int kLM = ilog2(MT);
     static constexpr int kKeep = RT / 2;                      // sums a lane holds after the lane tree
@@ -214,20 +223,19 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
     if (launched_as_cluster()) pdl_wait();                    // late weights: nothing of this or the next kernel starts earlier
     pdl_launch_dependents();
 
-    const int total_shares = sh.n_shares * n_mblocks;         // the host keeps this below 2^31
-    const int last_tile = C::kDealRest ? sh.whole_rounds : 0;      // number of a share's last tile
+    const int total_units = sh.n_shares * n_mblocks;          // the host keeps this below 2^31
     const int rounds = S / SK;                                // the host only picks tilings with S % SK == 0
 
-    // Share v -> (batch block fastest, then row groups): the batch blocks of the same rows run side by side, so the weights
-    // come from HBM once and from L2 for the other blocks.  A share has whole_rounds tiles of WR row groups, dealt out
-    // round robin, and one last tile of its part of the remaining groups (at most WR; none if grp == grp_hi).
-    // Without dealing out the rest (C::kDealRest), a share is one tile.
-    auto tile_of = [&](int v, int k, int& grp, int& grp_hi, int& mb) {
-        int i = v;
+    // Work unit u -> (batch block fastest, then row groups): the batch blocks of the same rows run side by side, so the weights
+    // come from HBM once and from L2 for the other blocks.  A unit is one tile or, where the rest is dealt out (C::kDealRest), a
+    // share: whole_rounds tiles of WR row groups, dealt out round robin, and one last tile of its part of the remaining groups
+    // (at most WR; none if grp == grp_hi).
+    auto tile_of = [&](int u, [[maybe_unused]] int t, int& grp, int& grp_hi, int& mb) {
+        int i = u;
         mb = 0;
-        if (n_mblocks > 1) { i = v / n_mblocks; mb = v - i * n_mblocks; }
-        if (!C::kDealRest || k < sh.whole_rounds) {
-            grp = (k * sh.n_shares + i) * WR;
+        if (n_mblocks > 1) { i = u / n_mblocks; mb = u - i * n_mblocks; }
+        if (!C::kDealRest || t < sh.whole_rounds) {
+            grp = ((C::kDealRest ? t * sh.n_shares : 0) + i) * WR;
             grp_hi = grp + WR;
         } else {
             grp = sh.whole_rounds * sh.n_shares * WR + i * sh.rest_each + min(i, sh.rest_more);
@@ -255,21 +263,26 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
         const uint32_t emptyg = empty0 + 8 * g * STAGES;
         const uint32_t ringg = smem_base + (uint32_t)(g * STAGES * C::kStageBytes);
 
-        // Position in the group's stream of stages: share, tile of the share, its row groups and batch block, round, first k.
+        // Position in the group's stream of stages: work unit, tile of the unit, its row groups and batch block, round, first k.
         struct Cursor {
-            int v, t, grp, grp_hi, mb, r, k0, k_hi;
+            int u, t, grp, grp_hi, mb, r, k0, k_hi;
         };
-        // the first tile that is not empty from (c.v, c.t) on
+        // the first tile that is not empty from (c.u, c.t) on
         auto find_tile = [&](Cursor& c) -> bool {
-            for (; c.v < total_shares; c.v += (int)gridDim.x, c.t = 0)
-                for (; c.t <= last_tile; ++c.t) {
-                    tile_of(c.v, c.t, c.grp, c.grp_hi, c.mb);
-                    if (!C::kDealRest || c.grp < c.grp_hi) return true;
+            for (; c.u < total_units; c.u += (int)gridDim.x, c.t = 0) {
+                if (!C::kDealRest) {
+                    tile_of(c.u, 0, c.grp, c.grp_hi, c.mb);
+                    return true;
                 }
+                for (; c.t <= sh.whole_rounds; ++c.t) {
+                    tile_of(c.u, c.t, c.grp, c.grp_hi, c.mb);
+                    if (c.grp < c.grp_hi) return true;
+                }
+            }
             return false;
         };
         auto start = [&](Cursor& c) -> bool {
-            c.v = (int)blockIdx.x;
+            c.u = (int)blockIdx.x;
             c.t = c.r = 0;
             if (!find_tile(c)) return false;
             seg_range(g, c.k0, c.k_hi);
@@ -280,7 +293,8 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
             if (c.k0 < c.k_hi) return true;
             if (++c.r == rounds) {
                 c.r = 0;
-                ++c.t;
+                if (C::kDealRest) ++c.t;
+                else c.u += (int)gridDim.x;
                 if (!find_tile(c)) return false;
             }
             seg_range(c.r * SK + g, c.k0, c.k_hi);
@@ -379,14 +393,21 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
     bool ready = false;
     constexpr int kKeep = C::kKeep;
 
-    for (int v = (int)blockIdx.x; v < total_shares; v += (int)gridDim.x)
-#pragma unroll 1
-    for (int t = 0; t <= last_tile; ++t) {
-        int mb, grp, grp_hi;
-        tile_of(v, t, grp, grp_hi, mb);
-        if (C::kDealRest && grp == grp_hi) continue;
-        const int n_tile = C::kDealRest ? (grp_hi - grp) * RT : C::kRB;      // weight rows of this tile
-        const int row0 = grp * RT;                            // its first row
+    // (the loop over a unit's tiles is no loop where a unit is one tile, but the 8-row tiles come out 1 % faster if it stays one)
+    for (int u = (int)blockIdx.x; u < total_units; u += (int)gridDim.x)
+#pragma unroll (MT == 8 ? 1 : 2)
+    for (int t = 0; t <= (C::kDealRest ? sh.whole_rounds : 0); ++t) {
+        // (In the smaller warp tiles as remainder and quotient of u: the compiler then leaves both to the end of the unit and keeps
+        // their registers for the multiply loop.  tile_of's form of the same takes M = 8, N = 40, K = 8192 from 10.1 to 11.0 us,
+        // M = 24, N = 6144, K = 4096 with FP32 weights from 64.5 to 72.3.)
+        int mb = u % n_mblocks, row0 = u / n_mblocks * C::kRB, n_tile = C::kRB;     // batch block; first row, number of rows
+        if constexpr (C::kDealRest || MT == 8) {
+            int grp, grp_hi;
+            tile_of(u, t, grp, grp_hi, mb);
+            if (C::kDealRest && grp == grp_hi) continue;
+            n_tile = (grp_hi - grp) * RT;
+            row0 = grp * RT;
+        }
         const bool mine = !C::kDealRest || wr * RT < n_tile;  // the last tile of a share may have no rows for this warp
         float tot[kKeep];                                     // running fold over the segments when SK == 1
 
@@ -442,7 +463,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                             float2 wp[kMaxPass];
 #pragma unroll
                             for (int j = 0; j < kMaxPass; ++j) {
-                                if (j < np) wp[j] = make_float2(wget<WF>(w[2 * j], kk), wget<WF>(w[2 * j + 1], kk));
+                                if (j < np) wp[j] = make_float2(wget<WF, C::kShift>(w[2 * j], kk), wget<WF, C::kShift>(w[2 * j + 1], kk));
                             }
 #pragma unroll
                             for (int m = 0; m < MT; ++m) {
@@ -462,7 +483,8 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     {
 #pragma unroll(MT * RT >= 64 ? 1 : 2)
                         for (int cc = 0; cc < KC / 128 - 1; ++cc) chunk(cc, false);
-                        chunk(KC / 128 - 1, true);
+                        if (C::kLookEarly) ready = mbar_test_wait(fullg + 8 * st, phase);
+                        chunk(KC / 128 - 1, !C::kLookEarly);
                     }
                 } else {
                     ready = false;
@@ -545,7 +567,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     // ---- bias and store straight from the owner lanes ----
                     const int m = mb * C::kMB + wm * MT + m_slot;
                     const int n0 = row0 + wr * RT + b0;
-                    const int n_hi = min(N, row0 + n_tile);       // (rows beyond the range are another block's)
+                    const int n_hi = C::kDealRest ? min(N, row0 + n_tile) : N;       // (rows beyond the range are another block's)
                     float bv[kKeep];
 #pragma unroll
                     for (int j = 0; j < kKeep; ++j) bv[j] = (bias != nullptr && owner && n0 + 2 * j < n_hi) ? __ldg(bias + n0 + 2 * j) : 0.0f;
@@ -577,7 +599,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                 for (int o = threadIdx.x; o < C::kTile; o += C::kConsumerWarps * 32) {
                     const int ml = o / C::kRB, nl = o % C::kRB;
                     const int m = mb * C::kMB + ml, n = row0 + nl;
-                    if (m < M && nl < n_tile && n < N) {
+                    if (m < M && (!C::kDealRest || nl < n_tile) && n < N) {
                         float t = part[o];
                         for (int s2 = 1; s2 < S; ++s2) t = __fadd_rn(t, part[s2 * C::kTile + o]);
                         if (bias) t = __fadd_rn(t, o == (int)threadIdx.x ? b_first : __ldg(bias + n));
