@@ -30,8 +30,8 @@
 // every lane copies the elements that it will itself consume, K first, then V, through a ring of its own in shared
 // memory (cp.async: no registers held, no barrier, nobody else reads them), several groups ahead; while the cluster agrees on
 // maxima and weights, the ring fills with V.  (Asking for more of V in L2 ahead of use, by bulk prefetch, gained nothing.)
-// A block whose scores leave no room for the ring (three groups) loads through registers instead; such shapes have more blocks
-// than fit at once, and their phases overlap each other.  Next come the instructions: the lane trees (their operands are
+// A block whose scores leave no room for the ring (three groups), or with too little to do for it, loads through registers instead
+// (ring_or_registers below).  Next come the instructions: the lane trees (their operands are
 // permuted so that no step selects between registers), P.V in packed FMAs.  Small shapes are bound by latency, of reads
 // from other blocks' shared memory among others: what crosses blocks is read many values at a time.
 // Measured on B200, 32 query / 8 KV heads, D = 128, us a call before -> now: B = 8, T = 4096 59.3 -> 53.5; B = 8, T = 8192 105.6 -> 86.9;
@@ -46,11 +46,15 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kAttnWarps = 8;            // warps that score keys and multiply values; one more forms the denominators meanwhile
-constexpr int kAttnThreads = 32 * (kAttnWarps + 1);
+constexpr int kAttnWarps = 8;            // warps that score keys and multiply values
 constexpr int kWorkThreads = 32 * kAttnWarps;
+// NS slots of the ring (see below); 0 and 1 stand for loads through registers, by eight warps or with a ninth one that forms the
+// denominators meanwhile (as it does with the ring).
+template <int NS> constexpr int kAttnThreads = kWorkThreads + (NS > 0 ? 32 : 0);
+// Blocks to an SM, which cap a thread's registers: with eight warps, as many as leave eight keys in flight their registers.
+template <int G, int DC, int NS> constexpr int kAttnBlocks = NS != 0 ? 2 : G * DC <= 2 ? 4 : G * DC <= 8 ? 2 : 1;
 // keys a warp scores together when they come through registers
-template <int G, int DC> constexpr int kPassKeys = G * DC >= 16 ? 2 : G * DC >= 8 ? 4 : 8;
+template <int G, int DC, int NS> constexpr int kPassKeys = NS == 1 && G * DC >= 16 ? 2 : 8;
 constexpr int kGroupBytes = 2048;        // ring: bytes a warp copies as one group
 constexpr int kSegKeys = 256;            // P.V segment length (part of the order)
 constexpr int kMaxCluster = 16;          // blocks per row at most (8 is the portable cluster size, 16 needs the opt-in below)
@@ -399,7 +403,7 @@ __device__ __forceinline__ void ring_pv(Ring<DC, NS>& ring, VCursor<VW>& ahead, 
 // ring (0: loads through registers); VW: consecutive d per lane in P.V.
 // Grid (C, B Hkv) in clusters of (C, 1, 1); Tc = keys per block (a multiple of 256), t_pitch = Tc.
 template <int G, int DC, int NS, int VW>
-__global__ void __launch_bounds__(kAttnThreads, 2)
+__global__ void __launch_bounds__(kAttnThreads<NS>, kAttnBlocks<G, DC, NS>)
 attention_decode_kernel(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, float scale,
                         int Hq, int Hkv, int T, int D, int Tc, float* __restrict__ o)
 {
@@ -431,7 +435,7 @@ attention_decode_kernel(const float* __restrict__ q, const float* __restrict__ k
 
     const int n_slices = (D + 32 * VW - 1) / (32 * VW);
     [[maybe_unused]] const int n_items = n_seg_l * n_slices;
-    [[maybe_unused]] Ring<DC, NS == 0 ? 3 : NS> ring;
+    [[maybe_unused]] Ring<DC, NS < 2 ? 3 : NS> ring;
     [[maybe_unused]] VCursor<VW> ahead;
 
     // the lane's elements of a row of D floats: d = 128 c + 4 lane + jj (all four inside or outside D: D % 4 == 0)
@@ -442,14 +446,14 @@ attention_decode_kernel(const float* __restrict__ q, const float* __restrict__ k
     // ---- step 1: scores of the block's keys ----
     if (warp < kAttnWarps) {
         // (with the ring, the lane's own order of the heads: see ring_scores)
-        const int head_perm = NS > 0 ? lane_perm<Scatter<(4 / DC) * G>::kSteps>(lane) % G : 0;
+        const int head_perm = NS > 1 ? lane_perm<Scatter<(4 / DC) * G>::kSteps>(lane) % G : 0;
         float4 qv[G][DC];
 #pragma unroll
         for (int g = 0; g < G; ++g)
 #pragma unroll
             for (int c = 0; c < DC; ++c)
                 qv[g][c] = d_ok[c] ? __ldg(reinterpret_cast<const float4*>(qb + (size_t)(g ^ head_perm) * D + 128 * c + 4 * lane)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        if constexpr (NS > 0) {
+        if constexpr (NS > 1) {
             ring.init(ring0 + warp * NS * kGroupBytes, lane);
             ahead.open(warp, n_items, n_slices, Tl);
             float m = ring_scores<G, DC, NS, VW>(ring, ahead, qv, d_ok, scale, kb, vb, e_s, Tc, Tl, D, n_items, n_slices, warp, lane);
@@ -459,7 +463,7 @@ attention_decode_kernel(const float* __restrict__ q, const float* __restrict__ k
             for (int i = 0; i < kKeyBits; ++i) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1 << i));
             if ((lane >> kKeyBits) < G && (lane & ((1 << kKeyBits) - 1)) == 0) red[head_perm * kAttnWarps + warp] = m;
         } else {
-        constexpr int kKeysPerPass = kPassKeys<G, DC>;
+        constexpr int kKeysPerPass = kPassKeys<G, DC, NS>;
         float top[G];                                          // the lane's row maxima
 #pragma unroll
         for (int g = 0; g < G; ++g) top[g] = -INFINITY;
@@ -549,11 +553,11 @@ attention_decode_kernel(const float* __restrict__ q, const float* __restrict__ k
     }
     cluster.sync();                                            // every block's weights are in place
 
-    // ---- step 4: denominators, by a warp of their own (head g in block g mod C) while the others go on; the 32 chains of a
-    // sum are the warp's lanes and run over ALL keys in ascending chunks of 128, reading the other blocks' weights in place,
-    // eight chunks at a time (a read from another block takes as long as some hundred instructions) ----
-    if (warp == kAttnWarps) {
-        for (int g = rank; g < G; g += C) {
+    // ---- step 4: denominators (head g in block g mod C), with the ring by a warp of their own while the others go on; the 32
+    // chains of a sum are a warp's lanes and run over ALL keys in ascending chunks of 128, reading the other blocks' weights in
+    // place, eight chunks at a time (a read from another block takes as long as some hundred instructions) ----
+    if (NS == 0 || warp == kAttnWarps) {
+        for (int g = rank + (NS == 0 ? C * warp : 0); g < G; g += NS == 0 ? C * kAttnWarps : C) {
             float a = 0.0f;
             int owner = 0, c = 0;                              // next chunk: block and first key in the block
             for (int k0 = 0; k0 < T; k0 += 1024) {
@@ -585,7 +589,7 @@ attention_decode_kernel(const float* __restrict__ q, const float* __restrict__ k
     // Items are dealt to the warps round robin; the slices are as wide as still leaves every warp an item, so a
     // block with two segments keeps all eight warps loading and a block with many uses 16-byte loads ----
     if (warp < kAttnWarps) {
-        if constexpr (NS > 0) ring_pv<G, DC, NS, VW>(ring, ahead, e_s, part, vb, Tc, Tl, D, n_items, n_slices, warp, lane);
+        if constexpr (NS > 1) ring_pv<G, DC, NS, VW>(ring, ahead, e_s, part, vb, Tc, Tl, D, n_items, n_slices, warp, lane);
         else pv_items<G, VW>(e_s, part, vb, Tc, Tl, D, n_seg_l, warp, lane);
     }
     cluster.sync();                                            // segment sums and denominators are in place
@@ -594,7 +598,7 @@ attention_decode_kernel(const float* __restrict__ q, const float* __restrict__ k
     {
         const int per = (G * D + C - 1) / C;
         const int i_lo = rank * per, i_hi = min(G * D, i_lo + per);
-        for (int i = i_lo + (int)threadIdx.x; i < i_hi; i += kAttnThreads) {
+        for (int i = i_lo + (int)threadIdx.x; i < i_hi; i += kAttnThreads<NS>) {
             const int g = i / D;
             const float l = cluster.map_shared_rank(l_s, g % C)[g];
             float t = 0.0f;
@@ -642,6 +646,32 @@ int ring_slots(size_t base)
     return base + 5 * slot <= limit ? 5 : base + 3 * slot <= limit ? 3 : 0;
 }
 
+// The ring's slots, or 0 or 1 for loads through registers (see kAttnThreads).  Times in us on 148 SMs.
+int ring_or_registers(int G, int DC, int D, int Tc, long long blocks, int sm_count, int slots)
+{
+    const int work = G * DC;                         // float4s of q a lane holds
+    // Few blocks of a single segment each: half of the warps have no P.V item and the others' 256 keys are one chain of loads and
+    // additions, which starts sooner through registers (32 / 8 heads, D = 128: B = 1, T = 512 14.6, with the ring 17.1; but B = 4,
+    // T = 1024, 128 blocks, 24.2 and 21.2).  A ninth warp takes 0.3 off where it leaves eight keys their registers.
+    if (Tc <= kSegKeys && blocks <= sm_count / 2) return work < 8 ? 1 : 0;
+    // Many blocks with little to do, or rows of half a chunk, which fill half of a ring: four blocks to an SM without the ring's
+    // shared memory (16 / 8 heads, D = 128, B = 64: T = 64 13.6 and 17.8 with the ring, T = 512 53.0 and 58.5; 32 / 32, D = 64, B = 16,
+    // T = 8192 333 and 435; but 32 / 32, D = 128, B = 16, T = 4096 3.5 % slower)
+    if (work <= 2 && blocks > 2 * sm_count && (Tc <= 1024 || D <= 64)) return 0;
+    if (work >= 16) {
+        // Eight heads of more than 128 elements take 168 registers for eight keys in flight: one block to an SM, the better form where
+        // one is enough (64 / 8, D = 256: B = 4, T = 1024 34.1, with the ring 44.2; B = 1, T = 8192 83.5, with two keys in flight
+        // and two blocks to an SM 182) ...
+        if (blocks <= sm_count) return 0;
+        // ... and where not even two make it a single wave (B = 16, T = 4096 325 and 420); in between 248 and 213 (B = 4, T = 8192)
+        if (slots == 0) return blocks <= 2 * sm_count ? 1 : 0;
+    }
+    // no room for a ring (eight heads, D = 128, B = 16, T = 4096 138 by eight warps, 193 by nine with four keys in flight; four
+    // heads, B = 8, T = 32768 393 and 384 with eight keys in flight either way)
+    if (slots == 0) return work < 8 ? 1 : 0;
+    return slots;
+}
+
 template <int G, int DC, int NS, int VW>
 cudaError_t launch_variant(const cudaLaunchConfig_t* cfg, bool query, const float* q, const float* k, const float* v, float scale, int Hq, int Hkv, int T, int D,
                            int Tc, float* o)
@@ -676,17 +706,13 @@ cudaError_t launch_attention_t(const float* q, const float* k, const float* v, f
         const int Tc = keys_per_block(T, C);
         const size_t base = block_smem_bytes(G, Tc, D);
         if (base > 227u * 1024u) return cudaErrorLaunchOutOfResources;
-        // Few blocks of a single segment each: half of the warps have no P.V item and the others' 256 keys are one chain of loads and
-        // additions, which starts sooner through registers (B = 1, T = 512 13.7 us, with the ring 17.1; but B = 4, T = 1024,
-        // 128 blocks, 24.2 and 21.2)
-        const bool tiny = Tc <= kSegKeys && (long long)C * B * Hkv <= sm_count / 2;
-        const int ns = tiny ? 0 : ring_slots(base);
+        const int ns = ring_or_registers(G, DC, D, Tc, (long long)C * B * Hkv, sm_count, ring_slots(base));
         // P.V items: (segment, slice of 32 VW consecutive d), the widest slices that still give every warp of a block an item
         const int segs = Tc / kSegKeys;
         const int vw = segs * ((D + 127) / 128) >= kAttnWarps ? 4 : segs * ((D + 63) / 64) >= kAttnWarps ? 2 : 1;
         cfg.gridDim = dim3((unsigned)C, (unsigned)(B * Hkv));
-        cfg.blockDim = dim3(kAttnThreads);
-        cfg.dynamicSmemBytes = base + (ns ? (size_t)ns * kAttnWarps * kGroupBytes + kGroupBytes : 0);     // + alignment
+        cfg.blockDim = dim3(ns ? kAttnThreads<1> : kAttnThreads<0>);
+        cfg.dynamicSmemBytes = base + (ns > 1 ? (size_t)ns * kAttnWarps * kGroupBytes + kGroupBytes : 0);     // + alignment
         cfg.stream = stream;
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = (unsigned)C;
@@ -698,10 +724,12 @@ cudaError_t launch_attention_t(const float* q, const float* k, const float* v, f
         auto go = [&](bool query) -> cudaError_t {
             cfg.numAttrs = query ? 1 : 2;
 #define DET_ATTN_V(NS_, VW_) return launch_variant<G, DC, NS_, VW_>(&cfg, query, q, k, v, scale, Hq, Hkv, T, D, Tc, o)
-#define DET_ATTN_N(NS_) do { if (vw == 4) DET_ATTN_V(NS_, 4); if (vw == 2) DET_ATTN_V(NS_, 2); DET_ATTN_V(NS_, 1); } while (0)
-            if (ns == 5) DET_ATTN_N(5);
-            if (ns == 3) DET_ATTN_N(3);
-            DET_ATTN_N(0);
+#define DET_ATTN_N(NS_) { if (vw == 4) DET_ATTN_V(NS_, 4); if (vw == 2) DET_ATTN_V(NS_, 2); DET_ATTN_V(NS_, 1); }
+            if (ns == 5) DET_ATTN_N(5)
+            if (ns == 3) DET_ATTN_N(3)
+            if constexpr (G * DC != 8) { if (ns == 1) DET_ATTN_N(1) }
+            if constexpr (G * DC != 4) DET_ATTN_N(0)      // (never without the ninth warp)
+            return cudaErrorInvalidValue;
 #undef DET_ATTN_N
 #undef DET_ATTN_V
         };

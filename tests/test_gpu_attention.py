@@ -145,3 +145,17 @@ def test_attention_streaming_schedules(B_, Hq, Hkv, T, D):
     got = run_gpu_attention(q, k, v, scale)
     assert not np.isnan(got).any()
     assert_bits_equal(got, want, f"attention {B_},{Hq},{Hkv},{T},{D}")
+
+
+# loads through registers: by eight warps at four, two and one block to an SM (many short rows, half-filled chunks, eight heads
+# without room for a ring, eight heads of more than 128 elements), by nine warps (few blocks; eight such heads between one and
+# two blocks to an SM)
+@pytest.mark.parametrize("B_,Hq,Hkv,T,D", [(40, 8, 8, 130, 128), (40, 16, 8, 257, 64), (75, 8, 4, 33, 4), (300, 1, 1, 2049, 64), (38, 8, 8, 200, 256), (19, 64, 8, 1500, 128),
+                                           (1, 16, 2, 700, 256), (4, 64, 8, 1025, 252), (38, 64, 8, 1030, 256), (20, 64, 8, 1030, 256), (3, 8, 4, 256, 128), (2, 16, 4, 500, 132)])
+def test_attention_through_registers(B_, Hq, Hkv, T, D):
+    q, k, v = make_qkv(B_, Hq, Hkv, T, D, seed=T + B_)
+    scale = float(np.float32(1.0 / math.sqrt(D)))
+    want = oracle.attention_decode(q.numpy(), k.numpy(), v.numpy(), scale)
+    got = run_gpu_attention(q, k, v, scale)
+    assert not np.isnan(got).any()
+    assert_bits_equal(got, want, f"attention {B_},{Hq},{Hkv},{T},{D}")
