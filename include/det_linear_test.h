@@ -36,6 +36,14 @@ DET_API det_status_t det_test_plan_set_variant(det_linear_plan_t* plan, int vari
 DET_API void det_test_fail_next_alloc(int nth);
 
 /*
+ * The decision of det_linear_run_host* whether kernels may touch the host buffer [host, host + bytes) themselves, from what the
+ * driver says about its first byte: memory type (CUmemorytype), managed or not, device address, start and size of the
+ * allocation or registration.  Host arithmetic only.
+ */
+DET_API int det_test_kernels_reach(unsigned memory_type, unsigned managed, uint64_t device_address, uint64_t range_start,
+                                   uint64_t range_bytes, uint64_t host, uint64_t bytes);
+
+/*
  * det_attention_decode spreads the keys of one (batch, KV head) row over a cluster of 1, 2, 4, 8 or 16 thread
  * blocks, chosen from the shape and the SM count (schedule only: every choice gives the same bits).  This
  * forces the choice for the calls that follow (capped by the number of 256-key segments of the row);

@@ -87,6 +87,9 @@ def lib() -> ctypes.CDLL:
         L.det_test_attention_schedule.restype = i32
         L.det_test_attention_set_split.argtypes = [i32]
         L.det_test_attention_set_split.restype = None
+        u32, u64 = ctypes.c_uint, ctypes.c_uint64
+        L.det_test_kernels_reach.argtypes = [u32, u32, u64, u64, u64, u64, u64]
+        L.det_test_kernels_reach.restype = i32
         L.det_test_fail_next_alloc.argtypes = [i32]
         L.det_test_fail_next_alloc.restype = None
         L.det_test_plan_set_wait.argtypes = [p, ctypes.c_uint64, i32]
@@ -386,6 +389,11 @@ def det_test_attention_schedule(B_: int, Hq: int, Hkv: int, T: int, D: int, sm_c
 def det_test_attention_set_split(blocks_per_row: int) -> None:
     """Force the cluster size of det_attention_decode (1, 2, 4, 8, 16; 0 = automatic).  Same bits for every value."""
     lib().det_test_attention_set_split(blocks_per_row)
+
+
+def det_test_kernels_reach(memory_type: int, managed: int, device_address: int, range_start: int, range_bytes: int, host: int, nbytes: int) -> bool:
+    """May kernels touch the host buffer [host, host + nbytes), given what the driver says about its first byte?  Host arithmetic only."""
+    return bool(lib().det_test_kernels_reach(memory_type, managed, device_address, range_start, range_bytes, host, nbytes))
 
 
 def det_test_fail_next_alloc(nth: int = 1) -> None:

@@ -291,12 +291,28 @@ det_status_t det_linear_run_w(const det_linear_plan_t* plan, const float* x, con
     return run_device(const_cast<det_linear_plan_t*>(plan), x, W, b, y, static_cast<cudaStream_t>(stream));
 }
 
-// The device address of pinned host memory, or nullptr (pageable memory, or the query failed).
-static void* mapped_host(const void* host)
+// May kernels read and write [host, host + bytes)?  Only if one allocation or registration of pinned memory holds all of it, under
+// the same address on the device: behind the end of a registration that stops inside the buffer a kernel would fault, where a
+// copy reports an error.
+static bool kernels_reach(unsigned memory_type, unsigned managed, uint64_t device_address, uint64_t range_start, uint64_t range_bytes,
+                          uint64_t host, uint64_t bytes)
 {
-    cudaPointerAttributes at{};
-    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+    return memory_type == CU_MEMORYTYPE_HOST && !managed && device_address == host && host >= range_start && bytes <= range_bytes &&
+           host - range_start <= range_bytes - bytes;
+}
+static bool pinned_range(const void* host, size_t bytes)
+{
+    typedef CUresult (*AttributesFn)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+    static AttributesFn attributes = driver_fn<AttributesFn>("cuPointerGetAttributes");
+    if (!attributes) return false;
+    unsigned type = 0, managed = 0;
+    CUdeviceptr device = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* out[5] = {&type, &managed, &device, &start, &size};
+    if (attributes(5, what, out, (CUdeviceptr)(uintptr_t)host) != CUDA_SUCCESS) return false;
+    return kernels_reach(type, managed, device, start, size, (uint64_t)(uintptr_t)host, bytes);
 }
 constexpr size_t kDirectHostBytes = 1u << 20;
 
@@ -329,15 +345,14 @@ static det_status_t run_host_impl(det_linear_plan_t* plan, const float* x_host, 
     // kernel instead, under which the decode kernel's weight stream already starts, and a small decode output is stored to
     // pinned memory by the kernel that computes it (M = 8, N = K = 4096: 48.4 -> 35.9 us a call).  Beyond a MiB the copy engines'
     // rate counts.
-    const void* x_dev = (xb <= kDirectHostBytes && xb % 16 == 0 && aligned16(x_host)) ? mapped_host(x_host) : nullptr;
-    e = (x_dev && aligned16(x_dev)) ? launch_copy_from_host(x_dev, plan->x_stage, xb, st)
-                                    : cudaMemcpyAsync(plan->x_stage, x_host, xb, cudaMemcpyHostToDevice, st);
+    const bool x_direct = xb <= kDirectHostBytes && xb % 16 == 0 && aligned16(x_host) && pinned_range(x_host, xb);
+    e = x_direct ? launch_copy_from_host(x_host, plan->x_stage, xb, st)
+                 : cudaMemcpyAsync(plan->x_stage, x_host, xb, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_fail("run_host: copy of x", e);
-    void* y_dev = (p.bucket == 0 && yb <= kDirectHostBytes && aligned16(y_host)) ? mapped_host(y_host) : nullptr;
-    if (y_dev && !aligned16(y_dev)) y_dev = nullptr;
-    det_status_t s = run_device(plan, plan->x_stage, W, b, y_dev ? static_cast<float*>(y_dev) : plan->y_stage, st);
+    const bool y_direct = p.bucket == 0 && yb <= kDirectHostBytes && aligned16(y_host) && pinned_range(y_host, yb);
+    det_status_t s = run_device(plan, plan->x_stage, W, b, y_direct ? y_host : plan->y_stage, st);
     if (s != DET_OK) return s;
-    if (!y_dev) {
+    if (!y_direct) {
         e = cudaMemcpyAsync(y_host, plan->y_stage, yb, cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return cuda_fail("run_host: copy of y", e);
     }
@@ -605,6 +620,12 @@ int det_test_attention_schedule(int64_t B, int64_t Hq, int64_t Hkv, int64_t T, i
     while (C < 16 && attention_block_smem_bytes(G, (int)T, (int)D, C) > 227u * 1024u) C *= 2;
     if (smem_bytes_out) *smem_bytes_out = attention_block_smem_bytes(G, (int)T, (int)D, C);
     return C;
+}
+
+int det_test_kernels_reach(unsigned memory_type, unsigned managed, uint64_t device_address, uint64_t range_start, uint64_t range_bytes,
+                           uint64_t host, uint64_t bytes)
+{
+    return kernels_reach(memory_type, managed, device_address, range_start, range_bytes, host, bytes);
 }
 
 void det_test_fail_next_alloc(int nth)

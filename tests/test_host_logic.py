@@ -81,6 +81,25 @@ def test_attention_cluster_rule(built_lib):
     assert sched(0, 32, 8, 4096, 128)[0] == 0
 
 
+HOST, DEVICE = 1, 2
+
+
+@pytest.mark.parametrize("memory_type,managed,device,start,size,host,nbytes,reach", [
+    (HOST, 0, 0x10000, 0x10000, 4096, 0x10000, 4096, True),              # a whole allocation
+    (HOST, 0, 0x10400, 0x10000, 4096, 0x10400, 0xc00, True),             # to the end of one
+    (HOST, 0, 0x10400, 0x10000, 4096, 0x10400, 0xc01, False),            # a byte beyond it
+    (HOST, 0, 0x10000, 0x10000, 4096, 0x10000, 65536, False),            # only the head of the buffer is registered
+    (HOST, 0, 0x10ff0, 0x10000, 4096, 0x10ff0, 32, False),
+    (HOST, 0, 0x50000, 0x50000, 4096, 0x10000, 64, False),               # another address on the device
+    (HOST, 1, 0x10000, 0x10000, 4096, 0x10000, 64, False),               # managed memory
+    (DEVICE, 0, 0x10000, 0x10000, 4096, 0x10000, 64, False),
+    (0, 0, 0, 0, 0, 0x10000, 64, False),                                 # pageable
+    (HOST, 0, 2**64 - 64, 2**64 - 64, 64, 2**64 - 64, 64, True),
+])
+def test_kernels_touch_only_pinned_host_memory_that_holds_the_whole_buffer(built_lib, memory_type, managed, device, start, size, host, nbytes, reach):
+    assert built_lib.det_test_kernels_reach(memory_type, managed, device, start, size, host, nbytes) is reach
+
+
 def test_bad_shapes_are_rejected_with_a_message(built_lib):
     B = built_lib
     for shp in [(0, 1, 1), (1, 0, 1), (1, 1, 0), (-3, 4, 8), (1, 1 << 31, 8), (1 << 21, 1 << 21, 8)]:
