@@ -197,9 +197,10 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
-    // Set-up without a block-wide stop: the producer of group g initialises that group's barriers and goes
-    // straight on to request weight tiles; producer warps only ARRIVE at named barrier 2, the consumers wait
-    // on it (so they see initialised barriers), nobody waits for the consumers.
+    // Set-up without a block-wide stop: the weight producer of group g initialises that group's barriers and goes
+    // straight on to request weight tiles; it only ARRIVES at named barrier 2.  Consumers and activation producers wait on it:
+    // they use barriers that another warp initialises (a copy that completes on a barrier before it is initialised is an error, and
+    // lost), and the activation producers have the previous kernel to wait for anyway.
     if (warp >= C::kConsumerWarps) {
         const int pg = warp - C::kConsumerWarps;
         if (pg < SK && lane == 0) {
@@ -208,7 +209,7 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                 mbar_init(full0 + 8 * (pg * STAGES + i), 1);
                 mbar_init(empty0 + 8 * (pg * STAGES + i), C::kGroupWarps);
             }
-            if (pg == 0) sts_volatile_i32(abort_flag, 0);
+            sts_volatile_i32(abort_flag, 0);                  // (by every weight producer: each may read it before the others get here)
             // make the initialised barriers visible to the bulk-copy engine
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             if (!C::kSplitProducers) asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
@@ -216,7 +217,8 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
             asm volatile("prefetch.tensormap [%0];" ::"l"(&map_x) : "memory");
         }
         __syncwarp();
-        asm volatile("bar.arrive 2, %0;" ::"r"(C::kThreads) : "memory");
+        if (C::kSplitProducers && pg >= SK && pg < 2 * SK) asm volatile("bar.sync 2, %0;" ::"r"(C::kThreads) : "memory");
+        else asm volatile("bar.arrive 2, %0;" ::"r"(C::kThreads) : "memory");
     } else {
         asm volatile("bar.sync 2, %0;" ::"r"(C::kThreads) : "memory");
     }
