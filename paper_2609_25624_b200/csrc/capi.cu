@@ -314,7 +314,41 @@ static bool pinned_range(const void* host, size_t bytes)
     if (attributes(5, what, out, (CUdeviceptr)(uintptr_t)host) != CUDA_SUCCESS) return false;
     return kernels_reach(type, managed, device, start, size, (uint64_t)(uintptr_t)host, bytes);
 }
-constexpr size_t kDirectHostBytes = 1u << 20;
+
+// How x and y cross the bus where kernels reach them: by a copy engine, which takes some 8 us to begin and end a copy of any size;
+// by a kernel that copies in whole lines (for x, the decode kernel's weight stream already starts under it); y also straight from the
+// kernel that computes it, which costs no extra launch but writes short pieces of rows and holds its SMs until the bus has taken
+// them.  From 226 shapes, 1 .. 512 rows, x and y 4 KB .. 1 MiB each, all combinations of routes.
+enum class Across { kCopy, kKernel, kDirect };
+struct HostRoute { bool x_by_kernel; Across y; };
+static HostRoute host_route(int64_t M, int64_t N, int64_t K, bool sync)
+{
+    constexpr int64_t KiB = 1024;
+    const int64_t xb = 4 * M * K, yb = 4 * M * N;
+    HostRoute route{false, Across::kCopy};
+    if (M > 64) {
+        // the prefill kernel waits for x in any case (x of 128 KB 0.83 of two copies' time, 512 KB 1.03; several streams 0.99, 1.07)
+        route.x_by_kernel = sync && xb <= 256 * KiB;
+        return route;
+    }
+    if (sync) {
+        // One call's latency.  y straight from the kernel up to 192 KB (M = 8, N = K = 4096 34.9 us, by a copying kernel 35.5; at M = 30,
+        // N = 4369, K = 512, 512 KB, 61 and 42), and beyond where the weight stream is long enough to hide the stores of
+        // earlier tiles (M = 8, N = 28672, K = 4096, 896 KB 73.5, by a copying kernel 87.5, by copies 95).
+        // All in all 0.87 of two copies' time, nowhere above 1.08.
+        constexpr int64_t most = 1024 * KiB + 4 * KiB;
+        route.x_by_kernel = xb <= most;
+        if (yb <= 192 * KiB || (yb <= most && K >= 256 * M && N >= 8192)) route.y = Across::kDirect;
+        else if (yb <= most) route.y = Across::kKernel;
+    } else if (xb <= 256 * KiB && yb <= 256 * KiB) {
+        // Calls of several streams overlap: the copy engines work beside the kernels, while SMs that wait for the bus are lost to the
+        // other streams.  Small calls gain all the same (three streams, M = 8, N = 1024, K = 1024 6.4 us a call, by copies 8.8); M =
+        // 64, N = 4096, K = 512 takes 25 by copies, 117 with direct stores.  0.89 of two copies' time, nowhere above 1.08.
+        route.x_by_kernel = true;
+        route.y = yb <= (M <= 4 ? 128 : 64) * KiB ? Across::kDirect : Across::kKernel;
+    }
+    return route;
+}
 
 static det_status_t run_host_impl(det_linear_plan_t* plan, const float* x_host, const void* W, const float* b,
                                   float* y_host, void* stream, bool sync)
@@ -341,19 +375,18 @@ static det_status_t run_host_impl(det_linear_plan_t* plan, const float* x_host, 
         }
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // A copy engine takes some 8 us to begin and end a copy of any size.  Small activations in pinned memory come over by a
-    // kernel instead, under which the decode kernel's weight stream already starts, and a small decode output is stored to
-    // pinned memory by the kernel that computes it (M = 8, N = K = 4096: 48.4 -> 35.9 us a call).  Beyond a MiB the copy engines'
-    // rate counts.
-    const bool x_direct = xb <= kDirectHostBytes && xb % 16 == 0 && aligned16(x_host) && pinned_range(x_host, xb);
-    e = x_direct ? launch_copy_from_host(x_host, plan->x_stage, xb, st)
-                 : cudaMemcpyAsync(plan->x_stage, x_host, xb, cudaMemcpyHostToDevice, st);
+    HostRoute route = host_route(p.M, p.N, p.K, sync);
+    if (route.x_by_kernel) route.x_by_kernel = xb % 16 == 0 && aligned16(x_host) && pinned_range(x_host, xb);
+    if (route.y != Across::kCopy && !((route.y == Across::kDirect || yb % 16 == 0) && aligned16(y_host) && pinned_range(y_host, yb)))
+        route.y = Across::kCopy;
+    e = route.x_by_kernel ? launch_copy_across_bus(x_host, plan->x_stage, xb, st)
+                          : cudaMemcpyAsync(plan->x_stage, x_host, xb, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_fail("run_host: copy of x", e);
-    const bool y_direct = p.bucket == 0 && yb <= kDirectHostBytes && aligned16(y_host) && pinned_range(y_host, yb);
-    det_status_t s = run_device(plan, plan->x_stage, W, b, y_direct ? y_host : plan->y_stage, st);
+    det_status_t s = run_device(plan, plan->x_stage, W, b, route.y == Across::kDirect ? y_host : plan->y_stage, st);
     if (s != DET_OK) return s;
-    if (!y_direct) {
-        e = cudaMemcpyAsync(y_host, plan->y_stage, yb, cudaMemcpyDeviceToHost, st);
+    if (route.y != Across::kDirect) {
+        e = route.y == Across::kKernel ? launch_copy_across_bus(plan->y_stage, y_host, yb, st)
+                                       : cudaMemcpyAsync(y_host, plan->y_stage, yb, cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return cuda_fail("run_host: copy of y", e);
     }
     if (sync) {

@@ -91,8 +91,8 @@ cudaError_t launch_attention_decode(const float* q, const float* k, const float*
                                     int D, float* o, cudaStream_t stream);
 // Read `bytes` at buf through L2 (evicts what was there without leaving dirty lines); sink: 4 bytes of device memory.
 cudaError_t launch_l2_evict(const void* buf, size_t bytes, unsigned* sink, int sm_count, cudaStream_t stream);
-// bytes (a multiple of 16) from mapped host memory to device memory, both 16-byte aligned
-cudaError_t launch_copy_from_host(const void* src, void* dst, size_t bytes, cudaStream_t stream);
+// bytes (a multiple of 16) between pinned host memory and device memory, both 16-byte aligned
+cudaError_t launch_copy_across_bus(const void* src, void* dst, size_t bytes, cudaStream_t stream);
 cudaError_t launch_argmax(const float* y, int64_t M, int64_t N, int32_t* idx, cudaStream_t stream);
 
 // Decode-kernel tiling chosen for a shape (numerically inert); used by the host to build the

@@ -1,5 +1,5 @@
 // The dispatch for shapes and buffers that TMA cannot read (K % 8 != 0 or FP32 weights with K % 4 != 0, misaligned buffers),
-// the split-K second pass, the copy of small activations from the host and the row argmax.
+// the split-K second pass, the copy of small activations and results across the bus and the row argmax.
 #include "internal.h"
 #include "device_utils.cuh"
 #include <cooperative_groups.h>
@@ -50,17 +50,17 @@ cudaError_t launch_combine(const LaunchArgs& a)
     return cudaLaunchKernelEx(&cfg, combine_kernel, (const float*)a.partials, a.b, a.y, MN, a.N, a.S, a.ldy);
 }
 
-// Small activations from (mapped) pinned host memory to device memory: 16-byte loads across the bus, all of them on their way at
-// once, and the kernel after this one may start its prologue and its weight stream meanwhile.  Not before this kernel's own
+// Activations from pinned host memory to device memory, or results the other way: whole lines across the bus, all of them on their
+// way at once, and the kernel after this one may start its prologue and its weight stream meanwhile.  Not before this kernel's own
 // wait: W and b may have been written by the kernel before it.
-__global__ void __launch_bounds__(256) copy_from_host_kernel(const float4* __restrict__ src, float4* __restrict__ dst, unsigned n)
+__global__ void __launch_bounds__(256) copy_across_bus_kernel(const float4* __restrict__ src, float4* __restrict__ dst, unsigned n)
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) dst[i] = __ldcv(src + i);
 }
 
-cudaError_t launch_copy_from_host(const void* src, void* dst, size_t bytes, cudaStream_t stream)
+cudaError_t launch_copy_across_bus(const void* src, void* dst, size_t bytes, cudaStream_t stream)
 {
     const unsigned n = (unsigned)(bytes / 16), blocks = (n + 255) / 256;
     cudaLaunchConfig_t cfg{};
@@ -72,7 +72,7 @@ cudaError_t launch_copy_from_host(const void* src, void* dst, size_t bytes, cuda
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, copy_from_host_kernel, static_cast<const float4*>(src), static_cast<float4*>(dst), n);
+    return cudaLaunchKernelEx(&cfg, copy_across_bus_kernel, static_cast<const float4*>(src), static_cast<float4*>(dst), n);
 }
 
 // Row argmax, lowest index on ties (the paper's stated tie rule for greedy decoding).  Ordering

@@ -330,3 +330,25 @@ def test_run_host_by_kernel_and_by_copy(M, N, K, where):
         torch.cuda.current_stream().synchronize()
         assert_bits_equal(yh.numpy(), want, where + ", asynchronous")
     plan.close()
+
+
+# results of 200 to 1100 KB: stored by the kernel that computes them, by a copying kernel, by the copy engines; the routes of
+# calls that wait and of calls that do not differ
+@pytest.mark.parametrize("M,N,K", [(8, 6145, 264), (3, 17000, 1024), (8, 8192, 2048), (16, 3200, 40), (30, 2184, 520), (64, 1021, 264), (63, 3601, 136), (64, 4196, 264),
+                                   (2, 70000, 512), (4, 1024, 16392)])
+def test_run_host_with_large_decode_results(M, N, K):
+    x, W, b = inputs.make_case(M, N, K)
+    want = oracle_y(x, W, b)
+    xh, yh = x.pin_memory(), torch.empty(M, N).pin_memory()
+    plan = B.det_linear_plan(M, N, K)
+    Wd, bd = W.cuda(), b.cuda()
+    for rep in range(2):
+        yh.fill_(float("nan"))
+        B.det_linear_run_host(plan, xh, Wd, bd, yh)
+        assert_bits_equal(yh.numpy(), want, f"call {rep}")
+    for rep in range(2):
+        yh.fill_(float("nan"))
+        B.det_linear_run_host_async(plan, xh, Wd, bd, yh)
+        torch.cuda.current_stream().synchronize()
+        assert_bits_equal(yh.numpy(), want, f"asynchronous call {rep}")
+    plan.close()
