@@ -91,6 +91,7 @@ DET_API det_status_t det_linear_plan_params(int64_t M, int64_t N, int64_t K, det
  * status word and, in the prefill bucket when S > 1, the split-K partials workspace (device); the
  * decode bucket folds its segments inside the kernel and needs none.  Returns NULL on failure
  * (det_last_error(), det_last_status()).
+ * (The partials are kept by whole tiles where that takes up to 16 MiB, or up to twice workspace_bytes.)
  * A prefill plan also asks for the schedule workspace of its TMA-fed kernel (a few KB of flags and, where there are more
  * work units than SMs, 128 KiB per SM of accumulators that blocks hand over; not in workspace_bytes).  If that
  * allocation fails the plan is still created and runs the register-staged kernel, which computes the same bits.

@@ -91,6 +91,7 @@ det_status_t run_device(det_linear_plan_t* plan, const float* x, const void* W, 
     a.x = x; a.W = W; a.b = b; a.y = y;
     a.wfmt = p.weight_format;
     a.partials = plan->partials;
+    a.partial_floats = plan->partial_floats;
     // Prefill with several segments: the warps that complete a tile fold it.  Test flag 2 forces the second pass.  Same
     // bits either way.
     a.tile_counters = (plan->test_flags & 2) ? nullptr : plan->tile_counters;
@@ -242,6 +243,7 @@ det_linear_plan_t* det_linear_plan_shard(int64_t M, int64_t N, int64_t K, int64_
     if (e == cudaSuccess && prm.workspace_bytes) {
         e = device_alloc(reinterpret_cast<void**>(&plan->partials), counters_at + 4 * n_counters);
         if (e == cudaSuccess) {
+            plan->partial_floats = pw.partial_floats;
             plan->tile_counters = reinterpret_cast<unsigned*>(reinterpret_cast<char*>(plan->partials) + counters_at);
             plan->n_tile_counters = n_counters;
             e = cudaMemset(plan->tile_counters, 0, 4 * n_counters);

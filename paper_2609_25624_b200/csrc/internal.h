@@ -42,6 +42,7 @@ struct LaunchArgs {
     float* y;             // final output [M,N], row pitch ldy
     int64_t ldy;          // floats between consecutive rows of y (N unless the plan is a column shard)
     float* partials;      // [S,M,N] when S > 1, else nullptr
+    uint64_t partial_floats;   // what it holds: with room for whole tiles, and counters, the prefill kernel folds in place
     unsigned* tile_counters;   // prefill with S > 1: zeroed counters per output tile and warp (the TMA-fed kernel folds in place), or nullptr
     unsigned* sync;       // TMA-fed prefill kernel: zeroed ticket and hand-over flags
     float* handoff;       // prefill in equal stretches: accumulators on their way from one block to the next, or nullptr
@@ -115,7 +116,8 @@ struct det_linear_plan {
     det_linear_params_t prm;
     int device;
     int sm_count;
-    float* partials;                 // device, S*M*n_count floats or nullptr
+    float* partials;                 // device, S*M*n_count floats and more (prefill_workspace), or nullptr
+    uint64_t partial_floats;
     unsigned* tile_counters;         // device, inside the partials allocation (prefill, S > 1) or nullptr
     uint64_t n_tile_counters;
     unsigned* sync;                  // device, prefill: ticket and hand-over flags of the TMA-fed kernel, or nullptr

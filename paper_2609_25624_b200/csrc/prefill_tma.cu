@@ -47,7 +47,11 @@ PrefillWorkspace prefill_workspace(int64_t M, int64_t N, int64_t K, int S, int64
     if (S > 1) {
         // any tile height and width (tests force them): tiles of at least 80 x 32, eight warps each
         w.counter_words = ((uint64_t)M + 79) / 80 * (((uint64_t)N + 31) / 32) * 8;
-        w.partial_floats = (uint64_t)S * ((uint64_t)M + 127) * (((uint64_t)N + 255) / 256 * 256);
+        // Segment sums by whole tiles, for the fold in place, where that is a matter of 16 MiB for any tile or of twice the sums
+        // themselves for this one; layers of a few columns would pay many times over (64 000 x 1 x 2000: 131 MB for 0.5) and take a second pass.
+        const uint64_t sums = (uint64_t)S * (uint64_t)M * (uint64_t)N, own = units * bm * (uint64_t)width;
+        const uint64_t any = (uint64_t)S * ((uint64_t)M + 127) * (((uint64_t)N + 255) / 256 * 256);
+        w.partial_floats = any <= (4u << 20) ? any : own <= 2 * sums ? own : sums;
     }
     return w;
 }

@@ -30,7 +30,8 @@ cudaError_t launch_t(const LaunchArgs& la, const CUtensorMap* map_w, const CUten
     Args a{};
     a.x = la.x; a.w = la.W;
     a.bias = la.b; a.y = la.y; a.partials = la.partials; a.handoff = la.handoff; a.sync = la.sync;
-    a.tile_counters = la.tile_counters; a.status = la.status;
+    a.tile_counters = (uint64_t)units * T::BM * T::BN <= la.partial_floats ? la.tile_counters : nullptr;
+    a.status = la.status;
     a.ldy = la.ldy;
     a.M = (int)la.M; a.N = (int)la.N; a.K = (int)la.K;
     a.seg_slabs = (int)(la.seg_len / BK);
@@ -60,7 +61,7 @@ cudaError_t launch_t(const LaunchArgs& la, const CUtensorMap* map_w, const CUten
     const CUtensorMap none{};
     e = cudaLaunchKernelEx(&cfg, kern, PLAIN ? none : *map_x, PLAIN ? none : *map_w, a);
     if (e != cudaSuccess) return e;
-    if (la.S > 1 && !la.tile_counters) return launch_combine(la);
+    if (la.S > 1 && !a.tile_counters) return launch_combine(la);
     return cudaSuccess;
 }
 

@@ -98,3 +98,25 @@ def test_plain_loads_special_values_at_a_ragged_end():
     assert np.array_equal(np.isnan(got), np.isnan(want))
     assert np.signbit(want[::2, :20]).all() and not want[::2, :20].any()
     assert_bits_equal(np.nan_to_num(got, nan=0.0, posinf=1.0, neginf=2.0), np.nan_to_num(want, nan=0.0, posinf=1.0, neginf=2.0), "special values")
+
+
+# a few columns, split in K: the plan's memory stays near that of the segment sums (a second pass folds them), and the sums of whole
+# tiles are kept where they take little more
+@pytest.mark.parametrize("M,N,K,most_mb", [(64000, 1, 2000, 16), (20000, 3, 2001, 16), (30000, 33, 1500, 32), (3000, 130, 2048, 24)])
+def test_partials_of_narrow_layers(M, N, K, most_mb):
+    x, W, b = inputs.make_case(M, N, K)
+    want = oracle_y(x, W, b)
+    xd, Wd, bd, y = x.cuda(), W.cuda(), b.cuda(), torch.full((M, N), float("nan"), device="cuda")
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    plan = B.det_linear_plan(M, N, K)
+    took = free - torch.cuda.mem_get_info()[0]
+    params = B.det_linear_plan_get_params(plan)
+    assert params.S > 1 and params.workspace_bytes <= took + (2 << 20)
+    assert took <= (most_mb + 24) << 20              # (19 MB are accumulators that blocks hand over)
+    for rep in range(2):
+        y.fill_(float("nan"))
+        B.det_linear_run(plan, xd, Wd, bd, y)
+        B.det_linear_plan_check(plan)
+        assert_bits_equal(y.cpu().numpy(), want, f"run {rep}")
+    plan.close()
