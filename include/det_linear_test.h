@@ -58,9 +58,9 @@ DET_API int det_test_attention_schedule(int64_t B, int64_t Hq, int64_t Hkv, int6
 
 /*
  * Bound of one device-side wait for the kernels launched through this plan (default 2 s), and flags:
- * bit 0 (value 1) is a deliberate stall: thread block 0 of the decode kernel (of the TMA-fed prefill
- * kernel likewise) never requests the activations of its first stage, so the wait for that stage runs
- * into the bound.  The
+ * bit 0 (value 1) is a deliberate stall: thread block 0 of the decode kernel (the first block of the prefill
+ * kernel likewise) never requests the activations of its first stage -- with plain loads, never announces its first slab --, so
+ * the wait for that stage runs into the bound, and where another block carries one of its units on, that block's wait too.  The
  * kernel then records the timeout in the plan's status word, drains and returns (no trap, no endless
  * loop; the other blocks finish normally), and det_linear_plan_check reports DET_ERR_DEVICE_TIMEOUT.
  * The output of such a run is undefined.  Bit 1 (value 2) makes a prefill plan with several K segments fold them

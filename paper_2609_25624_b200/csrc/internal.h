@@ -20,7 +20,7 @@ enum KernelId : int { kKernelGeneric = 0, kKernelDecode = 1, kKernelPrefill = 2 
 // Device-side status word written by kernels that give up a bounded wait.
 struct DeviceStatus {
     unsigned int timeout_flag;   // nonzero: some wait expired
-    unsigned int where;          // which wait (diagnostic)
+    unsigned int where;          // which wait (diagnostic); of several, the highest number
 };
 
 // LaunchArgs::test_flags beyond the test hooks: the decode kernel also waits for the previous kernel in the stream before it

@@ -95,7 +95,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
         if (lds_volatile_i32(abort_flag)) return false;
         if (global_timer_ns() - t0 > limit_ns) {
             sts_volatile_i32(abort_flag, 1);
-            atomicExch(&status->where, site);
+            atomicMax(&status->where, site);
             atomicExch(&status->timeout_flag, 1u);
             return false;
         }

@@ -212,6 +212,7 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
     __syncthreads();
     const int blk = shared_ticket;
+
     Walk w;
     if (a.cut) {
         w.lo = a.total * blk / (int)gridDim.x;
@@ -225,6 +226,7 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     w.u_last = unit_at(a, w.hi - 1);
     const int n_it = (int)(w.hi - w.lo);             // slabs of this block
     const int n_pieces = w.count();
+
     if (warp >= kMulWarps) {
         // ---------------- preparing warps ----------------
         if constexpr (T::kWide) reg_dec<T::kPrepRegs>();
@@ -369,7 +371,8 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                     if constexpr (NB & 1) r[0] = r[1];
                 }
                 __syncwarp();
-                if (lane == 0) mbar_arrive(full0 + 8 * st);
+                // (test hook: the first block's first slab is never announced, so the multiplying warps' wait for it expires)
+                if (lane == 0 && !((a.test_flags & 1) && blk == 0 && it == 0)) mbar_arrive(full0 + 8 * st);
                 if (++st == ST) { st = 0; phase ^= 1u; }
             }
             return;
@@ -385,8 +388,8 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             c.m0 = (p.tile % a.tiles_m) * BM;
             c.n0 = (p.tile / a.tiles_m) * BN;
         };
-        // (test hook: block 0 never requests its first activation tile, so its first wait expires)
-        const bool withhold = (a.test_flags & 1) && blockIdx.x == 0;
+        // (test hook: the first block never requests its first activation tile, so its first wait expires)
+        const bool withhold = (a.test_flags & 1) && blk == 0;
         auto request = [&](int it, int slot) {       // one thread: the raw stage at the cursor, which moves on
             const uint32_t bar = rawfull0 + 8 * slot, dst = raw0 + (uint32_t)slot * T::kRawBytes;
             mbar_arrive_expect_tx(bar, T::kRawBytes);
@@ -643,7 +646,7 @@ prefill_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
                     if (lds_volatile_i32(abort_flag)) break;
                     if (global_timer_ns() - t0 > a.wait_limit_ns) {
                         sts_volatile_i32(abort_flag, 1);
-                        atomicExch(&a.status->where, 5u);
+                        atomicMax(&a.status->where, 5u);
                         atomicExch(&a.status->timeout_flag, 1u);
                         break;
                     }

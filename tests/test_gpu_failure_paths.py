@@ -153,3 +153,31 @@ def test_prefill_without_its_activation_workspace(M, N, K, nth):
     plan = B.det_linear_plan(M, N, K)
     assert B.det_linear_plan_describe(plan)["prefill_tile"]["feed"] == "tma"
     plan.close()
+
+
+@pytest.mark.parametrize("M,N,K,wfmt,plain", [(400, 8200, 264, "bf16", False), (300, 3000, 1000, "fp32", False), (520, 2570, 1030, "bf16", True), (400, 8200, 262, "fp16", True)])
+def test_bounded_wait_expires_in_a_hand_over_between_blocks(M, N, K, wfmt, plain):
+    """More units than SMs: the block that carries on the first one's unit waits for it in vain, gives up after the limit as the first one
+    does, and the plan works again afterwards (ticket, hand-over flags and tile counts are back at zero)."""
+    x, W, b = inputs.make_case_w(M, N, K, wfmt)
+    want = oracle_y(x, W, b)
+    xd, Wd, bd = x.cuda(), W.cuda(), b.cuda()
+    y = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+    plan = B.det_linear_plan_w(M, N, K, wfmt)
+    assert (B.det_linear_plan_get_params(plan).kernel == 0) == plain
+    B.det_test_plan_set_wait(plan, 5_000_000, withhold_first_copy=True)     # 5 ms per wait
+    t0 = time.perf_counter()
+    B.det_linear_run(plan, xd, Wd, bd, y)
+    with pytest.raises(B.DetLinearError) as ei:
+        B.det_linear_plan_check(plan)
+    elapsed = time.perf_counter() - t0
+    assert ei.value.status == DET_ERR_DEVICE_TIMEOUT
+    assert "site 5" in B.det_last_error()                        # the highest of the sites that expired is on record
+    assert elapsed < 5.0, f"the stalled kernel took {elapsed:.2f} s to give up"
+    B.det_test_plan_set_wait(plan, 2_000_000_000, withhold_first_copy=False)
+    for rep in range(2):
+        y.fill_(float("nan"))
+        B.det_linear_run(plan, xd, Wd, bd, y)
+        B.det_linear_plan_check(plan)
+        assert_bits_equal(y.cpu().numpy(), want, f"after the expired wait, run {rep}")
+    plan.close()
