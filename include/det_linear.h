@@ -284,11 +284,18 @@ DET_API det_status_t det_attention_decode(const float* q, const float* k, const 
  * make that first call before starting any stream capture.  The address is kept for the life of the
  * process: after a cudaDeviceReset the library must be reloaded before this entry point is used again.  The kernels are
  * those of det_linear_run (the prefill bucket without cutting work units across thread blocks, which needs a
- * workspace); W and b may be written by the kernel before this call in the stream.  There is no plan to ask about an
- * expired wait.  Enqueues on `stream`, no synchronisation.
+ * workspace); W and b may be written by the kernel before this call in the stream.  Whether a kernel gave up a bounded wait,
+ * and left its output undefined, is asked with det_linear_noalloc_check.  Enqueues on `stream`, no synchronisation.
  */
 DET_API det_status_t det_linear_run_noalloc(int64_t M, int64_t N, int64_t K, const float* x, const uint16_t* W,
                                             const float* b, float* y, void* stream);
+
+/*
+ * Synchronise `stream` and report whether any kernel that det_linear_run_noalloc launched on the current device, in any stream,
+ * has given up a bounded wait since the last such call (det_linear_plan_check for callers without a plan).  DET_OK,
+ * DET_ERR_DEVICE_TIMEOUT or DET_ERR_CUDA.  The record is cleared by the call.  No allocation.
+ */
+DET_API det_status_t det_linear_noalloc_check(void* stream);
 
 /* Message of the last error on the calling thread ("" if none).  Never NULL. */
 DET_API const char* det_last_error(void);

@@ -69,6 +69,9 @@ DET_API int det_test_attention_schedule(int64_t B, int64_t Hq, int64_t Hkv, int6
  */
 DET_API det_status_t det_test_plan_set_wait(det_linear_plan_t* plan, uint64_t wait_limit_ns, int flags);
 
+/* The same bound and flag (0 or 1) for det_linear_run_noalloc, process-wide. */
+DET_API det_status_t det_test_noalloc_set_wait(uint64_t wait_limit_ns, int flags);
+
 /*
  * Create a CUDA green context holding (at least) `sm_count` SMs of the current device and a
  * stream on it.  *stream_out receives a cudaStream_t usable with det_linear_run; *handle_out an

@@ -106,6 +106,10 @@ def lib() -> ctypes.CDLL:
         L.det_test_green_stream_destroy.restype = None
         L.det_linear_run_noalloc.argtypes = [i64, i64, i64, p, p, p, p, p]
         L.det_linear_run_noalloc.restype = i32
+        L.det_linear_noalloc_check.argtypes = [p]
+        L.det_linear_noalloc_check.restype = i32
+        L.det_test_noalloc_set_wait.argtypes = [u64, i32]
+        L.det_test_noalloc_set_wait.restype = i32
         L.det_test_linear_atomic_splitk.argtypes = [i64, i64, i64, ctypes.c_int32, p, p, p, p, p]
         L.det_test_linear_atomic_splitk.restype = i32
         L.det_test_scale_cols.argtypes = [p, i64, p, i64, i64, ctypes.c_float, p]
@@ -319,6 +323,11 @@ def det_linear_run_noalloc(x, W, b, y, stream=None) -> None:
                                         y.data_ptr(), _stream_ptr(stream)))
 
 
+def det_linear_noalloc_check(stream=None) -> None:
+    """Synchronise the stream; raises DetLinearError if a kernel of det_linear_run_noalloc gave up a bounded wait since the last call."""
+    _check(lib().det_linear_noalloc_check(_stream_ptr(stream)))
+
+
 def det_linear_plan_tune(plan: Plan, x, W, b, y, stream=None):
     """Time the plan's candidate tilings on these buffers and pin the fastest (schedule only: every
     candidate gives the same bits).  Returns (variant, microseconds); (0, -1.0) when there is nothing
@@ -406,6 +415,11 @@ def det_test_plan_set_wait(plan: Plan, wait_limit_ns: int, withhold_first_copy: 
     prefill plan fold its K segments with the second launch instead of inside the kernel (same bits)."""
     flags = (1 if withhold_first_copy else 0) | (2 if two_pass_combine else 0)
     _check(lib().det_test_plan_set_wait(plan.handle, int(wait_limit_ns), flags))
+
+
+def det_test_noalloc_set_wait(wait_limit_ns: int = 2_000_000_000, withhold_first_copy: bool = False) -> None:
+    """The bound of one device-side wait and the deliberate stall for det_linear_run_noalloc, process-wide."""
+    _check(lib().det_test_noalloc_set_wait(int(wait_limit_ns), int(withhold_first_copy)))
 
 
 def det_test_green_stream_create(sm_count: int):

@@ -11,6 +11,7 @@
 // order, same bits, same kernels) as det_linear_plan + det_linear_run.  With the generic kernels that it used before,
 // M = 3, N = K = 4096 took 44.8 us a call.
 #include "internal.h"
+#include "det_linear_test.h"
 #include <mutex>
 
 namespace detlin {
@@ -48,6 +49,10 @@ static cudaError_t static_addresses(int dev, NoallocAddresses* out)
     *out = g_addr[dev];
     return cudaSuccess;
 }
+
+// Bound of one device-side wait and test flag (det_test_noalloc_set_wait; never set outside the tests).
+static unsigned long long g_wait_limit_ns = kDefaultWaitLimitNs;
+static int g_test_flags = 0;
 
 // The decode tiling depends on the shape and the device only; a loop that repeats a shape does not search again.
 static thread_local struct {
@@ -102,8 +107,8 @@ extern "C" det_status_t det_linear_run_noalloc(int64_t M, int64_t N, int64_t K, 
     plan.n_count = N;
     plan.ldy = N;
     plan.forced_kernel = -1;
-    plan.wait_limit_ns = kDefaultWaitLimitNs;
-    plan.test_flags = kFlagLateWeights;                     // nothing was said here about W and b being older than the stream's last kernel
+    plan.wait_limit_ns = g_wait_limit_ns;
+    plan.test_flags = kFlagLateWeights | g_test_flags;                     // nothing was said here about W and b being older than the stream's last kernel
     plan.decode_cfg_variant = -1;
     plan.map_cfg_id = -1;
     auto& t = g_last_tiling;
@@ -118,4 +123,31 @@ extern "C" det_status_t det_linear_run_noalloc(int64_t M, int64_t N, int64_t K, 
         t.cfg = plan.decode_cfg;
     }
     return st;
+}
+
+extern "C" det_status_t det_linear_noalloc_check(void* stream)
+{
+    int dev = 0;
+    NoallocAddresses at{};
+    DeviceStatus h{};
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = static_addresses(dev, &at);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, at.words, sizeof h, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(at.words, 0, sizeof h, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) { set_error("noalloc_check: %s", cudaGetErrorString(e)); return DET_ERR_CUDA; }
+    if (h.timeout_flag) {
+        set_error("noalloc_check: a kernel gave up a bounded wait (site %u)", h.where);
+        return DET_ERR_DEVICE_TIMEOUT;
+    }
+    return DET_OK;
+}
+
+extern "C" det_status_t det_test_noalloc_set_wait(uint64_t wait_limit_ns, int flags)
+{
+    if (wait_limit_ns == 0 || flags < 0 || flags > 1) { set_error("noalloc_set_wait: bad argument"); return DET_ERR_INVALID_ARG; }
+    g_wait_limit_ns = wait_limit_ns;
+    g_test_flags = flags;
+    return DET_OK;
 }

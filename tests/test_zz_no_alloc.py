@@ -86,3 +86,28 @@ def test_noalloc_fast_kernels_with_weights_written_just_before(M, N, K):
     B.det_linear_run_noalloc(xd, W2, b2, y)
     torch.cuda.synchronize()
     assert_bits_equal(y.cpu().numpy(), want, f"{M},{N},{K}")
+
+
+@pytest.mark.parametrize("M,N,K", [(8, 4096, 1024), (1, 300, 264), (130, 200, 1024), (130, 200, 1021)])
+def test_noalloc_check_reports_an_expired_wait(M, N, K):
+    """The kernels bound their waits; callers without a plan ask about an expired one, and the next calls are right again."""
+    x, W, b = inputs.make_case(M, N, K)
+    want = oracle_y(x, W, b)
+    xd, Wd, bd = x.cuda(), W.cuda(), b.cuda()
+    y = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+    B.det_linear_run_noalloc(xd, Wd, bd, y)
+    B.det_linear_noalloc_check()
+    assert_bits_equal(y.cpu().numpy(), want, "before")
+    B.det_test_noalloc_set_wait(5_000_000, withhold_first_copy=True)        # 5 ms per wait
+    try:
+        B.det_linear_run_noalloc(xd, Wd, bd, y)
+        with pytest.raises(B.DetLinearError) as ei:
+            B.det_linear_noalloc_check()
+    finally:
+        B.det_test_noalloc_set_wait()
+    assert ei.value.status == 6 and "site" in B.det_last_error()
+    for call in range(2):
+        y.fill_(float("nan"))
+        B.det_linear_run_noalloc(xd, Wd, bd, y)
+        B.det_linear_noalloc_check()                 # the record was cleared
+        assert_bits_equal(y.cpu().numpy(), want, f"after the expired wait, call {call}")
