@@ -134,7 +134,7 @@ def test_bounded_wait_expires_in_the_prefill_kernel():
 
 @pytest.mark.parametrize("M,N,K,nth", [(128, 256, 4096, 3), (96, 136, 256, 2)])
 def test_prefill_without_its_activation_workspace(M, N, K, nth):
-    """The transposed-activation workspace is optional: when its allocation fails the plan is still created,
+    """The schedule workspace is optional: when its allocation fails the plan is still created,
     runs the register-staged kernel and produces the same bits."""
     x, W, b = inputs.make_case(M, N, K)
     want = oracle_y(x, W, b)

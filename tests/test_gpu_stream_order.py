@@ -111,3 +111,12 @@ def test_weights_written_before_a_run_on_host_activations():
     plan = B.det_linear_plan_w(2, 64, 256, "fp32")
     _check(_writer(64, 256, 16384), W, lambda: None, lambda: B.det_linear_run_host(plan, x, W, None, y), y)
     plan.close()
+
+
+# the bias by a long run that lets its successors start early, straight before: decode kernels with one and two segment groups and one
+# producer for both operands, decode for any K, prefill by TMA and by plain loads
+@pytest.mark.parametrize("M,N,K", [(3, 256, 512), (16, 300, 512), (1, 20000, 264), (3, 256, 511), (65, 256, 512), (65, 256, 63)])
+def test_bias_written_before_a_run_without_a_plan(M, N, K):
+    x, W, y = _normal(21, M, K), _normal(22, N, K).to(torch.bfloat16), torch.empty(M, N, device="cuda")
+    b = torch.empty(1, N, device="cuda")
+    _check(_writer(1, N, 65536 if N < 1000 else 4096), b, lambda: None, lambda: B.det_linear_run_noalloc(x, W, b[0], y), y)

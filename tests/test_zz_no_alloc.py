@@ -73,7 +73,8 @@ def test_noalloc_rejects_shapes_beyond_the_builtin_scratch():
 @pytest.mark.parametrize("M,N,K", [(64, 520, 1024), (1, 20000, 264), (65, 300, 40), (100, 1000, 1000), (3000, 9000, 256)])
 def test_noalloc_fast_kernels_with_weights_written_just_before(M, N, K):
     """The kernels of the planned path, on aligned buffers: decode with and without a split, prefill with one unit per
-    thread block (more units than SMs too) and a second pass.  The weights are written by the stream's previous kernel."""
+    thread block (more units than SMs too) and a second pass.  The weights are written by copies in the same stream just before (by a
+    kernel that lets its successors start early: tests/test_gpu_stream_order.py)."""
     x, W, b = inputs.make_case(M, N, K)
     xd, Wd, bd = x.cuda(), W.cuda(), b.cuda()
     assert B.det_linear_plan_params(M, N, K).workspace_bytes <= (4 << 20)
