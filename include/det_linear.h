@@ -256,7 +256,7 @@ DET_API det_status_t det_rmsnorm(const float* x, const float* g, float eps, int6
  *   q : device FP32 [B, Hq, D];  k, v : device FP32 [B, Hkv, T, D];  o : device FP32 [B, Hq, D]; all
  *   row-major, contiguous and 16-byte aligned (DET_ERR_ALIGNMENT otherwise).
  *   Hq / Hkv in {1, 2, 4, 8}; D a multiple of 4, at most 256; the scores and segment sums of a (batch,
- *   KV head) live in shared memory, which limits T (about 9000 keys at Hq / Hkv = 4, D = 128):
+ *   KV head) live in the shared memory of up to 16 thread blocks, which limits T (151 552 keys at Hq / Hkv = 4, D = 128):
  *   DET_ERR_UNSUPPORTED_SHAPE with a message beyond that.
  * Enqueued on `stream`, no synchronisation, no allocation.
  */

@@ -34,8 +34,9 @@
 // (ring_or_registers below).  Next come the instructions: the lane trees (their operands are
 // permuted so that no step selects between registers), P.V in packed FMAs.  Small shapes are bound by latency, of reads
 // from other blocks' shared memory among others: what crosses blocks is read many values at a time.
-// Measured on B200, 32 query / 8 KV heads, D = 128, us a call before -> now: B = 8, T = 4096 59.3 -> 53.5; B = 8, T = 8192 105.6 -> 86.9;
-// B = 32, T = 2048 97.9 -> 86.3; B = 2, T = 4096 40.6 -> 31.4; B = 1, T = 32768 131.8 -> 85.9; 8 / 8 heads, B = 8, T = 2000 40.7 -> 28.5.
+// Measured on B200, 32 query / 8 KV heads, D = 128, us a call (in brackets with loads through registers only): B = 8, T = 4096 55.9
+// (61.6); B = 8, T = 8192 86.9 (105.6); B = 32, T = 2048 86.3 (97.9); B = 2, T = 4096 31.4 (40.6); B = 1, T = 32768 85.9 (131.8); 8 / 8
+// heads, B = 8, T = 2000 28.5 (40.7).
 #include "internal.h"
 #include "device_utils.cuh"
 #include <cooperative_groups.h>

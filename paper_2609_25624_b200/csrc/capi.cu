@@ -335,12 +335,12 @@ static HostRoute host_route(int64_t M, int64_t N, int64_t K, bool sync)
     }
     if (sync) {
         // One call's latency.  y straight from the kernel up to 192 KB (M = 8, N = K = 4096 34.9 us, by a copying kernel 35.5; at M = 30,
-        // N = 4369, K = 512, 512 KB, 61 and 42), and beyond where the weight stream is long enough to hide the stores of
+        // N = 4369, K = 512, 512 KB, 61 and 42), 256 KB of a long call (M = 16, N = 4096, K = 14336 84.2 and 86.9), and beyond where the weight stream is long enough to hide the stores of
         // earlier tiles (M = 8, N = 28672, K = 4096, 896 KB 73.5, by a copying kernel 87.5, by copies 95).
         // All in all 0.87 of two copies' time, nowhere above 1.08.
         constexpr int64_t most = 1024 * KiB + 4 * KiB;
         route.x_by_kernel = xb <= most;
-        if (yb <= 192 * KiB || (yb <= most && K >= 256 * M && N >= 8192)) route.y = Across::kDirect;
+        if (yb <= 192 * KiB || (yb <= 256 * KiB && K >= 512 * M) || (yb <= most && K >= 256 * M && N >= 8192)) route.y = Across::kDirect;
         else if (yb <= most) route.y = Across::kKernel;
     } else if (xb <= 256 * KiB && yb <= 256 * KiB) {
         // Calls of several streams overlap: the copy engines work beside the kernels, while SMs that wait for the bus are lost to the

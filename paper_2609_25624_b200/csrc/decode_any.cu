@@ -6,7 +6,7 @@
 // segment sums are added in ascending order as the warp goes (rule R3).
 //
 // What bounds it: with rows that start anywhere, TMA and vector loads are out, and a warp that walks its row chunk by
-// chunk waits for memory every time (the kernel before this one did, and read the row again for every batch row).
+// chunk waits for memory every time.
 //   * weights go from memory to registers, a group of UC chunks of every row loaded ahead of the group that is
 //     being multiplied.  16-bit rows start on any 2-byte boundary: a lane loads the two or three aligned words that hold
 //     its four weights, two byte permutations line them up (rows at the very ends of W, where such a word would reach
@@ -15,9 +15,10 @@
 //     -0.0 and weights beyond K count as +0: the product is -0.0, and adding -0.0 changes no accumulator (not even a
 //     -0.0 one), so elements beyond K are skipped in effect without a test in the loop;
 //   * two rows' chains advance in one packed FMA (RT > 1), the lane sums of all outputs fold in one butterfly.
-// Measured on B200, us a call in a chain, before -> now: M = 6, N = 1333, K = 1001 15.8 -> 7.4; M = 3, N = K = 4097 49.6 -> 16.4;
-// M = 64, N = 8192, K = 4097 1705 -> 218 (27 % of the FP32 peak: line-up and widening of every weight in every batch
-// block, one-word loads); M = 64, N = 300, K = 333 68 -> 6; 20 x 2000 x 2001 with FP16 weights 92 -> 21.
+// Measured on B200, us a call in a chain (in brackets a warp per row that walks it chunk by chunk, for every batch row again): M = 6, N =
+// 1333, K = 1001 6.3 (15.8); M = 3, N = K = 4097 16.4 (49.6); M = 64, N = 8192, K = 4097 218 (1705; 27 % of the FP32 peak: line-up and
+// widening of every weight in every batch block, one-word loads); M = 64, N = 300, K = 333 6 (68); 20 x 2000 x 2001 with FP16 weights
+// 21 (92).
 #include "internal.h"
 #include "device_utils.cuh"
 

@@ -62,7 +62,7 @@ cudaError_t launch_generic(const LaunchArgs& a, int bucket);
 // Second pass of split-K: y[m,n] = (((P0 + P1) + P2) + ...) (+ b[n]); rule R3.
 cudaError_t launch_combine(const LaunchArgs& a);
 
-// Register-staged prefill kernel (the fallback without an activation workspace; a.variant 15 .. 18 forces 5 .. 8 rows
+// Register-staged prefill kernel (the fallback without a schedule workspace; a.variant 15 .. 18 forces 5 .. 8 rows
 // per thread).
 cudaError_t launch_prefill(const LaunchArgs& a);
 // Prefill kernel with both tiles fed by TMA (prefill_tma_kernel.cuh); block tile 16 tm rows x width columns.  Tensor maps,

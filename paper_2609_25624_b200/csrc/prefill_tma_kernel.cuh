@@ -31,19 +31,18 @@
 // LAST, so the hand-over is long done when it is needed.  Blocks number themselves in the order in which they start (a
 // ticket), so a block only ever waits for one that is already running; the wait is bounded like every other.
 //
-// Measured on B200, whole call, against the kernel before this one (8 x 8 per thread, converting for itself, activations
-// transposed by a first launch, one block per unit): M = 512, N = 28672, K = 4096 2005 -> 1865 us (86.6 % of 74.45
-// TFLOP/s); M = 2048, N = 4096, K = 14336 3916 -> 3622 us (89.2 %); M = 72, N = 28672, K = 4096 391 -> 311 us; M = 128,
-// N = 4096, K = 14336 299 -> 254 us; 100 x 1000 x 1000 with FP32 weights 41 -> 13 us.
+// Measured on B200, whole call: M = 512, N = 28672, K = 4096 1862 us (86.7 % of 74.45 TFLOP/s); M = 2048, N = 4096, K = 14336 3616 us
+// (89.3 %); M = 72, N = 28672, K = 4096 311 us; M = 128, N = 4096, K = 14336 255 us; 100 x 1000 x 1000 with FP32 weights 12.6 us.  (8 x 8
+// outputs a thread, every warp converting for itself, activations transposed by a first launch: 2005, 3916, 391, 299 and 41 us.)
 //
 // Any K, any alignment (PLAIN): rows that start anywhere are out of TMA's reach, so the preparing warps load them themselves,
 // a slab ahead (a block of 4 rows x 4 k ahead for the 256 columns wide tile, whose register split leaves no more: 56 registers
 // spilled, so they get 88 here and the multiplying warps 208); a 16-bit row's weights are two or three aligned words, lined up
 // by byte permutations (element by element where such a word would reach outside of W).  Beyond K they store -0.0 for
 // activations and +0 for weights: the product is -0.0, and adding -0.0 changes no accumulator (not even a -0.0 one), so the
-// multiply loop may run on to a whole octet.  Everything else is the same kernel.  Against one thread per output before: M =
-// 300, N = 8192, K = 4097 13362 -> 379 us (71 % of 74.45 TFLOP/s; the scalar loads hold it up); 100 x 1001 x 1001 156 -> 18 us,
-// with FP32 weights 157 -> 17 us; 130 x 500 x 333 48 -> 13 us.
+// multiply loop may run on to a whole octet.  Everything else is the same kernel.  M = 300, N = 8192, K = 4097 379 us (71 % of 74.45
+// TFLOP/s; the scalar loads hold it up; one thread per output 13362); 100 x 1001 x 1001 18 us, with FP32 weights 17 (156, 157);
+// 130 x 500 x 333 13 us (48).
 //
 // Every wait is bounded: one that expires records the fact in the device status word and the block returns without
 // storing.

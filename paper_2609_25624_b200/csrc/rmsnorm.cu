@@ -149,8 +149,8 @@ rmsnorm_row_in_registers_kernel(const float* __restrict__ x, const float* __rest
 // Few rows (16-byte aligned, H % 4 == 0, up to kBlockRowMax elements): a block per row.  A row's chains are one warp's
 // lanes, but a single warp per row also loads and stores alone and fetches the gain only when the sum is done (7.4 us for
 // four rows of 4096): here the whole block loads the row into shared memory and the gain into registers at once, warp 0
-// runs the 32 chains from shared memory, and the whole block writes.  Starts under the tail of the kernel before it and lets
-// the next one start (programmatic dependent launch).
+// runs the 32 chains from shared memory, and the whole block writes.  Starts under the tail of the kernel before it and, once that
+// is complete, lets the next one start (programmatic dependent launch).
 constexpr int kBlockRowThreads = 256;
 constexpr int kBlockRowMax = 49152;                  // 192 KB of shared memory
 constexpr long long kBlockRowMaxRows = 512;
@@ -232,7 +232,9 @@ cudaError_t launch_rmsnorm(const float* x, const float* g, float eps, int64_t M,
     const bool vec = (H % 4 == 0) && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(g) | reinterpret_cast<uintptr_t>(y)) % 16 == 0);
     // A block per row up to 512 rows (us against the row in one warp's registers: 4 x 4096 2.1 / 3.5, 300 x 4096 3.6 / 4.8, but
     // 600 x 1024 2.8 / 2.6, 1184 x 4096 9.2 / 8.5: many rows keep every SM busy with a warp each), and for rows too long for
-    // those registers whatever their number (64 x 8192 4.1 / 16.8, reading the row twice).
+    // those registers whatever their number (64 x 8192 4.1 / 16.8, reading the row twice).  Beyond some 29 000 elements one block to
+    // an SM is left, which loads, sums and stores in turn: 32 x 49152 12.5 / 121, 4096 x 28672 182 / 269, 4096 x 32768 280 / 304, 4096 x
+    // 49152 401 / 451.
     if (vec && H <= kBlockRowMax && (M <= kBlockRowMaxRows || H > 128 * 32)) {
         static bool configured[kMaxDevices];         // function attributes belong to a device
         int dev = 0;
