@@ -335,19 +335,23 @@ static HostRoute host_route(int64_t M, int64_t N, int64_t K, bool sync)
     }
     if (sync) {
         // One call's latency.  y straight from the kernel up to 192 KB (M = 8, N = K = 4096 34.9 us, by a copying kernel 35.5; at M = 30,
-        // N = 4369, K = 512, 512 KB, 61 and 42), 256 KB of a long call (M = 16, N = 4096, K = 14336 84.2 and 86.9), and beyond where the weight stream is long enough to hide the stores of
-        // earlier tiles (M = 8, N = 28672, K = 4096, 896 KB 73.5, by a copying kernel 87.5, by copies 95).
+        // N = 4369, K = 512, 512 KB, 61 and 42), 256 KB of a long call (M = 16, N = 4096, K = 14336 84.2 and 86.9), and beyond where the
+        // weight stream is long enough to hide the stores of earlier tiles (M = 8, N = 28672, K = 4096, 896 KB 73.5, by a copying
+        // kernel 87.5, by copies 95).
         // All in all 0.87 of two copies' time, nowhere above 1.08.
         constexpr int64_t most = 1024 * KiB + 4 * KiB;
         route.x_by_kernel = xb <= most;
         if (yb <= 192 * KiB || (yb <= 256 * KiB && K >= 512 * M) || (yb <= most && K >= 256 * M && N >= 8192)) route.y = Across::kDirect;
         else if (yb <= most) route.y = Across::kKernel;
-    } else if (xb <= 256 * KiB && yb <= 256 * KiB) {
+    } else {
         // Calls of several streams overlap: the copy engines work beside the kernels, while SMs that wait for the bus are lost to the
-        // other streams.  Small calls gain all the same (three streams, M = 8, N = 1024, K = 1024 6.4 us a call, by copies 8.8); M =
-        // 64, N = 4096, K = 512 takes 25 by copies, 117 with direct stores.  0.89 of two copies' time, nowhere above 1.08.
-        route.x_by_kernel = true;
-        route.y = yb <= (M <= 4 ? 128 : 64) * KiB ? Across::kDirect : Across::kKernel;
+        // other streams.  Small sides gain all the same (three streams, M = 8, N = 1024, K = 1024 6.4 us a call, by copies 8.8); M =
+        // 64, N = 4096, K = 512 takes 25 by copies, 117 with direct stores.  0.89 of two copies' time, at most 1.12; the four
+        // projections of a layer at 1 .. 32 rows, on three streams, 2930 GB/s of weights, by copies 2765, with 256 KB as the line for
+        // x too 2830, and only where both sides are below it 2640.
+        route.x_by_kernel = xb <= 128 * KiB;
+        if (yb <= (M <= 8 ? 128 : 64) * KiB) route.y = Across::kDirect;
+        else if (yb <= 512 * KiB) route.y = Across::kKernel;
     }
     return route;
 }
