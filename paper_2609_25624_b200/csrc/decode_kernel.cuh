@@ -30,6 +30,7 @@
 #include "internal.h"
 #include "device_utils.cuh"
 #include "pipeline_utils.cuh"
+#include <type_traits>
 
 namespace detlin {
 
@@ -58,6 +59,15 @@ __device__ __forceinline__ float wget(const typename WVec<WF>::type& v, int kk)
         if (WF == 0 && SHIFT && !(kk & 1)) return __uint_as_float(w << 16);
         return (kk & 1) ? up16_hi<WF>(w) : up16_lo<WF>(w);
     }
+}
+
+// The same as a move that keeps its place in the instruction order (Cfg::kPipelined).
+template <int WF>
+__device__ __forceinline__ float wget_here(const typename WVec<WF>::type& v, int kk)
+{
+    float f;
+    asm volatile("mov.b32 %0, %1;" : "=f"(f) : "f"(wget<WF, false>(v, kk)));
+    return f;
 }
 
 constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v / 2); }
@@ -123,6 +133,12 @@ struct Cfg {
     static constexpr int kConsumerRegsRaw =
         kMoveRegs ? ((kThreads * kLaunchRegs - kPG * 32 * kProducerRegs) / (kConsumerWarps * 32)) / 8 * 8 : 0;
     static constexpr int kConsumerRegs = kConsumerRegsRaw > 240 ? 240 : kConsumerRegsRaw;
+    // Multiply with the next chunk's loads under this chunk's last steps?  FP32 weights only: their pairs are formed by moves that
+    // the compiler otherwise piles up together with all loads of a chunk (M = 32, N = 28672, K = 4096 254 -> 178 us, M = 24, N =
+    // 6144 68 -> 44; the widenings of 16-bit weights fill those gaps by themselves: 71.4 us there, 75 with it at M = 32, N = 4096,
+    // K = 14336).  4-row tiles only where the second set of operands fits the registers (M = 8, N = 4096, K = 14336 41.6 -> 36.7 us;
+    // with 128 registers it spills: 50 -> 138); tiles of one or two rows wait for memory either way.
+    static constexpr bool kPipelined = WF == 2 && (MT == 8 || (MT == 4 && kLaunchRegs >= 168));
     static_assert(!kMoveRegs || kConsumerRegs * kConsumerWarps * 32 + kProducerRegs * kPG * 32 <= kThreads * kLaunchRegs,
                   "register move must fit in the block's own allocation");
     static_assert(!kMoveRegs || kConsumerRegs >= kLaunchRegs, "consumers only ever grow");
@@ -424,6 +440,119 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
 #pragma unroll
                 for (int j = 0; j < RT / 2; ++j) acc[m][j] = make_float2(0.0f, 0.0f);
 
+            if constexpr (C::kPipelined) {
+                // The operands of a chunk are in registers when its multiplications start: their registers are loaded again for the
+                // next chunk right after the last use, under the last two of the chunk's four steps.
+                const int n_chunks = (k_hi - k_lo + 127) / 128;
+                if (!mine) {
+                    // no rows here: only keeps the ring in step
+                    for (int k0 = k_lo; ok && k0 < k_hi; k0 += KC) {
+                        if (!__all_sync(0xffffffffu, mbar_wait(fullg + 8 * st, phase, abort_flag, status, wait_limit_ns, 2))) { ok = false; break; }
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(emptyg + 8 * st);
+                        if (++st == STAGES) { st = 0; phase ^= 1; }
+                    }
+                    ready = false;
+                } else {
+                    constexpr int kChunks = KC / 128, kPairs = RT / 2;
+                    constexpr int kPerBox = C::kKB / 128;     // chunks of a box
+                    float4 xv[MT];
+                    typename WVec<WF>::type w[RT];
+                    uint32_t xs = 0, ws = 0;                  // where the next loads come from
+                    auto at_chunk = [&](int stage, int ci) {
+                        const uint32_t box = ringg + (uint32_t)(stage * C::kStageBytes) + (uint32_t)(ci / kPerBox * C::kSubBytes);
+                        xs = box + (wm * MT) * C::kXPitch + lane * 16 + (ci % kPerBox) * 512;
+                        ws = box + C::kXBytes + (wr * RT) * C::kWPitch + lane * (4 * C::kEB) + (ci % kPerBox) * (128 * C::kEB);
+                    };
+                    auto load_x = [&](int m) { xv[m] = lds128((m < (MT + 1) / 2 ? xs + x_lo_off : xs - x_lo_off) + m * C::kXPitch); };
+                    auto load_w = [&](int q) { w[q] = wload<WF>(((q & 1) ? ws - w_off : ws + w_off) + q * C::kWPitch); };
+                    float2 wp[2][kPairs];                     // weights (row slot 2 j, row slot 2 j + 1) of this step and of the next
+                    auto form_pairs = [&](auto kk_c) {
+                        constexpr int kk = decltype(kk_c)::value;
+#pragma unroll
+                        for (int j = 0; j < kPairs; ++j) wp[kk & 1][j] = make_float2(wget_here<WF>(w[2 * j], kk), wget_here<WF>(w[2 * j + 1], kk));
+                    };
+                    // Step kk: the lane's element kk of every row, one half of the batch rows after the other.  more: another chunk follows.
+                    auto step = [&](auto kk_c, auto more_c) {
+                        constexpr int kk = decltype(kk_c)::value;
+                        constexpr bool more = decltype(more_c)::value;
+                        auto xk = [&](int m) { return kk == 0 ? xv[m].x : kk == 1 ? xv[m].y : kk == 2 ? xv[m].z : xv[m].w; };
+                        constexpr int kHalf = MT > 1 ? MT / 2 : 1;
+#pragma unroll
+                        for (int h = 0; h < MT; h += kHalf) {
+#pragma unroll
+                            for (int j = 0; j < kPairs; ++j)
+#pragma unroll
+                                for (int m = h; m < h + kHalf; ++m) fma2(acc[m][j], xk(m), wp[kk & 1][j]);
+                            if (h == 0) {
+                                if constexpr (kk < 3 || more) form_pairs(std::integral_constant<int, (kk + 1) % 4>());
+                                if constexpr (kk == 2 && more) {
+#pragma unroll
+                                    for (int q = 0; q < RT; ++q) load_w(q);
+                                }
+                            }
+                            if constexpr (kk == 3 && more) {
+#pragma unroll
+                                for (int m = h; m < h + kHalf; ++m) load_x(m);
+                            }
+                        }
+                    };
+                    using std::integral_constant;
+                    typedef integral_constant<bool, true> Next;
+                    typedef integral_constant<bool, false> Last;
+                    if (!__all_sync(0xffffffffu, ready)) {
+                        if (!__all_sync(0xffffffffu, mbar_wait(fullg + 8 * st, phase, abort_flag, status, wait_limit_ns, 2))) ok = false;
+                    }
+                    int st_cur = st, ci = 0;                  // stage and chunk of the stage in work; st is the stage after it
+                    if (ok) {
+                        at_chunk(st, 0);
+                        if (++st == STAGES) { st = 0; phase ^= 1; }
+#pragma unroll
+                        for (int q = 0; q < RT; ++q) load_w(q);
+#pragma unroll
+                        for (int m = 0; m < MT; ++m) load_x(m);
+                        form_pairs(integral_constant<int, 0>());
+                    }
+                    const int n_loop = ok ? n_chunks - 1 : 0;
+#pragma unroll 1
+                    for (int c = 0; c < n_loop; ++c) {
+                        // No branches but the rare wait: they would cut the loop into pieces that cannot overlap.  (The phase of st_cur,
+                        // which has landed, is the other one of st's if st has wrapped.)
+                        const bool cross = kChunks == 1 || ci == kChunks - 1;   // the next chunk lies in the next stage
+                        const int st_next = cross ? st : st_cur;
+                        const unsigned want = cross ? phase : phase ^ (unsigned)(st == 0);
+                        ready = mbar_test_wait(fullg + 8 * st_next, want);
+                        step(integral_constant<int, 0>(), Last());
+                        __syncwarp();                         // every load from the stage has returned (step 0 uses a part of each)
+                        mbar_arrive_if(emptyg + 8 * st_cur, cross && lane == 0);
+                        step(integral_constant<int, 1>(), Last());
+                        if (!__all_sync(0xffffffffu, ready)) {
+                            if (!__all_sync(0xffffffffu, mbar_wait(fullg + 8 * st_next, want, abort_flag, status, wait_limit_ns, 2))) { ok = false; break; }
+                        }
+                        ci = cross ? 0 : ci + 1;
+                        at_chunk(st_next, ci);
+                        st_cur = st_next;
+                        const bool wrap = st + 1 == STAGES;
+                        phase ^= (unsigned)(cross && wrap);
+                        st = cross ? (wrap ? 0 : st + 1) : st;
+                        step(integral_constant<int, 2>(), Next());
+                        step(integral_constant<int, 3>(), Next());
+                    }
+                    if (ok) {
+                        ready = mbar_test_wait(fullg + 8 * st, phase);
+                        // Elements beyond the end of a ragged K are skipped, not zero-filled (K % 4 == 0 here, so a lane's four elements
+                        // are all inside or all outside).
+                        if (k_lo + 128 * (n_chunks - 1) + 4 * lane < k_hi) {
+                            step(integral_constant<int, 0>(), Last());
+                            step(integral_constant<int, 1>(), Last());
+                            step(integral_constant<int, 2>(), Last());
+                            step(integral_constant<int, 3>(), Last());
+                        }
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(emptyg + 8 * st_cur);
+                    }
+                }
+            } else
             for (int k0 = k_lo; ok && k0 < k_hi; k0 += KC) {
                 // (the votes keep the decision warp-uniform even if a wait expires for some lanes only)
                 if (!__all_sync(0xffffffffu, ready)) {

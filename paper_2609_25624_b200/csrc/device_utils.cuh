@@ -32,6 +32,14 @@ __device__ __forceinline__ float up_elem(typename WeightElem<WF>::type v)
     else return __uint_as_float(((uint32_t)v) << 16);
 }
 
+// d = x * w + d in both halves, each an IEEE fma.rn.f32; volatile: keeps its place in the instruction order
+__device__ __forceinline__ void fma2(float2& d, float x, const float2& w)
+{
+    asm volatile("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %2};\n\tmov.b64 b, {%3, %4};\n\tmov.b64 c, {%0, %1};\n\t"
+                 "fma.rn.f32x2 c, a, b, c;\n\tmov.b64 {%0, %1}, c;\n\t}"
+                 : "+f"(d.x), "+f"(d.y) : "f"(x), "f"(w.x), "f"(w.y));
+}
+
 // Balanced tree over the 32 lanes of a warp, adjacent lanes first (xor 1, 2, 4, 8, 16 in that
 // order).  fadd is commutative, so both partners compute identical bits and every lane ends with
 // the tree's root.

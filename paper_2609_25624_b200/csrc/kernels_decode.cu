@@ -29,8 +29,10 @@ int m_class(int64_t M) { return M <= 1 ? 0 : M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 
 // and performs rb * mb * K multiply-adds at the FMA rate of an SM times an efficiency that depends on the
 // warp tile; whichever is larger binds.  Units resident on one SM share it.  Fewer than eight consumer
 // warps per SM hide latency badly; every unit pays for its lane trees (one per segment) and, with several
-// segment groups, for the fold through shared memory.
-double tiling_cost(const DecodeEntry& e, int64_t M, int64_t N, int64_t K, int S, int sm_count)
+// segment groups, for the fold through shared memory.  FP32 weights have rates of their own (fitted to sweeps of 52 shapes at
+// batch 1 .. 64, mean loss against the best tiling 2 %; with the rates of the 16-bit formats 24 %): their multiply loop is another
+// one in the larger tiles, which blocks of four consumer warps compile with a few spilled registers.
+double tiling_cost(const DecodeEntry& e, int wfmt, int64_t M, int64_t N, int64_t K, int S, int sm_count)
 {
     const DecodeConfig& c = e.cfg;
     const int occ = e.occupancy(S);
@@ -45,10 +47,17 @@ double tiling_cost(const DecodeEntry& e, int64_t M, int64_t N, int64_t K, int S,
     double eff = c.mt >= 8 ? 0.707 : c.mt == 4 ? 0.70 : c.mt == 2 ? 0.345 : 0.2;
     if (c.kc >= 512 && c.mt >= 8) eff *= 1.2;          // half as many stage boundaries; smaller tiles prefer a deeper ring
     if (c.kc <= 128) eff *= 0.9;
+    double row_bytes = (double)K * 2.0, hbm_rate = 22.5;
+    if (wfmt == DET_WEIGHT_FP32) {
+        const bool small = c.wm * c.wr * c.sk <= 4;
+        eff = c.mt >= 8 ? (small ? 0.47 : 0.52) : c.mt == 4 ? (small ? 0.24 : 0.43) : c.mt == 2 ? 0.49 : 0.075;
+        row_bytes = (double)K * 4.0;
+        hbm_rate = 32.0;
+    }
     const double latency = warps >= 8.0 ? 1.0 : 8.0 / warps;
     const double fma = (double)rb * (double)mb * (double)K / 128.0 / eff * resident;
-    // weights from HBM at 22.5 bytes per clock and SM; the unit's activations come again from L2 for every unit
-    const double hbm = ((double)rb * (double)K * 2.0 / 22.5 + 0.06 * (double)mb * (double)K * 4.0 / 64.0) * resident;
+    // weights from HBM at 22.5 bytes per clock and SM (FP32 32); the unit's activations come again from L2 for every unit
+    const double hbm = ((double)rb * row_bytes / hbm_rate + 0.06 * (double)mb * (double)K * 4.0 / 64.0) * resident;
     const double body = (fma > hbm ? fma : hbm) * latency;
     const double overhead = (double)S * 1020.0 * ((double)(mb * rb) / 896.0) + (c.sk > 1 ? 1500.0 : 0.0);
     if (rb >= 56 && mb >= 16) {
@@ -105,7 +114,7 @@ bool decode_config_for(int64_t M, int64_t N, int64_t K, int S, int wfmt, int var
         const DecodeClassTable* t = class_table(wfmt, classes[ci]);
         for (int i = 0; i < t->count; ++i) {
             if (variant == 0) {
-                const double c = tiling_cost(t->entries[i], M, N, K, S, sms);
+                const double c = tiling_cost(t->entries[i], wfmt, M, N, K, S, sms);
                 if (c < best) { best = c; pick_cls = classes[ci]; pick = i; }
             } else if (t->entries[i].occupancy(S) > 0 && ++seen == variant) {
                 pick_cls = classes[ci];

@@ -124,13 +124,6 @@ __device__ __forceinline__ void sts128(uint32_t addr, float a, float b, float c,
 {
     asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
-// d = x * w + d in both halves, each an IEEE fma.rn.f32; volatile: keeps its place in the instruction order
-__device__ __forceinline__ void fma2(float2& d, float x, const float2& w)
-{
-    asm volatile("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %2};\n\tmov.b64 b, {%3, %4};\n\tmov.b64 c, {%0, %1};\n\t"
-                 "fma.rn.f32x2 c, a, b, c;\n\tmov.b64 {%0, %1}, c;\n\t}"
-                 : "+f"(d.x), "+f"(d.y) : "f"(x), "f"(w.x), "f"(w.y));
-}
 __device__ __forceinline__ float2 lds_f2(uint32_t addr)
 {
     float2 v;
