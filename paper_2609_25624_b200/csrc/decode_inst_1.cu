@@ -25,6 +25,9 @@ static const DecodeEntry kEntries3[] = {
     ROW(8, 1, 14, 2, 2, 256),
     ROW(8, 1, 14, 4, 1, 256),
     ROW(4, 2, 14, 4, 1, 256),
+#if DET_WF != 2
+    ROW(8, 1, 14, 8, 1, 256),
+#endif
     ROW(4, 2, 14, 2, 1, 256),
 };
 extern const DecodeClassTable DET_TABLE_NAME2(3, DET_WF) = {kEntries3, (int)(sizeof(kEntries3) / sizeof(kEntries3[0]))};

@@ -107,8 +107,10 @@ struct Cfg {
     // that is nearly empty costs a whole tile: for the tall tiles, 3.46 -> 3.5 instead of 4 rounds at 28672 rows (M = 16: 84.0
     // -> 78.8 us).  Below that the weight stream binds, which the blocks of a thin last round share out among themselves (M = 8,
     // 128256 rows: 200 us without, 207 with), and tiles of 28 rows lose more by the extra bookkeeping (M = 32, 1 %) than
-    // their smaller rounds leave to gain.
-    static constexpr bool kDealRest = kMB >= 16 && kRB >= 56;
+    // their smaller rounds leave to gain.  Tiles of 112 rows (one block to an SM, whose eight warps share each stage's activations)
+    // serve matrices of many rounds only, where equal shares count: M = 8, 128256 rows 184.8 -> 181.4 us, under the power limit
+    // that this call reaches 221 -> 218.
+    static constexpr bool kDealRest = (kMB >= 16 && kRB >= 56) || kRB >= 112;
     // BF16: the lower half of a word is widened by a byte permutation, or by a shift in the 4-row tilings of two segment groups
     // that run two blocks to an SM at the full 128 registers: M = 24, N = 6144, K = 4096 35.5 us by shift, 39.4 by permutation (M =
     // 8, N = K = 4096 9.86 and 9.72).  Elsewhere the permutation is up to 3 % faster: M = 48, N = 28672, K = 4096 274.8 and 282.6.

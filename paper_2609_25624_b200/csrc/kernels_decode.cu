@@ -60,7 +60,7 @@ double tiling_cost(const DecodeEntry& e, int wfmt, int64_t M, int64_t N, int64_t
     const double hbm = ((double)rb * row_bytes / hbm_rate + 0.06 * (double)mb * (double)K * 4.0 / 64.0) * resident;
     const double body = (fma > hbm ? fma : hbm) * latency;
     const double overhead = (double)S * 1020.0 * ((double)(mb * rb) / 896.0) + (c.sk > 1 ? 1500.0 : 0.0);
-    if (rb >= 56 && mb >= 16) {
+    if ((rb >= 56 && mb >= 16) || rb >= 112) {
         // what is left after whole rounds is dealt out by row groups (Cfg::kDealRest); half a tile takes a little longer than
         // half the time (one warp per scheduler)
         int64_t shares = (int64_t)sm_count * occ / mblocks;
@@ -68,6 +68,9 @@ double tiling_cost(const DecodeEntry& e, int wfmt, int64_t M, int64_t N, int64_t
         shares = shares < 1 ? 1 : shares > groups ? groups : shares;
         const int64_t whole = groups / (shares * c.wr), rest = groups - whole * shares * c.wr;
         const double part = (double)((rest + shares - 1) / shares) / c.wr;
+        // tiles of 112 rows only for many rounds: M = 7, N = 50000, K = 2048 (3.02 rounds) 45.9 us, by 56 rows 44.1; M = 8, N = 28672,
+        // K = 4096 (1.7 rounds) 50.5 and 50.1; N = 128256 (7.7 rounds) 181.4 and 184.8
+        if (rb >= 112 && whole < 5) return 1e300;
         if (whole > 0) return (double)whole * (body + overhead) + (part < 1.0 ? part * 1.08 : 1.0) * body + (rest ? overhead : 0.0);
     }
     return (double)rounds * (body + overhead);
