@@ -105,6 +105,7 @@ det_status_t run_device(det_linear_plan_t* plan, const float* x, const void* W, 
     a.sm_count = plan->sm_count;
     a.max_blocks = plan->max_blocks;
     a.variant = plan->variant;
+    a.any_layout = &plan->any_layout;
 
     int kernel = plan->forced_kernel >= 0 ? plan->forced_kernel : p.kernel;
     const int64_t k_align = p.weight_format == DET_WEIGHT_FP32 ? 4 : 8;     // 16-byte row pitch of W (x: K % 4)

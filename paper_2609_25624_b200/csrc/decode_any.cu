@@ -15,10 +15,11 @@
 //     -0.0 and weights beyond K count as +0: the product is -0.0, and adding -0.0 changes no accumulator (not even a
 //     -0.0 one), so elements beyond K are skipped in effect without a test in the loop;
 //   * two rows' chains advance in one packed FMA (RT > 1), the lane sums of all outputs fold in one butterfly.
+//   * a small layer is one wave of warps that wait for their own instructions: batch blocks of fewer rows and a warp per segment
+//     spread them over the SMs (choose_layout).
 // Measured on B200, us a call in a chain (in brackets a warp per row that walks it chunk by chunk, for every batch row again): M = 6, N =
-// 1333, K = 1001 6.3 (15.8); M = 3, N = K = 4097 16.4 (49.6); M = 64, N = 8192, K = 4097 218 (1705; 27 % of the FP32 peak: line-up and
-// widening of every weight in every batch block, one-word loads); M = 64, N = 300, K = 333 6 (68); 20 x 2000 x 2001 with FP16 weights
-// 21 (92).
+// 1333, K = 1001 4.7 (15.8); M = 3, N = K = 4097 14.3 (49.6); M = 64, N = 8192, K = 4097 218 (1705; 27 % of the FP32 peak: line-up and
+// widening of every weight in every batch block, one-word loads); M = 64, N = 300, K = 333 4.6 (68).
 #include "internal.h"
 #include "device_utils.cuh"
 
@@ -28,8 +29,10 @@ namespace {
 
 constexpr int kAnySmemBytes = 110 * 1024;            // activations of one window of K with two blocks of 8 warps per SM ...
 constexpr int kAnySmemBytes1 = 220 * 1024;           // ... or one block of 16
+constexpr int kSplitBytes = 8 * 32 * 4;              // SPLIT: the second segments' sums, one a lane
 
-template <int WF, int MT, int RT>
+// SPLIT: the two segments of a row belong to two warps, the second half of the block's warps to the second ones.
+template <int WF, int MT, int RT, bool SPLIT>
 __global__ void __launch_bounds__(512, 1)
 decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::type* __restrict__ W, const float* __restrict__ b,
                   float* __restrict__ y, int M, int N, unsigned K, unsigned seg_len, long long ldy, unsigned win, int groups)
@@ -38,7 +41,10 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
     constexpr int UC = 8 / RT;                       // chunks of a row loaded together
     constexpr int NW = WF == 2 ? 4 : 3;              // words a lane loads of a chunk
     extern __shared__ __align__(16) float xs[];      // [MT][win]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, threads = blockDim.x;
+    const int lane = threadIdx.x & 31, threads = blockDim.x;
+    const int rows_of_warps = threads >> (SPLIT ? 6 : 5);     // warps that have rows of their own
+    const int warp = SPLIT ? (int)(threadIdx.x >> 5) % rows_of_warps : (int)(threadIdx.x >> 5);
+    const bool second = SPLIT && (int)(threadIdx.x >> 5) >= rows_of_warps;
     const int m0 = blockIdx.y * MT;
     // The next kernel may start, and request its weights, only once what precedes this kernel is complete.
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -48,20 +54,25 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
     auto stage = [&](unsigned w_lo) {
         const unsigned len = min(win, K - w_lo);
         const uint32_t base = (uint32_t)__cvta_generic_to_shared(xs);
-#pragma unroll 1
-        for (int m = 0; m < MT; ++m) {
-            const float* src = x + (size_t)min(m0 + m, M - 1) * K + w_lo;     // rows beyond M repeat the last one
-#pragma unroll 4
-            for (unsigned i = threadIdx.x; i < len; i += threads)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(base + (m * win + i) * 4u), "l"(src + i) : "memory");
-            for (unsigned i = len + threadIdx.x; i < win; i += threads) xs[m * win + i] = -0.0f;
+        for (unsigned i = threadIdx.x; i < win; i += threads) {
+            const float* src = x + (size_t)m0 * K + w_lo + i;
+            if (i < len) {
+#pragma unroll
+                for (int m = 0; m < MT; ++m) {
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(base + (m * win + i) * 4u), "l"(src) : "memory");
+                    if (m0 + m + 1 < M) src += K;    // rows beyond M repeat the last one
+                }
+            } else {
+#pragma unroll
+                for (int m = 0; m < MT; ++m) xs[m * win + i] = -0.0f;
+            }
         }
         asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
     };
 
     const bool one_window = K <= win;
     for (int grp = (int)blockIdx.x; grp < groups; grp += (int)gridDim.x) {
-        const int n0 = (grp * (threads >> 5) + warp) * RT;
+        const int n0 = (grp * rows_of_warps + warp) * RT;
 
         // The warp's rows, as the word that holds the lane's first weight, and how the lane's words are lined up: bytes
         // 0 .. 3 of two words for rows that start on a word, bytes 2 .. 5 for the others.  A warp with a row at
@@ -168,8 +179,13 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
         auto group_end = [&](unsigned c, unsigned s_hi, unsigned w_hi) { return min(min(K, s_hi), min(w_hi, c + 128 * UC)); };
         bool first = true;                           // no segment has ended yet
         unsigned w_hi = win, w_lo = ~0u;             // end of the window of the group loaded last; start of the one in shared memory
-        unsigned s_hi = seg_len;                     // end of the segment of the group being multiplied
-        unsigned c = 0, c_end = group_end(0, s_hi, w_hi);
+        unsigned s_hi = second ? 2 * seg_len : seg_len;      // end of the segment of the group being multiplied
+        unsigned c = second ? seg_len : 0, c_end = group_end(c, s_hi, w_hi);
+        const unsigned c_stop = SPLIT && !second ? seg_len : K;
+        if (second) {
+#pragma unroll
+            for (int r = 0; r < RT; ++r) pw[r] += seg_len * (unsigned)sizeof(WT) / 4;
+        }
         load(raw[0], c, c_end);
 #pragma unroll
         for (int m = 0; m < MT; ++m)
@@ -177,7 +193,7 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
             for (int r = 0; r < RT; ++r) acc[m][r] = 0.0f;
         int buf = 0;
 #pragma unroll 1
-        while (c < K) {
+        while (c < c_stop) {
             if (one_window ? (w_lo != 0 && grp == (int)blockIdx.x) : (w_lo == ~0u || c - w_lo >= win)) {
                 w_lo = one_window ? 0 : c;
                 __syncthreads();                     // everybody has finished with the window before
@@ -187,7 +203,7 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
             const bool seg_done = c_end == min(K, s_hi);
             if (seg_done) s_hi += seg_len;
             if (c_end == w_hi) w_hi += win;
-            const unsigned nc_end = c_end < K ? group_end(c_end, s_hi, w_hi) : c_end;
+            const unsigned nc_end = c_end < c_stop ? group_end(c_end, s_hi, w_hi) : c_end;
             const float* xl = xs + (one_window ? c : c - w_lo) + 4 * lane;
 #pragma unroll
             for (int half = 0; half < 2; ++half) {   // (the buffers are registers: their index has to be a constant)
@@ -218,13 +234,28 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
             c = c_end;
             c_end = nc_end;
         }
-        constexpr int kSteps = Scatter<MT * RT>::kSteps;
-        if ((lane >> kSteps) == 0) {
+        constexpr int kSteps = Scatter<MT * RT>::kSteps, kKeep = Scatter<MT * RT>::kKeep;
+        static_assert(!SPLIT || kKeep == 1, "room for one sum a lane");
+        if constexpr (SPLIT) {
+            // the second segments' sums meet the first ones' in shared memory, behind the activations
+            float* sums = xs + MT * win + (warp * kKeep << 5) + lane;
+            if (second) {
+#pragma unroll
+                for (int t = 0; t < kKeep; ++t) sums[t << 5] = tot[t];
+            }
+            __syncthreads();
+            if (!second) {
+#pragma unroll
+                for (int t = 0; t < kKeep; ++t) tot[t] = __fadd_rn(tot[t], sums[t << 5]);
+            }
+            if (grp + (int)gridDim.x < groups) __syncthreads();
+        }
+        if (!second && (lane >> kSteps) == 0) {
             int base = 0, cnt = MT * RT;
 #pragma unroll
             for (int i = 0; i < kSteps; ++i) { cnt >>= 1; base += ((lane >> i) & 1) * cnt; }
 #pragma unroll
-            for (int t = 0; t < Scatter<MT * RT>::kKeep; ++t) {
+            for (int t = 0; t < kKeep; ++t) {
                 const int idx = base + t;
                 const int m = m0 + idx / RT, n = n0 + idx % RT;
                 if (m < M && n < N) y[m * ldy + n] = b ? __fadd_rn(tot[t], __ldg(b + n)) : tot[t];
@@ -233,7 +264,7 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
     }
 }
 
-template <int WF, int MT, int RT>
+template <int WF, int MT, int RT, bool SPLIT>
 cudaError_t launch_t(const LaunchArgs& a, long long mblocks, int sms)
 {
     static bool configured[kMaxDevices];             // function attributes belong to a device
@@ -241,7 +272,7 @@ cudaError_t launch_t(const LaunchArgs& a, long long mblocks, int sms)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    auto kern = decode_any_kernel<WF, MT, RT>;
+    auto kern = decode_any_kernel<WF, MT, RT, SPLIT>;
     if (!configured[dev]) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kAnySmemBytes1);
         if (e != cudaSuccess) return e;
@@ -250,10 +281,10 @@ cudaError_t launch_t(const LaunchArgs& a, long long mblocks, int sms)
     // Two blocks of 8 warps per SM, or one of 16 where only that keeps all activations of a batch block in shared memory; the
     // window holds whole chunks of 128.
     const long long padded = (a.K + 127) / 128 * 128, cap = kAnySmemBytes / 4 / MT / 256 * 256, cap1 = kAnySmemBytes1 / 4 / MT / 256 * 256;
-    const bool big = padded > cap;
-    const int warps = big ? 16 : 8;
+    const bool big = SPLIT || padded > cap;
+    const int warps = big ? 16 : 8, row_warps = SPLIT ? 8 : warps;
     const unsigned win = (unsigned)(!big ? padded : padded < cap1 ? padded : cap1);
-    const long long groups = (a.N + warps * RT - 1) / (warps * RT);
+    const long long groups = (a.N + row_warps * RT - 1) / (row_warps * RT);
     long long grid = (big ? 1ll : 2ll) * sms / mblocks;
     if (grid < 1) grid = 1;
     if (a.max_blocks > 0 && grid > a.max_blocks) grid = a.max_blocks;
@@ -262,7 +293,7 @@ cudaError_t launch_t(const LaunchArgs& a, long long mblocks, int sms)
     cudaLaunchAttribute attr[1];
     cfg.gridDim = dim3((unsigned)grid, (unsigned)mblocks);
     cfg.blockDim = dim3(32 * warps);
-    cfg.dynamicSmemBytes = (size_t)MT * win * 4;
+    cfg.dynamicSmemBytes = (size_t)MT * win * 4 + (SPLIT ? kSplitBytes : 0);
     cfg.stream = a.stream;
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -272,18 +303,67 @@ cudaError_t launch_t(const LaunchArgs& a, long long mblocks, int sms)
                               (unsigned)a.K, (unsigned)a.seg_len, (long long)a.ldy, win, (int)groups);
 }
 
+// How a call is laid out: batch rows and weight rows of a warp, and whether two warps share a row's two segments (in sixteen-warp
+// blocks that hold all of K and run all at once).
+struct Layout { int mt, rt; bool split; };
+
+// Predicted cycles of a layout: instructions of a warp (operands, line-up and multiplications of its chunks, its part of the
+// activations, lane trees), at the rate of a lone warp or of the SM's schedulers, whichever is slower.  Constants fitted to every layout
+// of 68 drawn shapes (M 1 .. 64, N 64 .. 60000, K 101 .. 9001): mean loss against the best layout 2 %.
+double layout_cost(const LaunchArgs& a, int wfmt, const Layout& l, int sms)
+{
+    const long long padded = (a.K + 127) / 128 * 128, cap = kAnySmemBytes / 4 / l.mt / 256 * 256, cap1 = kAnySmemBytes1 / 4 / l.mt / 256 * 256;
+    const bool big = l.split || padded > cap;
+    const long long warps = big ? 16 : 8, row_warps = l.split ? 8 : warps, occ = big ? 1 : 2;
+    const long long win = !big ? padded : padded < cap1 ? padded : cap1;
+    const long long groups = (a.N + row_warps * l.rt - 1) / (row_warps * l.rt), mblocks = (a.M + l.mt - 1) / l.mt;
+    long long gx = occ * sms / mblocks;
+    gx = gx < 1 ? 1 : gx > groups ? groups : gx;
+    const long long blocks = gx * mblocks, per_sm = (blocks + sms - 1) / sms;
+    if (l.split && (blocks > sms || l.mt >= 8 || padded * 4 * l.mt + kSplitBytes > kAnySmemBytes1)) return 1e300;
+    const double iters = (double)((groups + gx - 1) / gx), waves = (double)((blocks + occ * sms - 1) / (occ * sms));
+    const double chunks = (double)padded / 128 / (l.split ? 2 : 1);
+    double per_chunk = l.mt * (2 + (l.rt == 1 ? 4 : 2 * l.rt));
+    if (l.mt * l.rt >= 32) per_chunk *= 1.31;        // registers run out
+    per_chunk += 6.4 + l.rt * (wfmt == 2 ? 14.6 : 11.6);
+    const double body = chunks * per_chunk + 1.34 * l.mt * l.rt * (l.split ? 1 : 2) + 254;
+    const double stage = 9.0 * l.mt * (double)win / (32.0 * warps) * (win >= padded ? 1.0 : (double)((padded + win - 1) / win) * iters);
+    const double shared = (double)(warps * (per_sm < occ ? per_sm : occ)) / 4 * 1.08;
+    return (l.split && l.rt == 4 ? 1.2 : 1.0) * waves * ((body * iters + stage) * (shared > 3.94 ? shared : 3.94) + 546);
+}
+
+// Fewer batch rows a warp than there are, where the layer leaves SMs idle otherwise (the weights then come from L2 for the other batch
+// blocks): M = 6, N = 1333, K = 1001 6.1 -> 4.7 us, M = 7, N = 250, K = 3001 with FP32 weights 10.1 -> 5.8; a warp a segment: M = 8, N = 64,
+// K = 4095 19.5 -> 6.8.  The largest batch block with one, two or four rows by the number of warps, the rule without this, keeps the calls
+// that would not gain 3 %.
+Layout choose_layout(const LaunchArgs& a, int wfmt, int sms)
+{
+    const int most = a.M <= 1 ? 1 : a.M <= 2 ? 2 : a.M <= 4 ? 4 : 8;
+    const long long rows = a.N * ((a.M + most - 1) / most);
+    Layout best{most, rows >= 4ll * 8 * sms ? 4 : rows >= 2ll * 4 * sms ? 2 : 1, false};
+    double best_cost = 0.97 * layout_cost(a, wfmt, best, sms);
+    for (int mt = most; mt >= 1 && 16 * mt >= a.M; mt /= 2)
+        for (int rt = 1; rt <= 4; rt *= 2)
+            for (int split = 0; split <= (a.S == 2 && mt < 8 ? 1 : 0); ++split) {
+                const Layout l{mt, rt, split != 0};
+                const double c = layout_cost(a, wfmt, l, sms);
+                if (c < best_cost) { best_cost = c; best = l; }
+            }
+    return best;
+}
+
 template <int WF, int MT>
-cudaError_t launch_m(const LaunchArgs& a)
+cudaError_t launch_m(const LaunchArgs& a, const Layout& l, int sms)
 {
     const long long mblocks = (a.M + MT - 1) / MT;
-    const int sms = a.sm_count > 0 ? a.sm_count : 148;
-    // Rows per warp: four from 8 warps' worth of work per SM on, two from 4, one for smaller layers (they need the warps).
-    // Measured, us with four / two rows against the next smaller number: M = 3, N = K = 4097 22.8 (four) 16.4 (two) 28.7 (one);
-    // M = 1, N = 1333, K = 1001 3.3 (two) 6.9 (one); M = 6 likewise 7.4 (two) 8.7 (one).
-    const long long rows = a.N * mblocks;
-    if (rows >= 4ll * 8 * sms) return launch_t<WF, MT, 4>(a, mblocks, sms);
-    if (rows >= 2ll * 4 * sms) return launch_t<WF, MT, 2>(a, mblocks, sms);
-    return launch_t<WF, MT, 1>(a, mblocks, sms);
+    if constexpr (MT < 8) {
+        if (l.split) {
+            if (l.rt == 4) return launch_t<WF, MT, 4, true>(a, mblocks, sms);
+            return l.rt == 2 ? launch_t<WF, MT, 2, true>(a, mblocks, sms) : launch_t<WF, MT, 1, true>(a, mblocks, sms);
+        }
+    }
+    if (l.rt == 4) return launch_t<WF, MT, 4, false>(a, mblocks, sms);
+    return l.rt == 2 ? launch_t<WF, MT, 2, false>(a, mblocks, sms) : launch_t<WF, MT, 1, false>(a, mblocks, sms);
 }
 
 }  // namespace
@@ -292,10 +372,21 @@ cudaError_t launch_m(const LaunchArgs& a)
 #define DET_CAT(a, b) DET_CAT2(a, b)
 cudaError_t DET_CAT(launch_decode_any_wf, DET_WF)(const LaunchArgs& a)
 {
-    if (a.M <= 1) return launch_m<DET_WF, 1>(a);
-    if (a.M <= 2) return launch_m<DET_WF, 2>(a);
-    if (a.M <= 4) return launch_m<DET_WF, 4>(a);
-    return launch_m<DET_WF, 8>(a);
+    const int sms = a.sm_count > 0 ? a.sm_count : 148;
+    // a plan keeps the choice: mt + 16 rt + 256 split
+    int code = a.any_layout ? *a.any_layout : 0;
+    if (code == 0) {
+        const Layout l = choose_layout(a, DET_WF, sms);
+        code = l.mt + 16 * l.rt + 256 * (l.split ? 1 : 0);
+        if (a.any_layout) *a.any_layout = code;
+    }
+    const Layout l{code & 15, (code >> 4) & 15, code >= 256};
+    switch (l.mt) {
+    case 1: return launch_m<DET_WF, 1>(a, l, sms);
+    case 2: return launch_m<DET_WF, 2>(a, l, sms);
+    case 4: return launch_m<DET_WF, 4>(a, l, sms);
+    default: return launch_m<DET_WF, 8>(a, l, sms);
+    }
 }
 
 }  // namespace detlin

@@ -54,6 +54,7 @@ struct LaunchArgs {
     int sm_count;
     int max_blocks;       // 0 = automatic
     int variant;          // 0 = automatic
+    int* any_layout;      // decode for any K: the layout that a plan keeps (0: none yet), or nullptr
     unsigned long long wait_limit_ns;   // bound of one device-side wait (TMA-fed kernels)
     int test_flags;       // decode kernel test hooks (0 outside the tests)
 };
@@ -134,6 +135,7 @@ struct det_linear_plan {
     int test_flags;
     // the decode tiling chosen for this plan (schedule only; cached so that a run does no search)
     detlin::DecodeConfig decode_cfg;
+    int any_layout;                  // decode for any K: the layout chosen (decode_any.cu), 0 = none yet
     int decode_cfg_variant;          // variant the cached tiling was chosen for, -1 = none yet
     // tensor-map cache for the decode kernel (keyed by the pointers they were built for)
     const void* map_w_ptr;

@@ -50,3 +50,15 @@ def test_padding_changes_no_accumulator():
     want, got = oracle_y(x, W, None), run_gpu(x, W, None, kernel=KERNEL_GENERIC)
     assert np.array_equal(np.isnan(got), np.isnan(want))
     assert_bits_equal(np.nan_to_num(got, nan=0.0, posinf=1.0), np.nan_to_num(want, nan=0.0, posinf=1.0), "special values")
+
+
+# small layers: batch blocks of fewer rows than there are, a warp for each of a row's two segments, a second segment of one chunk, a
+# last block of one row, the largest K that one block holds
+@pytest.mark.parametrize("M,N,K", [(6, 1333, 1001), (7, 250, 3001), (2, 3, 257), (1, 65, 385), (5, 129, 511), (13, 30, 4095), (30, 64, 1501),
+                                   (3, 17, 13999), (1, 9, 55001), (64, 60, 4001)])
+@pytest.mark.parametrize("wfmt", ["bf16", "fp16", "fp32"])
+def test_small_layers(M, N, K, wfmt):
+    x, W, b = inputs.make_case_w(M, N, K, wfmt)
+    want = oracle_y(x, W, b)
+    assert_bits_equal(run_gpu(x, W, b, kernel=KERNEL_GENERIC), want, f"{M},{N},{K} {wfmt}")
+    assert_bits_equal(run_gpu(x, W, b, kernel=KERNEL_GENERIC, max_blocks=2), want, "two blocks")
