@@ -23,18 +23,33 @@ const DecodeClassTable* class_table(int wfmt, int cls)
 
 int m_class(int64_t M) { return M <= 1 ? 0 : M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 3 : M <= 16 ? 4 : 5; }
 
-// Predicted time of a tiling in SM clock cycles (schedule heuristic; its constants were fitted to sweeps of
-// every tiling over the Llama-3-8B shapes at batch 1 .. 32 on a 148-SM B200, mean loss against the best
-// tiling 0.5 %).  A work unit streams rb weight rows (2 K bytes each, at the SM's share of the HBM rate)
-// and performs rb * mb * K multiply-adds at the FMA rate of an SM times an efficiency that depends on the
-// warp tile; whichever is larger binds.  Units resident on one SM share it.  Fewer than eight consumer
-// warps per SM hide latency badly; every unit pays for its lane trees (one per segment) and, with several
-// segment groups, for the fold through shared memory.  FP32 weights have rates of their own (fitted to sweeps of 52 shapes at
-// batch 1 .. 64, mean loss against the best tiling 2 %; with the rates of the 16-bit formats 24 %): their multiply loop is another
-// one in the larger tiles, which blocks of four consumer warps compile with a few spilled registers.
+// Predicted time of a tiling in SM clock cycles (schedule heuristic).  A work unit streams rb weight rows (at the SM's share of the
+// HBM rate) and performs rb * mb * K multiply-adds at the FMA rate of an SM times an efficiency that depends on the warp tile;
+// whichever is larger binds.  Units resident on one SM share it.  Fewer than eight consumer warps per SM hide latency badly; every
+// unit pays for its lane trees (one per segment) and, with several segment groups, for the fold through shared memory.
+// The rates were fitted to sweeps of every tiling on a 148-SM B200.  16-bit weights, up to 8 rows: the Llama-3-8B shapes, mean loss against
+// the best tiling 0.5 %.  More rows: 56 drawn and layer shapes, 9 to 64 rows, mean loss 2 % (3.5 % with the rates of few rows: M = 16, N =
+// 4096, K = 14336 44.5 -> 41.6 us, M = 16, N = 2083, K = 14096 49.8 -> 42.6, M = 17, N = 432, K = 5416 11.5 -> 10.5);
+// from K = 2560 on: short rows are a matter of latencies that this does not know (M = 16, N = 278, K = 2168 5.6 us, with the rates of few rows 4.8).  FP32 weights: 52 shapes at
+// batch 1 .. 64, 2 % (24 % with those of 16 bits): their multiply loop is another one in the larger tiles (Cfg::kPipelined).
+struct TilingRates {
+    double eff8, eff4, eff2, eff1;       // share of the FMA rate by batch rows of a warp tile
+    double wide, narrow;                 // ... times: 8-row tiles with half as many stage boundaries (KC 512); stages of 128
+    double small8, small4;               // ... times: blocks of at most four consumer warps
+    double hbm;                          // bytes per clock and SM
+    double other;                        // share of the term that does not bind
+    double latency;                      // exponent of 8 / warps
+    double tree, fold;                   // cycles per segment of a full tile; with several segment groups
+    double part, part_exp;               // a last tile of the share p of a tile's rows takes part * p ^ part_exp of its time
+};
+constexpr TilingRates kRatesFewRows = {0.707, 0.70, 0.345, 0.2, 1.2, 0.9, 1.0, 1.0, 22.5, 0.0, 1.0, 1020.0, 1500.0, 1.08, 1.0};
+constexpr TilingRates kRatesManyRows = {0.922, 0.844, 0.420, 0.141, 1.057, 0.9, 0.96, 0.973, 27.0, 0.0264, 1.703, 799.0, 1384.0, 0.7355, 0.567};
+constexpr TilingRates kRatesFp32 = {0.52, 0.43, 0.49, 0.075, 1.0, 1.0, 0.904, 0.558, 32.0, 0.0, 1.0, 1020.0, 1500.0, 1.08, 1.0};
+
 double tiling_cost(const DecodeEntry& e, int wfmt, int64_t M, int64_t N, int64_t K, int S, int sm_count)
 {
     const DecodeConfig& c = e.cfg;
+    const TilingRates& t = wfmt == DET_WEIGHT_FP32 ? kRatesFp32 : M > 8 && K >= 2560 ? kRatesManyRows : kRatesFewRows;
     const int occ = e.occupancy(S);
     if (occ <= 0) return 1e300;
     const int64_t rb = (int64_t)c.rt * c.wr, mb = (int64_t)c.mt * c.wm;
@@ -44,25 +59,22 @@ double tiling_cost(const DecodeEntry& e, int wfmt, int64_t M, int64_t N, int64_t
     const int64_t per_sm = (units + sm_count - 1) / sm_count;
     const double resident = (double)(per_sm < occ ? per_sm : occ);
     const double warps = resident * c.wm * c.wr * c.sk;
-    double eff = c.mt >= 8 ? 0.707 : c.mt == 4 ? 0.70 : c.mt == 2 ? 0.345 : 0.2;
-    if (c.kc >= 512 && c.mt >= 8) eff *= 1.2;          // half as many stage boundaries; smaller tiles prefer a deeper ring
-    if (c.kc <= 128) eff *= 0.9;
-    double row_bytes = (double)K * 2.0, hbm_rate = 22.5;
-    if (wfmt == DET_WEIGHT_FP32) {
-        const bool small = c.wm * c.wr * c.sk <= 4;
-        eff = c.mt >= 8 ? (small ? 0.47 : 0.52) : c.mt == 4 ? (small ? 0.24 : 0.43) : c.mt == 2 ? 0.49 : 0.075;
-        row_bytes = (double)K * 4.0;
-        hbm_rate = 32.0;
-    }
-    const double latency = warps >= 8.0 ? 1.0 : 8.0 / warps;
+    const bool small = c.wm * c.wr * c.sk <= 4;
+    double eff = c.mt >= 8 ? t.eff8 : c.mt == 4 ? t.eff4 : c.mt == 2 ? t.eff2 : t.eff1;
+    if (c.kc >= 512 && c.mt >= 8) eff *= t.wide;
+    if (c.kc <= 128) eff *= t.narrow;
+    if (small && c.mt >= 8) eff *= t.small8;
+    if (small && c.mt == 4) eff *= t.small4;
+    const double latency = warps >= 8.0 ? 1.0 : pow(8.0 / warps, t.latency);
     const double fma = (double)rb * (double)mb * (double)K / 128.0 / eff * resident;
-    // weights from HBM at 22.5 bytes per clock and SM (FP32 32); the unit's activations come again from L2 for every unit
-    const double hbm = ((double)rb * row_bytes / hbm_rate + 0.06 * (double)mb * (double)K * 4.0 / 64.0) * resident;
-    const double body = (fma > hbm ? fma : hbm) * latency;
-    const double overhead = (double)S * 1020.0 * ((double)(mb * rb) / 896.0) + (c.sk > 1 ? 1500.0 : 0.0);
+    // weights from HBM; the unit's activations come again from L2 for every unit
+    const double row_bytes = (double)K * (wfmt == DET_WEIGHT_FP32 ? 4.0 : 2.0);
+    const double hbm = ((double)rb * row_bytes / t.hbm + 0.06 * (double)mb * (double)K * 4.0 / 64.0) * resident;
+    const double body = ((fma > hbm ? fma : hbm) + t.other * (fma > hbm ? hbm : fma)) * latency;
+    const double overhead = (double)S * t.tree * ((double)(mb * rb) / 896.0) + (c.sk > 1 ? t.fold : 0.0);
     if ((rb >= 56 && mb >= 16) || rb >= 112) {
-        // what is left after whole rounds is dealt out by row groups (Cfg::kDealRest); half a tile takes a little longer than
-        // half the time (one warp per scheduler)
+        // what is left after whole rounds is dealt out by row groups (Cfg::kDealRest); part of a tile takes longer than its
+        // share of the time (one warp per scheduler)
         int64_t shares = (int64_t)sm_count * occ / mblocks;
         const int64_t groups = (N + c.rt - 1) / c.rt;
         shares = shares < 1 ? 1 : shares > groups ? groups : shares;
@@ -71,7 +83,7 @@ double tiling_cost(const DecodeEntry& e, int wfmt, int64_t M, int64_t N, int64_t
         // tiles of 112 rows only for many rounds: M = 7, N = 50000, K = 2048 (3.02 rounds) 45.9 us, by 56 rows 44.1; M = 8, N = 28672,
         // K = 4096 (1.7 rounds) 50.5 and 50.1; N = 128256 (7.7 rounds) 181.4 and 184.8
         if (rb >= 112 && whole < 5) return 1e300;
-        if (whole > 0) return (double)whole * (body + overhead) + (part < 1.0 ? part * 1.08 : 1.0) * body + (rest ? overhead : 0.0);
+        if (whole > 0) return (double)whole * (body + overhead) + (part < 1.0 ? t.part * pow(part, t.part_exp) : 1.0) * body + (rest ? overhead : 0.0);
     }
     return (double)rounds * (body + overhead);
 }
