@@ -73,7 +73,12 @@ cudaError_t launch_h(const LaunchArgs& a, int width, const CUtensorMap* map_w, c
     case 256: return launch_t<WF, 2 * TM, 8, 32, 8, DET_PLAIN>(a, map_w, map_x);
     case 128: return launch_t<WF, 8, 8, 16, 2 * TM, DET_PLAIN>(a, map_w, map_x);
     case 64: return launch_t<WF, 4, 8, 8, 4 * TM, DET_PLAIN>(a, map_w, map_x);
-    case 32: return launch_t<WF, 4, 4, 8, 4 * TM, DET_PLAIN>(a, map_w, map_x);
+    case 32:
+        // 128 rows: one multiplying warp a scheduler with 8 x 4 outputs a thread (three loads per 16 packed FMAs) beats two with 4 x 4
+        // (two per 8): 128 x 1000 x 1000 13.45 -> 12.35 us, 120 x 700 x 512 12.4 -> 11.5.  At 96 rows three such warps lose as often
+        // (96 x 1000 x 1000 11.85 -> 11.80, 90 x 64 x 4096 13.0 -> 14.2).
+        if constexpr (TM == 8) return launch_t<WF, 8, 4, 8, 2 * TM, DET_PLAIN>(a, map_w, map_x);
+        else return launch_t<WF, 4, 4, 8, 4 * TM, DET_PLAIN>(a, map_w, map_x);
     default: return cudaErrorInvalidValue;
     }
 }
