@@ -27,6 +27,10 @@ DET_API det_status_t det_test_plan_set_max_blocks(det_linear_plan_t* plan, int m
  * changes. DET_ERR_INVALID_ARG if the variant does not exist for this plan. */
 DET_API det_status_t det_test_plan_set_variant(det_linear_plan_t* plan, int variant);
 
+/* How often calls of this thread searched for a decode tiling or for a layout of decode with any K.  A program that repeats its
+ * calls searches once: with the plan or, of the TMA-fed kernel's tiling, in the plan's first run. */
+DET_API int64_t det_test_schedule_searches(void);
+
 /*
  * Host-side fault injection: make the nth device allocation the library attempts from now on (1 = the
  * next one) fail once with an out-of-memory error, without touching the device; 0 switches the hook

@@ -90,6 +90,8 @@ def lib() -> ctypes.CDLL:
         u32, u64 = ctypes.c_uint, ctypes.c_uint64
         L.det_test_kernels_reach.argtypes = [u32, u32, u64, u64, u64, u64, u64]
         L.det_test_kernels_reach.restype = i32
+        L.det_test_schedule_searches.argtypes = []
+        L.det_test_schedule_searches.restype = i64
         L.det_test_fail_next_alloc.argtypes = [i32]
         L.det_test_fail_next_alloc.restype = None
         L.det_test_plan_set_wait.argtypes = [p, ctypes.c_uint64, i32]
@@ -403,6 +405,11 @@ def det_test_attention_set_split(blocks_per_row: int) -> None:
 def det_test_kernels_reach(memory_type: int, managed: int, device_address: int, range_start: int, range_bytes: int, host: int, nbytes: int) -> bool:
     """May kernels touch the host buffer [host, host + nbytes), given what the driver says about its first byte?  Host arithmetic only."""
     return bool(lib().det_test_kernels_reach(memory_type, managed, device_address, range_start, range_bytes, host, nbytes))
+
+
+def det_test_schedule_searches() -> int:
+    """Searches for a decode tiling or layout that calls of this thread have made."""
+    return int(lib().det_test_schedule_searches())
 
 
 def det_test_fail_next_alloc(nth: int = 1) -> None:

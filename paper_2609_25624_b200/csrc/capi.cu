@@ -58,6 +58,9 @@ static bool encode_2d(CUtensorMap* map, CUtensorMapDataType dt, int elem_bytes, 
     return true;
 }
 
+static thread_local int64_t g_schedule_searches = 0;
+void count_schedule_search() { ++g_schedule_searches; }
+
 // Device allocation with the test hook of det_test_fail_next_alloc: the next `skip`-th call fails once
 // with cudaErrorMemoryAllocation without touching the device.
 static int g_fail_alloc_countdown = 0;          // 0 = off; n = the n-th allocation from now fails
@@ -105,7 +108,6 @@ det_status_t run_device(det_linear_plan_t* plan, const float* x, const void* W, 
     a.sm_count = plan->sm_count;
     a.max_blocks = plan->max_blocks;
     a.variant = plan->variant;
-    a.any_layout = &plan->any_layout;
 
     int kernel = plan->forced_kernel >= 0 ? plan->forced_kernel : p.kernel;
     const int64_t k_align = p.weight_format == DET_WEIGHT_FP32 ? 4 : 8;     // 16-byte row pitch of W (x: K % 4)
@@ -168,6 +170,9 @@ det_status_t run_device(det_linear_plan_t* plan, const float* x, const void* W, 
             e = launch_prefill_tma(a, tm, width, &plan->map_w, &plan->map_x);
         }
     } else {
+        if (p.bucket == 0 && plan->any_layout.mt == 0)         // (plans on the stack of a call; others have theirs from the start)
+            plan->any_layout = any_layout_for(p.M, plan->n_count, p.K, p.S, p.weight_format, plan->sm_count);
+        a.any_layout = plan->any_layout;
         e = launch_generic(a, p.bucket);
     }
     if (e != cudaSuccess) return cuda_fail("kernel launch", e);
@@ -234,6 +239,8 @@ det_linear_plan_t* det_linear_plan_shard(int64_t M, int64_t N, int64_t K, int64_
     plan->map_cfg_id = -1;
     plan->decode_cfg_variant = -1;
     plan->wait_limit_ns = kDefaultWaitLimitNs;
+    // (for any buffers: those of a run may turn out to be misaligned)
+    if (prm.bucket == 0) plan->any_layout = any_layout_for(M, n_count, K, prm.S, wfmt, sms);
     g_last_status = DET_OK;
     e = device_alloc(reinterpret_cast<void**>(&plan->status), sizeof(DeviceStatus));
     if (e == cudaSuccess) e = cudaMemset(plan->status, 0, sizeof(DeviceStatus));
@@ -290,7 +297,8 @@ det_status_t det_linear_run_w(const det_linear_plan_t* plan, const float* x, con
                               void* stream)
 {
     if (!plan || !x || !W || !y) { set_error("run: plan, x, W and y must not be NULL"); return DET_ERR_INVALID_ARG; }
-    // the plan's tensor-map cache is the only state a run touches
+    // what a run touches: the cache of tensor maps and, once, the tiling of the TMA-fed decode kernel.  Decode for any K and alignment
+    // has its layout from the start and writes nothing.
     return run_device(const_cast<det_linear_plan_t*>(plan), x, W, b, y, static_cast<cudaStream_t>(stream));
 }
 
@@ -649,6 +657,8 @@ det_status_t det_test_plan_set_variant(det_linear_plan_t* plan, int variant)
     plan->variant = variant;
     return DET_OK;
 }
+
+int64_t det_test_schedule_searches(void) { return g_schedule_searches; }
 
 void det_test_attention_set_split(int blocks_per_row) { attention_test_force_split(blocks_per_row); }
 

@@ -16,7 +16,7 @@
 //     -0.0 one), so elements beyond K are skipped in effect without a test in the loop;
 //   * two rows' chains advance in one packed FMA (RT > 1), the lane sums of all outputs fold in one butterfly.
 //   * a small layer is one wave of warps that wait for their own instructions: batch blocks of fewer rows and a warp per segment
-//     spread them over the SMs (choose_layout).
+//     spread them over the SMs (decode_any_layout.cpp).
 // Measured on B200, us a call in a chain (in brackets a warp per row that walks it chunk by chunk, for every batch row again): M = 6, N =
 // 1333, K = 1001 4.7 (15.8); M = 3, N = K = 4097 14.3 (49.6); M = 64, N = 8192, K = 4097 218 (1705; 27 % of the FP32 peak: line-up and
 // widening of every weight in every batch block, one-word loads); M = 64, N = 300, K = 333 4.6 (68).
@@ -26,10 +26,6 @@
 namespace detlin {
 
 namespace {
-
-constexpr int kAnySmemBytes = 110 * 1024;            // activations of one window of K with two blocks of 8 warps per SM ...
-constexpr int kAnySmemBytes1 = 220 * 1024;           // ... or one block of 16
-constexpr int kSplitBytes = 8 * 32 * 4;              // SPLIT: the second segments' sums, one a lane
 
 // SPLIT: the two segments of a row belong to two warps, the second half of the block's warps to the second ones.
 template <int WF, int MT, int RT, bool SPLIT>
@@ -265,7 +261,7 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
 }
 
 template <int WF, int MT, int RT, bool SPLIT>
-cudaError_t launch_t(const LaunchArgs& a, long long mblocks, int sms)
+cudaError_t launch_t(const LaunchArgs& a, int sms)
 {
     static bool configured[kMaxDevices];             // function attributes belong to a device
     int dev = 0;
@@ -278,92 +274,35 @@ cudaError_t launch_t(const LaunchArgs& a, long long mblocks, int sms)
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    // Two blocks of 8 warps per SM, or one of 16 where only that keeps all activations of a batch block in shared memory; the
-    // window holds whole chunks of 128.
-    const long long padded = (a.K + 127) / 128 * 128, cap = kAnySmemBytes / 4 / MT / 256 * 256, cap1 = kAnySmemBytes1 / 4 / MT / 256 * 256;
-    const bool big = SPLIT || padded > cap;
-    const int warps = big ? 16 : 8, row_warps = SPLIT ? 8 : warps;
-    const unsigned win = (unsigned)(!big ? padded : padded < cap1 ? padded : cap1);
-    const long long groups = (a.N + row_warps * RT - 1) / (row_warps * RT);
-    long long grid = (big ? 1ll : 2ll) * sms / mblocks;
-    if (grid < 1) grid = 1;
-    if (a.max_blocks > 0 && grid > a.max_blocks) grid = a.max_blocks;
-    if (grid > groups) grid = groups;
+    const AnyGrid g = any_grid({MT, RT, SPLIT}, a.M, a.N, a.K, sms);
+    const unsigned win = (unsigned)g.window;
+    const int64_t grid = a.max_blocks > 0 && g.blocks_x > a.max_blocks ? a.max_blocks : g.blocks_x;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
-    cfg.gridDim = dim3((unsigned)grid, (unsigned)mblocks);
-    cfg.blockDim = dim3(32 * warps);
-    cfg.dynamicSmemBytes = (size_t)MT * win * 4 + (SPLIT ? kSplitBytes : 0);
+    cfg.gridDim = dim3((unsigned)grid, (unsigned)g.batch_blocks);
+    cfg.blockDim = dim3(32 * g.warps);
+    cfg.dynamicSmemBytes = (size_t)MT * win * 4 + (SPLIT ? kAnySplitBytes : 0);
     cfg.stream = a.stream;
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, a.x, static_cast<const typename WeightElem<WF>::type*>(a.W), a.b, a.y, (int)a.M, (int)a.N,
-                              (unsigned)a.K, (unsigned)a.seg_len, (long long)a.ldy, win, (int)groups);
-}
-
-// How a call is laid out: batch rows and weight rows of a warp, and whether two warps share a row's two segments (in sixteen-warp
-// blocks that hold all of K and run all at once).
-struct Layout { int mt, rt; bool split; };
-
-// Predicted cycles of a layout: instructions of a warp (operands, line-up and multiplications of its chunks, its part of the
-// activations, lane trees), at the rate of a lone warp or of the SM's schedulers, whichever is slower.  Constants fitted to every layout
-// of 68 drawn shapes (M 1 .. 64, N 64 .. 60000, K 101 .. 9001): mean loss against the best layout 2 %.
-double layout_cost(const LaunchArgs& a, int wfmt, const Layout& l, int sms)
-{
-    const long long padded = (a.K + 127) / 128 * 128, cap = kAnySmemBytes / 4 / l.mt / 256 * 256, cap1 = kAnySmemBytes1 / 4 / l.mt / 256 * 256;
-    const bool big = l.split || padded > cap;
-    const long long warps = big ? 16 : 8, row_warps = l.split ? 8 : warps, occ = big ? 1 : 2;
-    const long long win = !big ? padded : padded < cap1 ? padded : cap1;
-    const long long groups = (a.N + row_warps * l.rt - 1) / (row_warps * l.rt), mblocks = (a.M + l.mt - 1) / l.mt;
-    long long gx = occ * sms / mblocks;
-    gx = gx < 1 ? 1 : gx > groups ? groups : gx;
-    const long long blocks = gx * mblocks, per_sm = (blocks + sms - 1) / sms;
-    if (l.split && (blocks > sms || l.mt >= 8 || padded * 4 * l.mt + kSplitBytes > kAnySmemBytes1)) return 1e300;
-    const double iters = (double)((groups + gx - 1) / gx), waves = (double)((blocks + occ * sms - 1) / (occ * sms));
-    const double chunks = (double)padded / 128 / (l.split ? 2 : 1);
-    double per_chunk = l.mt * (2 + (l.rt == 1 ? 4 : 2 * l.rt));
-    if (l.mt * l.rt >= 32) per_chunk *= 1.31;        // registers run out
-    per_chunk += 6.4 + l.rt * (wfmt == 2 ? 14.6 : 11.6);
-    const double body = chunks * per_chunk + 1.34 * l.mt * l.rt * (l.split ? 1 : 2) + 254;
-    const double stage = 9.0 * l.mt * (double)win / (32.0 * warps) * (win >= padded ? 1.0 : (double)((padded + win - 1) / win) * iters);
-    const double shared = (double)(warps * (per_sm < occ ? per_sm : occ)) / 4 * 1.08;
-    return (l.split && l.rt == 4 ? 1.2 : 1.0) * waves * ((body * iters + stage) * (shared > 3.94 ? shared : 3.94) + 546);
-}
-
-// Fewer batch rows a warp than there are, where the layer leaves SMs idle otherwise (the weights then come from L2 for the other batch
-// blocks): M = 6, N = 1333, K = 1001 6.1 -> 4.7 us, M = 7, N = 250, K = 3001 with FP32 weights 10.1 -> 5.8; a warp a segment: M = 8, N = 64,
-// K = 4095 19.5 -> 6.8.  The largest batch block with one, two or four rows by the number of warps, the rule without this, keeps the calls
-// that would not gain 3 %.
-Layout choose_layout(const LaunchArgs& a, int wfmt, int sms)
-{
-    const int most = a.M <= 1 ? 1 : a.M <= 2 ? 2 : a.M <= 4 ? 4 : 8;
-    const long long rows = a.N * ((a.M + most - 1) / most);
-    Layout best{most, rows >= 4ll * 8 * sms ? 4 : rows >= 2ll * 4 * sms ? 2 : 1, false};
-    double best_cost = 0.97 * layout_cost(a, wfmt, best, sms);
-    for (int mt = most; mt >= 1 && 16 * mt >= a.M; mt /= 2)
-        for (int rt = 1; rt <= 4; rt *= 2)
-            for (int split = 0; split <= (a.S == 2 && mt < 8 ? 1 : 0); ++split) {
-                const Layout l{mt, rt, split != 0};
-                const double c = layout_cost(a, wfmt, l, sms);
-                if (c < best_cost) { best_cost = c; best = l; }
-            }
-    return best;
+                              (unsigned)a.K, (unsigned)a.seg_len, (long long)a.ldy, win, (int)g.groups);
 }
 
 template <int WF, int MT>
-cudaError_t launch_m(const LaunchArgs& a, const Layout& l, int sms)
+cudaError_t launch_m(const LaunchArgs& a, int sms)
 {
-    const long long mblocks = (a.M + MT - 1) / MT;
+    const AnyLayout& l = a.any_layout;
     if constexpr (MT < 8) {
         if (l.split) {
-            if (l.rt == 4) return launch_t<WF, MT, 4, true>(a, mblocks, sms);
-            return l.rt == 2 ? launch_t<WF, MT, 2, true>(a, mblocks, sms) : launch_t<WF, MT, 1, true>(a, mblocks, sms);
+            if (l.rt == 4) return launch_t<WF, MT, 4, true>(a, sms);
+            return l.rt == 2 ? launch_t<WF, MT, 2, true>(a, sms) : launch_t<WF, MT, 1, true>(a, sms);
         }
     }
-    if (l.rt == 4) return launch_t<WF, MT, 4, false>(a, mblocks, sms);
-    return l.rt == 2 ? launch_t<WF, MT, 2, false>(a, mblocks, sms) : launch_t<WF, MT, 1, false>(a, mblocks, sms);
+    if (l.rt == 4) return launch_t<WF, MT, 4, false>(a, sms);
+    return l.rt == 2 ? launch_t<WF, MT, 2, false>(a, sms) : launch_t<WF, MT, 1, false>(a, sms);
 }
 
 }  // namespace
@@ -373,19 +312,12 @@ cudaError_t launch_m(const LaunchArgs& a, const Layout& l, int sms)
 cudaError_t DET_CAT(launch_decode_any_wf, DET_WF)(const LaunchArgs& a)
 {
     const int sms = a.sm_count > 0 ? a.sm_count : 148;
-    // a plan keeps the choice: mt + 16 rt + 256 split
-    int code = a.any_layout ? *a.any_layout : 0;
-    if (code == 0) {
-        const Layout l = choose_layout(a, DET_WF, sms);
-        code = l.mt + 16 * l.rt + 256 * (l.split ? 1 : 0);
-        if (a.any_layout) *a.any_layout = code;
-    }
-    const Layout l{code & 15, (code >> 4) & 15, code >= 256};
-    switch (l.mt) {
-    case 1: return launch_m<DET_WF, 1>(a, l, sms);
-    case 2: return launch_m<DET_WF, 2>(a, l, sms);
-    case 4: return launch_m<DET_WF, 4>(a, l, sms);
-    default: return launch_m<DET_WF, 8>(a, l, sms);
+    if (!any_layout_fits(a.any_layout, a.K, a.S)) return cudaErrorInvalidValue;
+    switch (a.any_layout.mt) {
+    case 1: return launch_m<DET_WF, 1>(a, sms);
+    case 2: return launch_m<DET_WF, 2>(a, sms);
+    case 4: return launch_m<DET_WF, 4>(a, sms);
+    default: return launch_m<DET_WF, 8>(a, sms);
     }
 }
 

@@ -33,6 +33,23 @@ constexpr int kMaxDevices = 64;     // per-device caches (function attributes, s
 void set_error(const char* fmt, ...);
 det_status_t fill_params(int64_t M, int64_t N, int64_t K, det_linear_params_t* out);
 
+// Decode for any K: batch rows and weight rows of a warp, and whether two warps share a row's two segments (in sixteen-warp blocks that
+// hold all of K).  mt = 0: none chosen yet.
+struct AnyLayout { int mt, rt, split; };
+struct AnyGrid {
+    int warps, row_warps, blocks_per_sm;         // warps of a block, those of them that have rows of their own
+    int64_t window;                              // k elements of the activations in shared memory
+    int64_t groups, batch_blocks, blocks_x;      // blocks_x thread blocks walk the row groups of each batch block
+};
+constexpr int kAnySmemBytes = 110 * 1024;        // activations of one window of K with two blocks of 8 warps per SM ...
+constexpr int kAnySmemBytes1 = 220 * 1024;       // ... or one block of 16
+constexpr int kAnySplitBytes = 8 * 32 * 4;       // split: the second segments' sums, one a lane
+AnyGrid any_grid(const AnyLayout& l, int64_t M, int64_t N, int64_t K, int sm_count);
+bool any_layout_fits(const AnyLayout& l, int64_t K, int S);
+AnyLayout any_layout_for(int64_t M, int64_t N, int64_t K, int S, int wfmt, int sm_count);
+// Searches for a layout or a tiling made by the calling thread (det_test_schedule_searches).
+void count_schedule_search();
+
 // ---- kernel launchers (defined in the .cu files) -------------------------------------------
 struct LaunchArgs {
     const float* x;
@@ -54,7 +71,7 @@ struct LaunchArgs {
     int sm_count;
     int max_blocks;       // 0 = automatic
     int variant;          // 0 = automatic
-    int* any_layout;      // decode for any K: the layout that a plan keeps (0: none yet), or nullptr
+    AnyLayout any_layout; // decode for any K
     unsigned long long wait_limit_ns;   // bound of one device-side wait (TMA-fed kernels)
     int test_flags;       // decode kernel test hooks (0 outside the tests)
 };
@@ -135,7 +152,7 @@ struct det_linear_plan {
     int test_flags;
     // the decode tiling chosen for this plan (schedule only; cached so that a run does no search)
     detlin::DecodeConfig decode_cfg;
-    int any_layout;                  // decode for any K: the layout chosen (decode_any.cu), 0 = none yet
+    detlin::AnyLayout any_layout;    // decode for any K and alignment: likewise, chosen with the plan
     int decode_cfg_variant;          // variant the cached tiling was chosen for, -1 = none yet
     // tensor-map cache for the decode kernel (keyed by the pointers they were built for)
     const void* map_w_ptr;

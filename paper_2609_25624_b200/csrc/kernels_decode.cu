@@ -118,6 +118,7 @@ bool decode_config_for(int64_t M, int64_t N, int64_t K, int S, int wfmt, int var
     if (variant < 0 || S < 1 || S > kDecodeMaxSegments) return false;
     int sms = 148;
     if (variant == 0) {
+        count_schedule_search();
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)

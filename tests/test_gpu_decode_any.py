@@ -62,3 +62,20 @@ def test_small_layers(M, N, K, wfmt):
     want = oracle_y(x, W, b)
     assert_bits_equal(run_gpu(x, W, b, kernel=KERNEL_GENERIC), want, f"{M},{N},{K} {wfmt}")
     assert_bits_equal(run_gpu(x, W, b, kernel=KERNEL_GENERIC, max_blocks=2), want, "two blocks")
+
+
+@pytest.mark.parametrize("M,N,K,offset", [(6, 1333, 1001, 0), (3, 200, 640, 1)])
+def test_runs_of_a_plan_search_for_nothing(M, N, K, offset):
+    """Runs take a const plan: what is chosen for any K and alignment is chosen with the plan."""
+    x, W, b = inputs.make_case(M, N, K)
+    xd, bd, y = x.cuda(), b.cuda(), torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
+    Wd = torch.empty(N * K + offset, dtype=W.dtype, device="cuda")[offset:].view(N, K)
+    Wd.copy_(W)
+    plan = B.det_linear_plan(M, N, K)
+    before = B.det_test_schedule_searches()
+    for _ in range(3):
+        B.det_linear_run(plan, xd, Wd, bd, y)
+    B.det_linear_plan_check(plan)
+    plan.close()
+    assert B.det_test_schedule_searches() == before
+    assert_bits_equal(y.cpu().numpy(), oracle_y(x, W, b), f"{M},{N},{K} + {offset}")
