@@ -53,12 +53,30 @@ static cudaError_t static_addresses(int dev, NoallocAddresses* out)
 static unsigned long long g_wait_limit_ns = kDefaultWaitLimitNs;
 static int g_test_flags = 0;
 
-// The decode tiling depends on the shape and the device only; a loop that repeats a shape does not search again.
-static thread_local struct {
-    int64_t M, N, K;
+// The decode schedule depends on the shape and the device only: a loop that repeats its shapes searches once for each.  A search for a
+// layout (any K, any alignment) takes 0.7 us of the host, one for a tiling more; sixteen entries hold the projections of a few
+// kinds of layer at two batch sizes.
+struct NoallocSchedule {
+    int64_t M, N, K;                 // M = 0: empty
     int dev;
+    bool tiled;                      // cfg is valid
     DecodeConfig cfg;
-} g_last_tiling;
+    AnyLayout layout;                // mt = 0: none yet
+};
+constexpr int kNoallocSchedules = 16;
+static thread_local NoallocSchedule g_schedules[kNoallocSchedules];
+static thread_local int g_next_schedule = 0;
+
+static NoallocSchedule& schedule_of(int64_t M, int64_t N, int64_t K, int dev)
+{
+    for (NoallocSchedule& s : g_schedules)
+        if (s.M == M && s.N == N && s.K == K && s.dev == dev) return s;
+    NoallocSchedule& s = g_schedules[g_next_schedule];
+    g_next_schedule = (g_next_schedule + 1) % kNoallocSchedules;
+    s = NoallocSchedule{};
+    s.M = M; s.N = N; s.K = K; s.dev = dev;
+    return s;
+}
 
 }  // namespace detlin
 
@@ -110,16 +128,18 @@ extern "C" det_status_t det_linear_run_noalloc(int64_t M, int64_t N, int64_t K, 
     plan.test_flags = kFlagLateWeights | g_test_flags;                     // nothing was said here about W and b being older than the stream's last kernel
     plan.decode_cfg_variant = -1;
     plan.map_cfg_id = -1;
-    auto& t = g_last_tiling;
-    const bool decode = p.kernel == kKernelDecode;
-    if (decode && t.M == M && t.N == N && t.K == K && t.dev == dev) {
-        plan.decode_cfg = t.cfg;
+    if (p.bucket != 0) return run_device(&plan, x, W, b, y, static_cast<cudaStream_t>(stream));
+    NoallocSchedule& s = schedule_of(M, N, K, dev);
+    if (s.tiled) {
+        plan.decode_cfg = s.cfg;
         plan.decode_cfg_variant = 0;
     }
+    plan.any_layout = s.layout;
     st = run_device(&plan, x, W, b, y, static_cast<cudaStream_t>(stream));
-    if (st == DET_OK && decode && plan.decode_cfg_variant == 0) {
-        t.M = M; t.N = N; t.K = K; t.dev = dev;
-        t.cfg = plan.decode_cfg;
+    if (st == DET_OK) {
+        s.tiled = plan.decode_cfg_variant == 0;
+        s.cfg = plan.decode_cfg;
+        s.layout = plan.any_layout;
     }
     return st;
 }

@@ -70,6 +70,24 @@ def test_noalloc_rejects_shapes_beyond_the_builtin_scratch():
     assert rc == 1
 
 
+def test_noalloc_searches_once_for_each_shape():
+    """A loop over several shapes and alignments, as a model's layers make it, chooses each call's schedule in the first pass only."""
+    calls = []
+    for M, N, K, offset in [(5, 300, 1001, 0), (3, 512, 768, 0), (3, 512, 768, 1), (7, 250, 3001, 0), (3, 512, 1024, 0)]:
+        x, W, b = inputs.make_case(M, N, K)
+        Wd = torch.empty(N * K + offset, dtype=W.dtype, device="cuda")[offset:].view(N, K)
+        Wd.copy_(W)
+        calls.append((x.cuda(), Wd, b.cuda(), torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda"), oracle_y(x, W, b)))
+    for passes in range(3):
+        before = B.det_test_schedule_searches()
+        for x, W, b, y, _ in calls:
+            y.fill_(float("nan"))
+            B.det_linear_run_noalloc(x, W, b, y)
+        assert passes == 0 or B.det_test_schedule_searches() == before
+        for i, (_, _, _, y, want) in enumerate(calls):
+            assert_bits_equal(y.cpu().numpy(), want, f"call {i}, pass {passes}")
+
+
 @pytest.mark.parametrize("M,N,K", [(64, 520, 1024), (1, 20000, 264), (65, 300, 40), (100, 1000, 1000), (3000, 9000, 256)])
 def test_noalloc_fast_kernels_with_weights_written_just_before(M, N, K):
     """The kernels of the planned path, on aligned buffers: decode with and without a split, prefill with one unit per
