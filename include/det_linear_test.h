@@ -24,7 +24,9 @@ DET_API det_status_t det_test_plan_force_kernel(det_linear_plan_t* plan, int ker
 DET_API det_status_t det_test_plan_set_max_blocks(det_linear_plan_t* plan, int max_blocks);
 
 /* Select a tile configuration variant of the plan's kernel (0 = automatic). Only the schedule
- * changes. DET_ERR_INVALID_ARG if the variant does not exist for this plan. */
+ * changes. DET_ERR_INVALID_ARG if the variant does not exist for this plan.  Decode plans: 1, 2, ... are the tilings of the
+ * TMA-fed kernel; 100 mt + 10 rt + split is a layout of decode for any K (mt batch rows x rt weight rows a warp; split = 1: two
+ * warps share a row's two segments) and leaves the tiling automatic. */
 DET_API det_status_t det_test_plan_set_variant(det_linear_plan_t* plan, int variant);
 
 /* How often calls of this thread searched for a decode tiling or for a layout of decode with any K.  A program that repeats its

@@ -644,6 +644,18 @@ det_status_t det_test_plan_set_variant(det_linear_plan_t* plan, int variant)
 {
     if (!plan || variant < 0) { set_error("set_variant: bad argument"); return DET_ERR_INVALID_ARG; }
     if (plan->prm.bucket == 0) {
+        const det_linear_params_t& p = plan->prm;
+        AnyLayout layout = any_layout_for(p.M, plan->n_count, p.K, p.S, p.weight_format, plan->sm_count);
+        if (variant >= 100) {
+            layout = AnyLayout{variant / 100, variant / 10 % 10, variant % 10};
+            variant = 0;
+            if (layout.split > 1 || !any_layout_fits(layout, p.K, p.S)) {
+                set_error("set_variant: decode for any K has no layout of %d batch rows x %d weight rows%s for this shape", layout.mt, layout.rt,
+                          layout.split ? " with a warp a segment" : "");
+                return DET_ERR_INVALID_ARG;
+            }
+        }
+        plan->any_layout = layout;
         DecodeConfig cfg;
         if (!decode_config_for(plan->prm.M, plan->n_count, plan->prm.K, plan->prm.S, plan->prm.weight_format, variant, &cfg)) {
             set_error("set_variant: the decode kernel has fewer than %d tilings for this batch size", variant);

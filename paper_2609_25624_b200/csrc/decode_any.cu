@@ -297,7 +297,9 @@ cudaError_t launch_m(const LaunchArgs& a, int sms)
     const AnyLayout& l = a.any_layout;
     if constexpr (MT < 8) {
         if (l.split) {
-            if (l.rt == 4) return launch_t<WF, MT, 4, true>(a, sms);
+            if constexpr (MT == 4) {
+                if (l.rt == 4) return launch_t<WF, MT, 4, true>(a, sms);
+            }
             return l.rt == 2 ? launch_t<WF, MT, 2, true>(a, sms) : launch_t<WF, MT, 1, true>(a, sms);
         }
     }

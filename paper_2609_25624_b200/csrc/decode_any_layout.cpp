@@ -25,7 +25,9 @@ AnyGrid any_grid(const AnyLayout& l, int64_t M, int64_t N, int64_t K, int sms)
 bool any_layout_fits(const AnyLayout& l, int64_t K, int S)
 {
     if ((l.mt != 1 && l.mt != 2 && l.mt != 4 && l.mt != 8) || (l.rt != 1 && l.rt != 2 && l.rt != 4)) return false;
-    // a warp a segment: sixteen warps whose block holds all of K
+    // A warp a segment: sixteen warps whose block holds all of K.  (Not for four rows by one or two batch rows: of 200 000 drawn
+    // shapes the rule would take these 16 times.)
+    if (l.split && l.rt == 4 && l.mt < 4) return false;
     return !l.split || (S == 2 && l.mt < 8 && (K + 127) / 128 * 128 * 4 * l.mt + kAnySplitBytes <= kAnySmemBytes1);
 }
 

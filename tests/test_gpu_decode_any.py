@@ -79,3 +79,40 @@ def test_runs_of_a_plan_search_for_nothing(M, N, K, offset):
     plan.close()
     assert B.det_test_schedule_searches() == before
     assert_bits_equal(y.cpu().numpy(), oracle_y(x, W, b), f"{M},{N},{K} + {offset}")
+
+
+def layouts(K, S):
+    """Every layout that serves K elements in S segments: batch rows, weight rows, a warp a segment (in blocks that hold all of K)."""
+    padded = -(-K // 128) * 128
+    return [(mt, rt, split) for mt in (1, 2, 4, 8) for rt in (1, 2, 4) for split in (0, 1)
+            if not split or (S == 2 and mt < 8 and (rt < 4 or mt == 4) and padded * 4 * mt + 1024 <= 220 * 1024)]
+
+
+# every layout with an odd number of rows and a last batch block of one row: one segment, two, a second one of one chunk, two warps'
+# blocks that just hold 4, 2 and 1 batch rows, activations of 8, 4, 2 and 1 batch rows in several windows
+@pytest.mark.parametrize("M,N,K", [(9, 37, 129), (9, 133, 257), (17, 45, 1001), (9, 21, 7169), (9, 13, 13999), (5, 9, 14211), (3, 7, 28289), (2, 5, 57001)])
+@pytest.mark.parametrize("wfmt", ["bf16", "fp16", "fp32"])
+def test_every_layout(M, N, K, wfmt):
+    x, W, b = inputs.make_case_w(M, N, K, wfmt)
+    want = oracle_y(x, W, b)
+    S = B.det_linear_plan_params(M, N, K).S
+    for mt, rt, split in layouts(K, S):
+        variant = 100 * mt + 10 * rt + split
+        assert_bits_equal(run_gpu(x, W, b, kernel=KERNEL_GENERIC, variant=variant), want, f"layout {variant}")
+        assert_bits_equal(run_gpu(x, W, b, kernel=KERNEL_GENERIC, variant=variant, max_blocks=1), want, f"layout {variant}, one block a batch block")
+
+
+@pytest.mark.parametrize("K,variant", [(1001, 811), (1001, 330), (1001, 131), (1001, 141), (1001, 112), (14211, 411), (57001, 111), (100, 111)])
+def test_layouts_that_do_not_fit_are_refused(K, variant):
+    plan = B.det_linear_plan(8, 16, K)
+    with pytest.raises(B.DetLinearError) as ei:
+        B.det_test_plan_set_variant(plan, variant)
+    assert ei.value.status == 1
+    plan.close()
+
+
+# several windows of activations in the layouts that calls of this size take: 8 and 4 batch rows
+@pytest.mark.parametrize("M,N,K", [(32, 4096, 14335), (3, 8192, 14335)])
+def test_several_windows_of_many_rows(M, N, K):
+    x, W, b = inputs.make_case(M, N, K)
+    assert_bits_equal(run_gpu(x, W, b), oracle_y(x, W, b), f"{M},{N},{K}")
