@@ -28,7 +28,10 @@ namespace detlin {
 namespace {
 
 // SPLIT: the two segments of a row belong to two warps, the second half of the block's warps to the second ones.
-template <int WF, int MT, int RT, bool SPLIT>
+// WINDOWS: shared memory does not hold the activations' whole K.  A kernel of its own: where all of K is there, the window's bookkeeping
+// in the loop costs registers that spill (M = 26, N = 4857, K = 2669 with FP32 weights 70.6 -> 58.4 us, M = 58, N = 9341, K = 4893 367 ->
+// 323; over 180 shapes in one layout each 0.88 of the time).
+template <int WF, int MT, int RT, bool SPLIT, bool WINDOWS>
 __global__ void __launch_bounds__(512, 1)
 decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::type* __restrict__ W, const float* __restrict__ b,
                   float* __restrict__ y, int M, int N, unsigned K, unsigned seg_len, long long ldy, unsigned win, int groups)
@@ -46,27 +49,47 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    // activations of the window [w_lo, w_lo + win) into shared memory
+    // Activations of the window [w_lo, w_lo + win) into shared memory.  All of K, once, for few rows of weights as a rule: column by
+    // column, the batch rows' copies of a column one after the other, under the first weights' way from memory.  Window by window: row
+    // by row (M = 16, N = 12155, K = 7337 with FP32 weights 213 us, by columns 229; M = 31, N = 2057, K = 7807 69 and 74).
     auto stage = [&](unsigned w_lo) {
         const unsigned len = min(win, K - w_lo);
         const uint32_t base = (uint32_t)__cvta_generic_to_shared(xs);
-        for (unsigned i = threadIdx.x; i < win; i += threads) {
-            const float* src = x + (size_t)m0 * K + w_lo + i;
-            if (i < len) {
+        if constexpr (WINDOWS) {
+#pragma unroll 1
+            for (int m = 0; m < MT; ++m) {
+                const float* src = x + (size_t)min(m0 + m, M - 1) * K + w_lo;     // rows beyond M repeat the last one
+#pragma unroll 4
+                for (unsigned i = threadIdx.x; i < len; i += threads)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(base + (m * win + i) * 4u), "l"(src + i) : "memory");
+                for (unsigned i = len + threadIdx.x; i < win; i += threads) xs[m * win + i] = -0.0f;
+            }
+        } else {
+            for (unsigned i = threadIdx.x; i < win; i += threads) {
+                const float* src = x + (size_t)m0 * K + i;
+                if (i < len) {
 #pragma unroll
-                for (int m = 0; m < MT; ++m) {
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(base + (m * win + i) * 4u), "l"(src) : "memory");
-                    if (m0 + m + 1 < M) src += K;    // rows beyond M repeat the last one
+                    for (int m = 0; m < MT; ++m) {
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(base + (m * win + i) * 4u), "l"(src) : "memory");
+                        if (m0 + m + 1 < M) src += K;    // (likewise)
+                    }
+                } else {
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) xs[m * win + i] = -0.0f;
                 }
-            } else {
-#pragma unroll
-                for (int m = 0; m < MT; ++m) xs[m * win + i] = -0.0f;
             }
         }
-        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto staged = [&]() {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
     };
 
-    const bool one_window = K <= win;
+    // (With WINDOWS never so, which the launcher knows.  Asked all the same: without it the compiler keeps other registers, M = 16, N =
+    // 3796, K = 8841 with FP16 weights 94 -> 121 us, M = 32, N = 4096, K = 14335 256 -> 288.)
+    [[maybe_unused]] const bool one_window = K <= win;
+    if constexpr (!WINDOWS) stage(0);
     for (int grp = (int)blockIdx.x; grp < groups; grp += (int)gridDim.x) {
         const int n0 = (grp * rows_of_warps + warp) * RT;
 
@@ -172,7 +195,7 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
         };
 
         // groups of up to UC chunks, never across the end of a segment or of a window
-        auto group_end = [&](unsigned c, unsigned s_hi, unsigned w_hi) { return min(min(K, s_hi), min(w_hi, c + 128 * UC)); };
+        auto group_end = [&](unsigned c, unsigned s_hi, unsigned w_hi) { return min(min(K, s_hi), WINDOWS ? min(w_hi, c + 128 * UC) : c + 128 * UC); };
         bool first = true;                           // no segment has ended yet
         unsigned w_hi = win, w_lo = ~0u;             // end of the window of the group loaded last; start of the one in shared memory
         unsigned s_hi = second ? 2 * seg_len : seg_len;      // end of the segment of the group being multiplied
@@ -183,6 +206,7 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
             for (int r = 0; r < RT; ++r) pw[r] += seg_len * (unsigned)sizeof(WT) / 4;
         }
         load(raw[0], c, c_end);
+        if (!WINDOWS && grp == (int)blockIdx.x) staged();
 #pragma unroll
         for (int m = 0; m < MT; ++m)
 #pragma unroll
@@ -190,17 +214,19 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
         int buf = 0;
 #pragma unroll 1
         while (c < c_stop) {
-            if (one_window ? (w_lo != 0 && grp == (int)blockIdx.x) : (w_lo == ~0u || c - w_lo >= win)) {
-                w_lo = one_window ? 0 : c;
-                __syncthreads();                     // everybody has finished with the window before
-                stage(w_lo);
-                __syncthreads();
+            if constexpr (WINDOWS) {
+                if (one_window ? (w_lo != 0 && grp == (int)blockIdx.x) : (w_lo == ~0u || c - w_lo >= win)) {
+                    w_lo = one_window ? 0 : c;
+                    __syncthreads();                 // everybody has finished with the window before
+                    stage(w_lo);
+                    staged();
+                }
             }
             const bool seg_done = c_end == min(K, s_hi);
             if (seg_done) s_hi += seg_len;
-            if (c_end == w_hi) w_hi += win;
+            if (WINDOWS && c_end == w_hi) w_hi += win;
             const unsigned nc_end = c_end < c_stop ? group_end(c_end, s_hi, w_hi) : c_end;
-            const float* xl = xs + (one_window ? c : c - w_lo) + 4 * lane;
+            const float* xl = xs + (!WINDOWS || one_window ? c : c - w_lo) + 4 * lane;
 #pragma unroll
             for (int half = 0; half < 2; ++half) {   // (the buffers are registers: their index has to be a constant)
                 if (buf == half) {
@@ -260,21 +286,20 @@ decode_any_kernel(const float* __restrict__ x, const typename WeightElem<WF>::ty
     }
 }
 
-template <int WF, int MT, int RT, bool SPLIT>
-cudaError_t launch_t(const LaunchArgs& a, int sms)
+template <int WF, int MT, int RT, bool SPLIT, bool WINDOWS>
+cudaError_t launch_w(const LaunchArgs& a, const AnyGrid& g)
 {
     static bool configured[kMaxDevices];             // function attributes belong to a device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    auto kern = decode_any_kernel<WF, MT, RT, SPLIT>;
+    auto kern = decode_any_kernel<WF, MT, RT, SPLIT, WINDOWS>;
     if (!configured[dev]) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kAnySmemBytes1);
         if (e != cudaSuccess) return e;
         configured[dev] = true;
     }
-    const AnyGrid g = any_grid({MT, RT, SPLIT}, a.M, a.N, a.K, sms);
     const unsigned win = (unsigned)g.window;
     const int64_t grid = a.max_blocks > 0 && g.blocks_x > a.max_blocks ? a.max_blocks : g.blocks_x;
     cudaLaunchConfig_t cfg{};
@@ -289,6 +314,16 @@ cudaError_t launch_t(const LaunchArgs& a, int sms)
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, a.x, static_cast<const typename WeightElem<WF>::type*>(a.W), a.b, a.y, (int)a.M, (int)a.N,
                               (unsigned)a.K, (unsigned)a.seg_len, (long long)a.ldy, win, (int)g.groups);
+}
+
+template <int WF, int MT, int RT, bool SPLIT>
+cudaError_t launch_t(const LaunchArgs& a, int sms)
+{
+    const AnyGrid g = any_grid({MT, RT, SPLIT}, a.M, a.N, a.K, sms);
+    if constexpr (!SPLIT) {
+        if (g.window < a.K) return launch_w<WF, MT, RT, SPLIT, true>(a, g);
+    }
+    return launch_w<WF, MT, RT, SPLIT, false>(a, g);
 }
 
 template <int WF, int MT>

@@ -33,7 +33,8 @@ bool any_layout_fits(const AnyLayout& l, int64_t K, int S)
 
 // Predicted cycles of a layout: instructions of a warp (operands, line-up and multiplications of its chunks, its part of the
 // activations, lane trees), at the rate of a lone warp or of the SM's schedulers, whichever is slower.  Constants fitted to every layout
-// of 68 drawn shapes (M 1 .. 64, N 64 .. 60000, K 101 .. 9001): mean loss against the best layout 2 %.
+// of 337 drawn shapes (M 1 .. 64, N 64 .. 20000, K 101 .. 10001): mean loss against the best layout 2 %; against the fixed rule below
+// 0.72 of the time on average, at most 1.034 (M = 1, N = 366, K = 7999 18.5 and 19.1 us).
 static double layout_cost(const AnyLayout& l, int64_t M, int64_t N, int64_t K, int S, int wfmt, int sms)
 {
     if (!any_layout_fits(l, K, S)) return 1e300;
@@ -43,14 +44,14 @@ static double layout_cost(const AnyLayout& l, int64_t M, int64_t N, int64_t K, i
     if (l.split && blocks > sms) return 1e300;
     const double iters = (double)((g.groups + g.blocks_x - 1) / g.blocks_x), waves = (double)((blocks + occ * sms - 1) / (occ * sms));
     const double chunks = (double)padded / 128 / (l.split ? 2 : 1);
-    double per_chunk = l.mt * (2 + (l.rt == 1 ? 4 : 2 * l.rt));
-    if (l.mt * l.rt >= 32) per_chunk *= 1.31;        // registers run out
-    per_chunk += 6.4 + l.rt * (wfmt == 2 ? 14.6 : 11.6);
-    const double body = chunks * per_chunk + 1.34 * l.mt * l.rt * (l.split ? 1 : 2) + 254;
-    const double stage = 9.0 * l.mt * (double)g.window / (32.0 * g.warps) *
+    double per_chunk = l.mt * (2.34 + (l.rt == 1 ? 4.81 : 1.94 * l.rt));
+    if (l.mt * l.rt >= 32 && wfmt != 2) per_chunk *= 1.37;       // registers run out
+    per_chunk += 7.65 + l.rt * (wfmt == 2 ? 20.6 : 10.8);
+    const double body = chunks * per_chunk + 1.42 * l.mt * l.rt * (l.split ? 1 : 2) + 256;
+    const double stage = 15.3 * l.mt * (double)g.window / (32.0 * g.warps) *
                          (g.window >= padded ? 1.0 : (double)((padded + g.window - 1) / g.window) * iters);
-    const double shared = (double)(g.warps * (per_sm < occ ? per_sm : occ)) / 4 * 1.08;
-    return (l.split && l.rt == 4 ? 1.2 : 1.0) * waves * ((body * iters + stage) * (shared > 3.94 ? shared : 3.94) + 546);
+    const double shared = (double)(g.warps * (per_sm < occ ? per_sm : occ)) / 4 * 1.09;
+    return (l.split && l.rt == 4 ? 1.065 : 1.0) * waves * ((body * iters + stage) * (shared > 3.92 ? shared : 3.92) + 521);
 }
 
 // Fewer batch rows a warp than there are, where the layer leaves SMs idle otherwise (the weights then come from L2 for the other batch
