@@ -61,7 +61,7 @@ __device__ __forceinline__ float wget(const typename WVec<WF>::type& v, int kk)
     }
 }
 
-// The same as a move that keeps its place in the instruction order (Cfg::kPipelined).
+// The same as a move that keeps its place in the instruction order (the loop that loads ahead).
 template <int WF>
 __device__ __forceinline__ float wget_here(const typename WVec<WF>::type& v, int kk)
 {
@@ -108,8 +108,9 @@ struct Cfg {
     // -> 78.8 us).  Below that the weight stream binds, which the blocks of a thin last round share out among themselves (M = 8,
     // 128256 rows: 200 us without, 207 with), and tiles of 28 rows lose more by the extra bookkeeping (M = 32, 1 %) than
     // their smaller rounds leave to gain.  Tiles of 112 rows (one block to an SM, whose eight warps share each stage's activations)
-    // serve matrices of many rounds only, where equal shares count: M = 8, 128256 rows 184.8 -> 181.4 us, under the power limit
-    // that this call reaches 221 -> 218.
+    // serve matrices of many rounds only, where equal shares count (the line: tiling_cost): 5 to 8 rows, M = 8, 128256 rows 184.8 -> 181.4
+    // us, under the power limit that this call reaches 221 -> 218, and three or more batch blocks of 8, M = 40, N = 28672 with FP16
+    // weights 223 -> 213.
     static constexpr bool kDealRest = (kMB >= 16 && kRB >= 56) || kRB >= 112;
     // BF16: the lower half of a word is widened by a byte permutation, or by a shift in the 4-row tilings of two segment groups
     // that run two blocks to an SM at the full 128 registers: M = 24, N = 6144, K = 4096 35.5 us by shift, 39.4 by permutation (M =
@@ -135,12 +136,14 @@ struct Cfg {
     static constexpr int kConsumerRegsRaw =
         kMoveRegs ? ((kThreads * kLaunchRegs - kPG * 32 * kProducerRegs) / (kConsumerWarps * 32)) / 8 * 8 : 0;
     static constexpr int kConsumerRegs = kConsumerRegsRaw > 240 ? 240 : kConsumerRegsRaw;
-    // Multiply with the next chunk's loads under this chunk's last steps?  FP32 weights only: their pairs are formed by moves that
-    // the compiler otherwise piles up together with all loads of a chunk (M = 32, N = 28672, K = 4096 254 -> 178 us, M = 24, N =
-    // 6144 68 -> 44; the widenings of 16-bit weights fill those gaps by themselves: 71.4 us there, 75 with it at M = 32, N = 4096,
-    // K = 14336).  4-row tiles only where the second set of operands fits the registers (M = 8, N = 4096, K = 14336 41.6 -> 36.7 us;
-    // with 128 registers it spills: 50 -> 138); tiles of one or two rows wait for memory either way.
-    static constexpr bool kPipelined = WF == 2 && (MT == 8 || (MT == 4 && kLaunchRegs >= 168));
+    // Is there a kernel whose multiply loop loads the next chunk under this chunk's last steps (template parameter AHEAD)?  FP32 weights
+    // only: their pairs are formed by moves that the compiler otherwise piles up together with all loads of a chunk (M = 32, N = 28672,
+    // K = 4096 254 -> 178 us, M = 24, N = 6144 68 -> 44; the widenings of 16-bit weights fill those gaps by themselves: 71.4 us there,
+    // 75 with it at M = 32, N = 4096, K = 14336).  Stages of one chunk; 4-row tiles only where the second set of operands fits the
+    // registers (M = 8, N = 4096, K = 14336 41.6 -> 36.7 us; with 128 registers it spills: 50 -> 138), no 8 x 16 tiles (they spill: 1.07 to
+    // 1.45 times as long); tiles of one or two rows wait for memory either way.
+    static constexpr bool kCanLoadAhead = WF == 2 && RT <= 14 && (MT == 8 || (MT == 4 && kLaunchRegs >= 168));
+    static_assert(!kCanLoadAhead || KC == 128, "the loop that loads ahead takes stages of one chunk");
     static_assert(!kMoveRegs || kConsumerRegs * kConsumerWarps * 32 + kProducerRegs * kPG * 32 <= kThreads * kLaunchRegs,
                   "register move must fit in the block's own allocation");
     static_assert(!kMoveRegs || kConsumerRegs >= kLaunchRegs, "consumers only ever grow");
@@ -193,7 +196,8 @@ struct Shares {
     int n_shares, whole_rounds, rest_each, rest_more;
 };
 
-template <int MT, int WM, int RT, int WR, int SK, int KC, int STAGES, int WF>
+// AHEAD: the multiply loop loads a chunk ahead (Cfg::kCanLoadAhead; which calls: decode_loads_ahead)
+template <int MT, int WM, int RT, int WR, int SK, int KC, int STAGES, int WF, bool AHEAD>
 __global__ void __launch_bounds__((Cfg<MT, WM, RT, WR, SK, KC, STAGES, WF>::kThreads), (Cfg<MT, WM, RT, WR, SK, KC, STAGES, WF>::kMinBlocks))
 decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
               const __grid_constant__ typename GroupMap<Cfg<MT, WM, RT, WR, SK, KC, STAGES, WF>::kDealRest>::type map_g,
@@ -442,13 +446,13 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
 #pragma unroll
                 for (int j = 0; j < RT / 2; ++j) acc[m][j] = make_float2(0.0f, 0.0f);
 
-            if constexpr (C::kPipelined) {
+            if constexpr (AHEAD) {
                 // The operands of a chunk are in registers when its multiplications start: their registers are loaded again for the
-                // next chunk right after the last use, under the last two of the chunk's four steps.
+                // next chunk right after the last use, under the last two of the chunk's four steps.  A stage is one chunk.
                 const int n_chunks = (k_hi - k_lo + 127) / 128;
                 if (!mine) {
                     // no rows here: only keeps the ring in step
-                    for (int k0 = k_lo; ok && k0 < k_hi; k0 += KC) {
+                    for (int c = 0; ok && c < n_chunks; ++c) {
                         if (!__all_sync(0xffffffffu, mbar_wait(fullg + 8 * st, phase, abort_flag, status, wait_limit_ns, 2))) { ok = false; break; }
                         __syncwarp();
                         if (lane == 0) mbar_arrive(emptyg + 8 * st);
@@ -456,15 +460,14 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     }
                     ready = false;
                 } else {
-                    constexpr int kChunks = KC / 128, kPairs = RT / 2;
-                    constexpr int kPerBox = C::kKB / 128;     // chunks of a box
+                    constexpr int kPairs = RT / 2;
                     float4 xv[MT];
                     typename WVec<WF>::type w[RT];
                     uint32_t xs = 0, ws = 0;                  // where the next loads come from
-                    auto at_chunk = [&](int stage, int ci) {
-                        const uint32_t box = ringg + (uint32_t)(stage * C::kStageBytes) + (uint32_t)(ci / kPerBox * C::kSubBytes);
-                        xs = box + (wm * MT) * C::kXPitch + lane * 16 + (ci % kPerBox) * 512;
-                        ws = box + C::kXBytes + (wr * RT) * C::kWPitch + lane * (4 * C::kEB) + (ci % kPerBox) * (128 * C::kEB);
+                    auto at_stage = [&](int stage) {
+                        const uint32_t box = ringg + (uint32_t)(stage * C::kStageBytes);
+                        xs = box + (wm * MT) * C::kXPitch + lane * 16;
+                        ws = box + C::kXBytes + (wr * RT) * C::kWPitch + lane * (4 * C::kEB);
                     };
                     auto load_x = [&](int m) { xv[m] = lds128((m < (MT + 1) / 2 ? xs + x_lo_off : xs - x_lo_off) + m * C::kXPitch); };
                     auto load_w = [&](int q) { w[q] = wload<WF>(((q & 1) ? ws - w_off : ws + w_off) + q * C::kWPitch); };
@@ -505,9 +508,9 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     if (!__all_sync(0xffffffffu, ready)) {
                         if (!__all_sync(0xffffffffu, mbar_wait(fullg + 8 * st, phase, abort_flag, status, wait_limit_ns, 2))) ok = false;
                     }
-                    int st_cur = st, ci = 0;                  // stage and chunk of the stage in work; st is the stage after it
+                    int st_cur = st;                          // stage in work; st is the one after it
                     if (ok) {
-                        at_chunk(st, 0);
+                        at_stage(st);
                         if (++st == STAGES) { st = 0; phase ^= 1; }
 #pragma unroll
                         for (int q = 0; q < RT; ++q) load_w(q);
@@ -518,25 +521,20 @@ decode_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__
                     const int n_loop = ok ? n_chunks - 1 : 0;
 #pragma unroll 1
                     for (int c = 0; c < n_loop; ++c) {
-                        // No branches but the rare wait: they would cut the loop into pieces that cannot overlap.  (The phase of st_cur,
-                        // which has landed, is the other one of st's if st has wrapped.)
-                        const bool cross = kChunks == 1 || ci == kChunks - 1;   // the next chunk lies in the next stage
-                        const int st_next = cross ? st : st_cur;
-                        const unsigned want = cross ? phase : phase ^ (unsigned)(st == 0);
-                        ready = mbar_test_wait(fullg + 8 * st_next, want);
+                        // no branches but the rare wait: they would cut the loop into pieces that cannot overlap
+                        ready = mbar_test_wait(fullg + 8 * st, phase);
                         step(integral_constant<int, 0>(), Last());
                         __syncwarp();                         // every load from the stage has returned (step 0 uses a part of each)
-                        mbar_arrive_if(emptyg + 8 * st_cur, cross && lane == 0);
+                        mbar_arrive_if(emptyg + 8 * st_cur, lane == 0);
                         step(integral_constant<int, 1>(), Last());
                         if (!__all_sync(0xffffffffu, ready)) {
-                            if (!__all_sync(0xffffffffu, mbar_wait(fullg + 8 * st_next, want, abort_flag, status, wait_limit_ns, 2))) { ok = false; break; }
+                            if (!__all_sync(0xffffffffu, mbar_wait(fullg + 8 * st, phase, abort_flag, status, wait_limit_ns, 2))) { ok = false; break; }
                         }
-                        ci = cross ? 0 : ci + 1;
-                        at_chunk(st_next, ci);
-                        st_cur = st_next;
+                        at_stage(st);
+                        st_cur = st;
                         const bool wrap = st + 1 == STAGES;
-                        phase ^= (unsigned)(cross && wrap);
-                        st = cross ? (wrap ? 0 : st + 1) : st;
+                        phase ^= (unsigned)wrap;
+                        st = wrap ? 0 : st + 1;
                         step(integral_constant<int, 2>(), Next());
                         step(integral_constant<int, 3>(), Next());
                     }
@@ -767,7 +765,7 @@ int decode_occupancy_t(int S)
     static bool attr_set[kMaxDevices];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return 0; }
-    auto kern = decode_kernel<MT, WM, RT, WR, SK, KC, STAGES, WF>;
+    auto kern = decode_kernel<MT, WM, RT, WR, SK, KC, STAGES, WF, false>;
     if (!attr_set[dev]) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::smem_bytes(kDecodeMaxSegments) > 227 * 1024 ? 227 * 1024 : C::smem_bytes(kDecodeMaxSegments)) != cudaSuccess) {
             cudaGetLastError();
@@ -791,9 +789,24 @@ template <int MT, int WM, int RT, int WR, int SK, int KC, int STAGES, int WF>
 cudaError_t launch_decode_t(const LaunchArgs& a, const CUtensorMap* map_w, const CUtensorMap* map_g, const CUtensorMap* map_x)
 {
     using C = Cfg<MT, WM, RT, WR, SK, KC, STAGES, WF>;
-    auto kern = decode_kernel<MT, WM, RT, WR, SK, KC, STAGES, WF>;
+    auto kern = decode_kernel<MT, WM, RT, WR, SK, KC, STAGES, WF, false>;
     const int blocks_per_sm = decode_occupancy_t<MT, WM, RT, WR, SK, KC, STAGES, WF>(a.S);
     if (blocks_per_sm <= 0) return cudaErrorLaunchOutOfResources;
+    if constexpr (C::kCanLoadAhead) {
+        if (decode_loads_ahead(a.wfmt, a.M, a.K, a.S)) {
+            // (as many blocks to an SM: shared memory decides, and both are compiled for kMinBlocks)
+            kern = decode_kernel<MT, WM, RT, WR, SK, KC, STAGES, WF, true>;
+            static bool attr_set[kMaxDevices];
+            int dev = 0;
+            cudaError_t e = cudaGetDevice(&dev);
+            if (e == cudaSuccess && (dev < 0 || dev >= kMaxDevices)) e = cudaErrorInvalidDevice;
+            if (e == cudaSuccess && !attr_set[dev]) {
+                e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::smem_bytes(kDecodeMaxSegments) > 227 * 1024 ? 227 * 1024 : C::smem_bytes(kDecodeMaxSegments));
+                attr_set[dev] = e == cudaSuccess;
+            }
+            if (e != cudaSuccess) return e;
+        }
+    }
     const long long n_groups = (a.N + RT - 1) / RT;
     const int n_mblocks = (int)((a.M + C::kMB - 1) / C::kMB);
     const long long slots = (long long)a.sm_count * blocks_per_sm;

@@ -27,16 +27,19 @@ int m_class(int64_t M) { return M <= 1 ? 0 : M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 
 // HBM rate) and performs rb * mb * K multiply-adds at the FMA rate of an SM times an efficiency that depends on the warp tile;
 // whichever is larger binds.  Units resident on one SM share it.  Fewer than eight consumer warps per SM hide latency badly; every
 // unit pays for its lane trees (one per segment) and, with several segment groups, for the fold through shared memory.
-// The rates were fitted to sweeps of every tiling on a 148-SM B200.  16-bit weights, up to 8 rows: the Llama-3-8B shapes, mean loss against
-// the best tiling 0.5 %.  More rows: 56 drawn and layer shapes, 9 to 64 rows, mean loss 2 % (3.5 % with the rates of few rows: M = 16, N =
-// 4096, K = 14336 44.5 -> 41.6 us, M = 16, N = 2083, K = 14096 49.8 -> 42.6, M = 17, N = 432, K = 5416 11.5 -> 10.5);
-// from K = 2560 on: short rows are a matter of latencies that this does not know (M = 16, N = 278, K = 2168 5.6 us, with the rates of few rows 4.8).  FP32 weights: 52 shapes at
-// batch 1 .. 64, 2 % (24 % with those of 16 bits): their multiply loop is another one in the larger tiles (Cfg::kPipelined).
+// The rates were fitted to sweeps of every tiling on a 148-SM B200.
+//   * 16-bit weights, up to 8 rows: the Llama-3-8B shapes, mean loss against the best tiling 0.5 %.
+//   * 16-bit weights, more rows, K from 2560 on: 56 drawn and layer shapes, 9 to 64 rows, mean loss 2 % (3.5 % with the rates of few
+//     rows: M = 16, N = 4096, K = 14336 44.5 -> 41.6 us, M = 16, N = 2083, K = 14096 49.8 -> 42.6).  Shorter rows are a matter of
+//     latencies that these rates do not know (M = 16, N = 278, K = 2168 5.6 us, with the rates of few rows 4.8).
+//   * FP32 weights whose loop loads a chunk ahead (decode_loads_ahead): 52 shapes at batch 1 .. 64, 2 % (24 % with the rates of few
+//     rows); the others by the rates of few rows.  Only where these choose a tiling with more units than SMs: in one wave of single blocks
+//     a block's rows and ring decide, not rates (M = 4, N = 97, K = 8552 11.4 us, by the rates for loading ahead 14.9).
 struct TilingRates {
     double eff8, eff4, eff2, eff1;       // share of the FMA rate by batch rows of a warp tile
     double wide, narrow;                 // ... times: 8-row tiles with half as many stage boundaries (KC 512); stages of 128
     double small8, small4;               // ... times: blocks of at most four consumer warps
-    double hbm;                          // bytes per clock and SM
+    double hbm;                          // bytes per clock and SM (FP32 weights by the rates of 16 bits: twice as many)
     double other;                        // share of the term that does not bind
     double latency;                      // exponent of 8 / warps
     double tree, fold;                   // cycles per segment of a full tile; with several segment groups
@@ -44,17 +47,23 @@ struct TilingRates {
 };
 constexpr TilingRates kRatesFewRows = {0.707, 0.70, 0.345, 0.2, 1.2, 0.9, 1.0, 1.0, 22.5, 0.0, 1.0, 1020.0, 1500.0, 1.08, 1.0};
 constexpr TilingRates kRatesManyRows = {0.922, 0.844, 0.420, 0.141, 1.057, 0.9, 0.96, 0.973, 27.0, 0.0264, 1.703, 799.0, 1384.0, 0.7355, 0.567};
+constexpr TilingRates kRatesFp32Short = {0.707, 0.70, 0.345, 0.2, 1.2, 0.9, 1.0, 1.0, 45.0, 0.0, 1.0, 1020.0, 1500.0, 1.08, 1.0};
 constexpr TilingRates kRatesFp32 = {0.52, 0.43, 0.49, 0.075, 1.0, 1.0, 0.904, 0.558, 32.0, 0.0, 1.0, 1020.0, 1500.0, 1.08, 1.0};
 
-double tiling_cost(const DecodeEntry& e, int wfmt, int64_t M, int64_t N, int64_t K, int S, int sm_count)
+int64_t tiling_units(const DecodeConfig& c, int64_t M, int64_t N)
+{
+    const int64_t rb = (int64_t)c.rt * c.wr, mb = (int64_t)c.mt * c.wm;
+    return ((N + rb - 1) / rb) * ((M + mb - 1) / mb);
+}
+
+double tiling_cost(const DecodeEntry& e, const TilingRates& t, int wfmt, int64_t M, int64_t N, int64_t K, int S, int sm_count)
 {
     const DecodeConfig& c = e.cfg;
-    const TilingRates& t = wfmt == DET_WEIGHT_FP32 ? kRatesFp32 : M > 8 && K >= 2560 ? kRatesManyRows : kRatesFewRows;
     const int occ = e.occupancy(S);
     if (occ <= 0) return 1e300;
     const int64_t rb = (int64_t)c.rt * c.wr, mb = (int64_t)c.mt * c.wm;
     const int64_t mblocks = (M + mb - 1) / mb;
-    const int64_t units = ((N + rb - 1) / rb) * mblocks;
+    const int64_t units = tiling_units(c, M, N);
     const int64_t rounds = (units + (int64_t)sm_count * occ - 1) / ((int64_t)sm_count * occ);
     const int64_t per_sm = (units + sm_count - 1) / sm_count;
     const double resident = (double)(per_sm < occ ? per_sm : occ);
@@ -124,19 +133,28 @@ bool decode_config_for(int64_t M, int64_t N, int64_t K, int S, int wfmt, int var
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
             sms = 148;
     }
-    int pick_cls = classes[0], pick = -1, seen = 0;
-    double best = 1e299;
-    for (int ci = 0; ci < n_classes && (variant == 0 || pick < 0); ++ci) {
-        const DecodeClassTable* t = class_table(wfmt, classes[ci]);
-        for (int i = 0; i < t->count; ++i) {
-            if (variant == 0) {
-                const double c = tiling_cost(t->entries[i], wfmt, M, N, K, S, sms);
+    int pick_cls = classes[0], pick = -1;
+    auto choose = [&](const TilingRates& t) {
+        double best = 1e299;
+        for (int ci = 0; ci < n_classes; ++ci) {
+            const DecodeClassTable* tab = class_table(wfmt, classes[ci]);
+            for (int i = 0; i < tab->count; ++i) {
+                const double c = tiling_cost(tab->entries[i], t, wfmt, M, N, K, S, sms);
                 if (c < best) { best = c; pick_cls = classes[ci]; pick = i; }
-            } else if (t->entries[i].occupancy(S) > 0 && ++seen == variant) {
-                pick_cls = classes[ci];
-                pick = i;
-                break;
             }
+        }
+    };
+    if (variant == 0) {
+        const bool fp32 = wfmt == DET_WEIGHT_FP32, many_rows = !fp32 && M > 8 && K >= 2560;
+        choose(fp32 ? kRatesFp32Short : many_rows ? kRatesManyRows : kRatesFewRows);
+        const TilingRates* better = fp32 && decode_loads_ahead(wfmt, M, K, S) ? &kRatesFp32 : nullptr;
+        if (better && pick >= 0 && tiling_units(class_table(wfmt, pick_cls)->entries[pick].cfg, M, N) > sms) choose(*better);
+    } else {
+        int seen = 0;
+        for (int ci = 0; ci < n_classes && pick < 0; ++ci) {
+            const DecodeClassTable* tab = class_table(wfmt, classes[ci]);
+            for (int i = 0; i < tab->count && pick < 0; ++i)
+                if (tab->entries[i].occupancy(S) > 0 && ++seen == variant) { pick_cls = classes[ci]; pick = i; }
         }
     }
     if (pick < 0) return false;

@@ -1,5 +1,6 @@
 """Helpers for the GPU parity tests: run the CUDA path through the C ABI and fetch bits."""
 import numpy as np
+import pytest
 import torch
 
 from paper_2609_25624_b200 import binding as B
@@ -36,6 +37,22 @@ def run_gpu(x, W, b, kernel=None, variant=0, max_blocks=0, stream=None, y_fill=f
     finally:
         plan.close()
     return y.cpu().numpy()
+
+
+def decode_tilings(M, N, K, wfmt="bf16"):
+    """How many tilings of the decode kernel serve a shape: those compiled for the batch size (more than 8 rows: the 8-row ones too;
+    FP32 weights have no tiles of 112 rows), with one segment only those without segment groups.  One more is refused."""
+    S = B.det_linear_plan_params(M, N, K).S
+    cls = next(c for c, top in enumerate((1, 2, 4, 8, 16, 64)) if M <= top)
+    eight = (10 if S == 2 else 4) - (wfmt == "fp32")
+    n = {0: 5, 1: 6, 2: 8, 3: eight, 4: 7 + eight, 5: 6 + eight}[cls] if S == 2 else {0: 2, 1: 2, 2: 2, 3: eight, 4: 5 + eight, 5: 5 + eight}[cls]
+    plan = B.det_linear_plan_w(M, N, K, wfmt)
+    B.det_test_plan_set_variant(plan, n)
+    with pytest.raises(B.DetLinearError) as ei:
+        B.det_test_plan_set_variant(plan, n + 1)
+    assert ei.value.status == 1
+    plan.close()
+    return n
 
 
 def oracle_y(x, W, b):
