@@ -6,7 +6,7 @@ import torch
 from oracle import oracle
 from paper_2609_25624_b200 import binding as B
 from paper_2609_25624_b200 import inputs
-from tests.gpu_util import (KERNEL_DECODE, KERNEL_GENERIC, KERNEL_PREFILL, assert_bits_equal, oracle_y,
+from tests.gpu_util import (KERNEL_DECODE, KERNEL_GENERIC, KERNEL_PREFILL, assert_bits_equal, decode_tilings, oracle_y,
                             run_gpu)
 
 pytestmark = pytest.mark.gpu
@@ -43,16 +43,8 @@ def test_decode_bit_exact_all_tilings(M, N, K):
     x, W, b = inputs.make_case(M, N, K)
     want = oracle_y(x, W, b)
     assert_bits_equal(run_gpu(x, W, b, kernel=KERNEL_GENERIC), want, "generic")
-    n_tilings = 0
-    for variant in range(0, 16):               # 0 = automatic choice, then every compiled tiling of this batch class
-        try:
-            got = run_gpu(x, W, b, kernel=KERNEL_DECODE, variant=variant)
-        except B.DetLinearError:
-            break
-        assert_bits_equal(got, want, f"variant={variant}")
-        n_tilings = variant
-    # tilings whose segment groups do not divide S cannot run the shape
-    assert n_tilings >= (4 if oracle.order_params(M, N, K)["S"] == 2 else 2)
+    for variant in range(decode_tilings(M, N, K) + 1):       # 0 = automatic choice, then every tiling that serves the shape
+        assert_bits_equal(run_gpu(x, W, b, kernel=KERNEL_DECODE, variant=variant), want, f"variant={variant}")
     assert_bits_equal(run_gpu(x, W, b, max_blocks=1), want, "one block")
     assert_bits_equal(run_gpu(x, W, b, max_blocks=3), want, "three blocks")
 

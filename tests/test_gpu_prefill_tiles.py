@@ -41,7 +41,7 @@ def test_units_cut_between_blocks(M, N, K, wfmt):
         B.det_linear_run(plan, xd, Wd, bd, y)
         B.det_linear_plan_check(plan)
         assert_bits_equal(y.cpu().numpy(), want, f"run {rep}")
-    for variant in (28, 37, 46, 55):             # other tiles of the same plan
+    for variant in (28, 37, 46, 55, 58):             # other tiles of the same plan
         B.det_test_plan_set_variant(plan, variant)
         y = torch.full((M, N), float("nan"), dtype=torch.float32, device="cuda")
         B.det_linear_run(plan, xd, Wd, bd, y)
