@@ -33,8 +33,10 @@ int m_class(int64_t M) { return M <= 1 ? 0 : M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 
 //     rows: M = 16, N = 4096, K = 14336 44.5 -> 41.6 us, M = 16, N = 2083, K = 14096 49.8 -> 42.6).  Shorter rows are a matter of
 //     latencies that these rates do not know (M = 16, N = 278, K = 2168 5.6 us, with the rates of few rows 4.8).
 //   * FP32 weights whose loop loads a chunk ahead (decode_loads_ahead): 52 shapes at batch 1 .. 64, 2 % (24 % with the rates of few
-//     rows); the others by the rates of few rows.  Only where these choose a tiling with more units than SMs: in one wave of single blocks
-//     a block's rows and ring decide, not rates (M = 4, N = 97, K = 8552 11.4 us, by the rates for loading ahead 14.9).
+//     rows); the others by the rates of few rows.
+// The last two only where the rates of few rows choose a tiling with more units than SMs.  In one wave of single blocks a block's rows
+// and ring decide, not rates: M = 12, N = 99, K = 5832 8.1 us, by the rates of many rows 10.8; M = 4, N = 97, K = 8552 with FP32
+// weights 11.4 and 14.9.  Of 220 shapes of 16-bit weights none is then slower than by the rates of few rows; 13 were, up to 1.4 times.
 struct TilingRates {
     double eff8, eff4, eff2, eff1;       // share of the FMA rate by batch rows of a warp tile
     double wide, narrow;                 // ... times: 8-row tiles with half as many stage boundaries (KC 512); stages of 128
@@ -89,8 +91,13 @@ double tiling_cost(const DecodeEntry& e, const TilingRates& t, int wfmt, int64_t
         shares = shares < 1 ? 1 : shares > groups ? groups : shares;
         const int64_t whole = groups / (shares * c.wr), rest = groups - whole * shares * c.wr;
         const double part = (double)((rest + shares - 1) / shares) / c.wr;
-        // tiles of 112 rows only for many rounds: M = 7, N = 50000, K = 2048 (3.02 rounds) 45.9 us, by 56 rows 44.1; M = 8, N = 28672,
-        // K = 4096 (1.7 rounds) 50.5 and 50.1; N = 128256 (7.7 rounds) 181.4 and 184.8
+        // Tiles of 112 rows only from five rounds of a batch block's shares on (8 rows share all SMs, 24 a third of them).  us, by 112 rows
+        // and by the better one of 28 and 56: M = 8, N = 28672, K = 4096 (1.7 rounds) 50.5 and 50.1; M = 8, N = 33152, K = 2048 (2) 27.9 and
+        // 27.5; M = 7, N = 50000 (3.02) 45.9 and 44.1; M = 8, N = 58016, K = 4096 (3.5) 93.0 and 83.6; M = 8, N = 66304 FP16 (4) 53.4 and
+        // 57.9; M = 8, N = 74592, K = 4096 (4.5) 110 and 106; M = 8, N = 82884 FP16 (5) 70.8 and 75.8; M = 5, N = 132608 (8) 99.5 and
+        // 98.8; N = 128256, K = 4096 (7.7) 181.4 and 184.8.  More rows: M = 24, N = 28672, K = 4096 (5.2) 127 and 122, M = 20 with FP16 134
+        // and 135; M = 40 (8.8) 200 and 202, with FP16 213 and 223; M = 24, N = 50000, K = 2560 (9.1) 138 and 135; M = 36, N = 40000 (12)
+        // 181 and 179.
         if (rb >= 112 && whole < 5) return 1e300;
         if (whole > 0) return (double)whole * (body + overhead) + (part < 1.0 ? t.part * pow(part, t.part_exp) : 1.0) * body + (rest ? overhead : 0.0);
     }
@@ -145,9 +152,9 @@ bool decode_config_for(int64_t M, int64_t N, int64_t K, int S, int wfmt, int var
         }
     };
     if (variant == 0) {
-        const bool fp32 = wfmt == DET_WEIGHT_FP32, many_rows = !fp32 && M > 8 && K >= 2560;
-        choose(fp32 ? kRatesFp32Short : many_rows ? kRatesManyRows : kRatesFewRows);
-        const TilingRates* better = fp32 && decode_loads_ahead(wfmt, M, K, S) ? &kRatesFp32 : nullptr;
+        const bool fp32 = wfmt == DET_WEIGHT_FP32;
+        choose(fp32 ? kRatesFp32Short : kRatesFewRows);
+        const TilingRates* better = fp32 ? (decode_loads_ahead(wfmt, M, K, S) ? &kRatesFp32 : nullptr) : M > 8 && K >= 2560 ? &kRatesManyRows : nullptr;
         if (better && pick >= 0 && tiling_units(class_table(wfmt, pick_cls)->entries[pick].cfg, M, N) > sms) choose(*better);
     } else {
         int seen = 0;

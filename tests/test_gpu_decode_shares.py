@@ -2,6 +2,7 @@
 where the last tile of a block holds one to four row groups, fewer than the block has warps for, or none."""
 import pytest
 
+from paper_2609_25624_b200 import binding as B
 from paper_2609_25624_b200 import inputs
 from tests.gpu_util import KERNEL_DECODE, assert_bits_equal, decode_tilings, oracle_y, run_gpu
 
@@ -35,3 +36,13 @@ def every_tiling(M, N, K, wfmt):
     for variant in range(decode_tilings(M, N, K, wfmt) + 1):
         assert_bits_equal(run_gpu(x, W, b, kernel=KERNEL_DECODE, variant=variant), want, f"variant {variant}")
     assert_bits_equal(run_gpu(x, W, b, max_blocks=7), want, "seven blocks")
+
+
+# one wave of at most a block an SM: small blocks
+@pytest.mark.gpu
+@pytest.mark.parametrize("M,N,K,wfmt", [(12, 99, 5832, "bf16"), (42, 89, 4416, "fp16"), (24, 246, 6112, "bf16"), (17, 59, 2704, "fp16")])
+def test_tilings_of_few_units(M, N, K, wfmt):
+    plan = B.det_linear_plan_w(M, N, K, wfmt)
+    t = B.det_linear_plan_describe(plan)["decode_tiling"]
+    plan.close()
+    assert (t["mt"], t["wm"], t["wr"], t["sk"]) == (4, 2, 1, 2)
