@@ -793,7 +793,7 @@ cudaError_t launch_decode_t(const LaunchArgs& a, const CUtensorMap* map_w, const
     const int blocks_per_sm = decode_occupancy_t<MT, WM, RT, WR, SK, KC, STAGES, WF>(a.S);
     if (blocks_per_sm <= 0) return cudaErrorLaunchOutOfResources;
     if constexpr (C::kCanLoadAhead) {
-        if (decode_loads_ahead(a.wfmt, a.M, a.K, a.S)) {
+        if (decode_loads_ahead(MT, a.M, a.K, a.S)) {
             // (as many blocks to an SM: shared memory decides, and both are compiled for kMinBlocks)
             kern = decode_kernel<MT, WM, RT, WR, SK, KC, STAGES, WF, true>;
             static bool attr_set[kMaxDevices];

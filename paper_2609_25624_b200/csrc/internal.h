@@ -123,15 +123,20 @@ struct DecodeConfig {
 // S = number of K segments of the order (it only scales the unit count in the schedule's cost model)
 bool decode_config_for(int64_t M, int64_t N, int64_t K, int S, int wfmt, int variant, DecodeConfig* out);
 int decode_num_variants();
-// FP32 weights: does the multiply loop load a chunk ahead?  The loads of a segment's first chunk, all of them before the first
-// multiplication, then cost what the later chunks gain; per tiling, times with against without: segments of 128 to 256 elements 1.05 to
-// 1.3 (M = 10, N = 22402, K = 208 13.4 us, without 10.8), 512 0.88 to 1.09, 768 0.83 to 1.05 (on average 0.91 of tiles of 8 rows, 0.97 of
-// 4), 2048 0.73 to 1.0.  Up to four batch rows are bound by memory and gain later: segments of 512 to 1024 1.03, from 2048 on 0.83 to 1.0.
-inline bool decode_loads_ahead(int wfmt, int64_t M, int64_t K, int S)
+// The longest K segment of the decode order.
+inline int64_t decode_segment(int64_t K, int S)
 {
     const int64_t granules = (K + kSegmentGranule - 1) / kSegmentGranule;
-    const int64_t longest = S > 1 ? (granules + S - 1) / S * kSegmentGranule : K;
-    return wfmt == DET_WEIGHT_FP32 && longest >= (M <= 4 ? 2048 : 768);
+    return S > 1 ? (granules + S - 1) / S * kSegmentGranule : K;
+}
+// FP32 weights: does the multiply loop of a tiling load a chunk ahead?  The loads of a segment's first chunk, all of them before the
+// first multiplication, then cost what the later chunks gain.  Times with against without, over the tilings of 161 shapes: segments of
+// 128 to 256 elements 1.05 to 1.3 (M = 10, N = 22402, K = 208 13.4 us, without 10.8); 512 on average 0.96 in tiles of 8 rows a warp (M =
+// 33, N = 6411, K = 880 18.6 and 21.0), 1.01 of 4; 768 0.91 and 0.97; 2048 0.82 and 0.89.  Up to four batch rows are bound by memory
+// and gain later: segments of 512 to 1024 1.03, from 2048 on 0.83 to 1.0.
+inline bool decode_loads_ahead(int rows_of_warp, int64_t M, int64_t K, int S)
+{
+    return decode_segment(K, S) >= (M <= 4 ? 2048 : rows_of_warp == 8 ? 512 : 768);
 }
 // map_w: box of a whole tile (rt * wr weight rows); map_g: of one row group (rt)
 cudaError_t launch_decode(const LaunchArgs& a, const DecodeConfig& cfg, const CUtensorMap* map_w, const CUtensorMap* map_g, const CUtensorMap* map_x);

@@ -32,11 +32,12 @@ int m_class(int64_t M) { return M <= 1 ? 0 : M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 
 //   * 16-bit weights, more rows, K from 2560 on: 56 drawn and layer shapes, 9 to 64 rows, mean loss 2 % (3.5 % with the rates of few
 //     rows: M = 16, N = 4096, K = 14336 44.5 -> 41.6 us, M = 16, N = 2083, K = 14096 49.8 -> 42.6).  Shorter rows are a matter of
 //     latencies that these rates do not know (M = 16, N = 278, K = 2168 5.6 us, with the rates of few rows 4.8).
-//   * FP32 weights whose loop loads a chunk ahead (decode_loads_ahead): 52 shapes at batch 1 .. 64, 2 % (24 % with the rates of few
-//     rows); the others by the rates of few rows.
-// The last two only where the rates of few rows choose a tiling with more units than SMs.  In one wave of single blocks a block's rows
-// and ring decide, not rates: M = 12, N = 99, K = 5832 8.1 us, by the rates of many rows 10.8; M = 4, N = 97, K = 8552 with FP32
-// weights 11.4 and 14.9.  Of 220 shapes of 16-bit weights none is then slower than by the rates of few rows; 13 were, up to 1.4 times.
+//   * FP32 weights, segments of more than two chunks: 52 shapes at batch 1 .. 64, 2 % (24 % with the rates of few rows).
+// The last two only where the rates of few rows choose a tiling with more units than half the SMs.  With fewer, a block's rows and ring
+// decide, not rates: M = 12, N = 99, K = 5832 (16 units) 8.1 us, by the rates of many rows 10.8; M = 4, N = 97, K = 8552 with FP32 weights
+// (7) 11.4 and 14.9; but M = 10, N = 871, K = 7248 (126) 14.4 and 13.3, M = 36, N = 388, K = 8976 with FP32 weights (140) 26.4 and 21.1.
+// Of 195 shapes of 16-bit weights none is then slower by more than 1.5 % than by the rates of many rows, of 144 of FP32 weights in long
+// segments none by more than 2.5 %.
 struct TilingRates {
     double eff8, eff4, eff2, eff1;       // share of the FMA rate by batch rows of a warp tile
     double wide, narrow;                 // ... times: 8-row tiles with half as many stage boundaries (KC 512); stages of 128
@@ -154,8 +155,8 @@ bool decode_config_for(int64_t M, int64_t N, int64_t K, int S, int wfmt, int var
     if (variant == 0) {
         const bool fp32 = wfmt == DET_WEIGHT_FP32;
         choose(fp32 ? kRatesFp32Short : kRatesFewRows);
-        const TilingRates* better = fp32 ? (decode_loads_ahead(wfmt, M, K, S) ? &kRatesFp32 : nullptr) : M > 8 && K >= 2560 ? &kRatesManyRows : nullptr;
-        if (better && pick >= 0 && tiling_units(class_table(wfmt, pick_cls)->entries[pick].cfg, M, N) > sms) choose(*better);
+        const TilingRates* better = fp32 ? (decode_segment(K, S) > 256 ? &kRatesFp32 : nullptr) : M > 8 && K >= 2560 ? &kRatesManyRows : nullptr;
+        if (better && pick >= 0 && tiling_units(class_table(wfmt, pick_cls)->entries[pick].cfg, M, N) > sms / 2) choose(*better);
     } else {
         int seen = 0;
         for (int ci = 0; ci < n_classes && pick < 0; ++ci) {
