@@ -13,8 +13,12 @@ DET_DECLARE(2)
 // Tile width (schedule only: every width gives the same bits).  Wide tiles multiply fastest, narrow ones make more units:
 // with more units than SMs the work is dealt out in equal stretches and the width's rate decides, with fewer the call
 // takes as long as one unit.  A block of the three narrow widths has 16 tm / 16 = 5 .. 8 multiplying warps on four
-// schedulers, so it takes as long as one of 128 rows whatever its height; the wide tile always has eight.  (128 rows by 32 columns: four warps of 8 x 4 outputs a thread, 5 to 9 % faster than eight of 4 x 4.)
-// Rates = share of the FP32 peak, measured at M = 512, N = 28672, K = 4096: 86.6, 82.2, 63.6 and 50.0 %.  Either side of the
+// schedulers, so it takes as long as one of 128 rows whatever its height; the wide tile always has eight.  128 rows by 32 columns
+// are the exception: four warps of 8 x 4 outputs a thread, 5 to 9 % faster than eight of 4 x 4.
+// Rates = share of the FP32 peak, measured at M = 512, N = 28672, K = 4096: 86.6, 82.2, 63.4 and 50.0 % (128 rows by 32 columns 56.7 %).
+// One or two cut units a block do not reach them: the hand-over costs 32 columns of 128 rows more than the rate gains, us at widths 64 /
+// 32, K = 1024, M = 128: N = 1216 (152 units of 32 columns) 18.2 / 15.4, 1400 (176) 18.4 / 17.2, 1600 (200) 18.4 / 18.5, 1800 (228) 18.3 /
+// 20.7; 0.42 puts the line at 198 units.  Either side of the
 // line, us at widths 256 / 128 / 64 / 32: M = 128, N = 4096, K = 14336 (128 units of 256 columns on 148 SMs, or 256 of
 // 128) 279 / 253 / 321 / 401; M = 96 likewise (tile height 96) 212 / 248 / 269 / 323; 100 x 1000 x 1000 with FP32 weights
 // 44 / 27 / 18 / 13; M = 66, N = 300, K = 1000 31 / 26 / 16 / 11.
@@ -29,7 +33,8 @@ int prefill_tile_width(int64_t M, int64_t N, int64_t K, int S, int64_t seg_len, 
     for (int i = 0; i < 4; ++i) {
         const int64_t tiles = tiles_m * ((N + widths[i] - 1) / widths[i]), units = tiles * S;
         const double k = units > sm_count ? (double)(tiles * K) / sm_count : (double)seg;       // k steps of the longest block
-        const double cost = k * (double)((i == 0 ? bm : 128) * widths[i]) / rates[i];
+        const double rate = i == 3 && tm == 8 && units > sm_count ? 0.42 : rates[i];
+        const double cost = k * (double)((i == 0 ? bm : 128) * widths[i]) / rate;
         if (i == 0 || cost < best_cost) { best = widths[i]; best_cost = cost; }
     }
     return best;
