@@ -131,12 +131,12 @@ inline int64_t decode_segment(int64_t K, int S)
 }
 // FP32 weights: does the multiply loop of a tiling load a chunk ahead?  The loads of a segment's first chunk, all of them before the
 // first multiplication, then cost what the later chunks gain.  Times with against without, over the tilings of 161 shapes: segments of
-// 128 to 256 elements 1.05 to 1.3 (M = 10, N = 22402, K = 208 13.4 us, without 10.8); 512 on average 0.96 in tiles of 8 rows a warp (M =
-// 33, N = 6411, K = 880 18.6 and 21.0), 1.01 of 4; 768 0.91 and 0.97; 2048 0.82 and 0.89.  Up to four batch rows are bound by memory
+// 128 to 256 elements 1.05 to 1.3 (M = 10, N = 22402, K = 208 13.4 us, without 10.8); 384 and 512 on average 0.95 in tiles of 8 rows a
+// warp (M = 33, N = 6411, K = 880 18.6 and 21.0; M = 44, N = 22508, K = 264 35.0 and 38.6), 1.01 of 4; 768 0.91 and 0.97; 2048 0.82 and 0.89.  Up to four batch rows are bound by memory
 // and gain later: segments of 512 to 1024 1.03, from 2048 on 0.83 to 1.0.
 inline bool decode_loads_ahead(int rows_of_warp, int64_t M, int64_t K, int S)
 {
-    return decode_segment(K, S) >= (M <= 4 ? 2048 : rows_of_warp == 8 ? 512 : 768);
+    return decode_segment(K, S) >= (M <= 4 ? 2048 : rows_of_warp == 8 ? 257 : 768);
 }
 // map_w: box of a whole tile (rt * wr weight rows); map_g: of one row group (rt)
 cudaError_t launch_decode(const LaunchArgs& a, const DecodeConfig& cfg, const CUtensorMap* map_w, const CUtensorMap* map_g, const CUtensorMap* map_x);

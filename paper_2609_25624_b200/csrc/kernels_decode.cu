@@ -32,10 +32,13 @@ int m_class(int64_t M) { return M <= 1 ? 0 : M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 
 //   * 16-bit weights, more rows, K from 2560 on: 56 drawn and layer shapes, 9 to 64 rows, mean loss 2 % (3.5 % with the rates of few
 //     rows: M = 16, N = 4096, K = 14336 44.5 -> 41.6 us, M = 16, N = 2083, K = 14096 49.8 -> 42.6).  Shorter rows are a matter of
 //     latencies that these rates do not know (M = 16, N = 278, K = 2168 5.6 us, with the rates of few rows 4.8).
-//   * FP32 weights, segments of more than two chunks: 52 shapes at batch 1 .. 64, 2 % (24 % with the rates of few rows).
-// The last two only where the rates of few rows choose a tiling with more units than half the SMs.  With fewer, a block's rows and ring
-// decide, not rates: M = 12, N = 99, K = 5832 (16 units) 8.1 us, by the rates of many rows 10.8; M = 4, N = 97, K = 8552 with FP32 weights
-// (7) 11.4 and 14.9; but M = 10, N = 871, K = 7248 (126) 14.4 and 13.3, M = 36, N = 388, K = 8976 with FP32 weights (140) 26.4 and 21.1.
+//   * FP32 weights, segments of more than two chunks: 52 shapes at batch 1 .. 64, 2 % (24 % with the rates of few rows).  Shorter ones
+//     only in one wave of units of two chunks (M = 16, N = 1478, K = 440 3.8 us, by the rates of few rows 4.5) or in more than seven (M = 44, N =
+//     22508, K = 264 38.7 and 44.6); between them the rates of few rows are better (M = 10, N = 3225, K = 368 4.6 us, otherwise 5.4).
+// The last two only where the rates of few rows choose a tiling with more units than two thirds (16 bits) or half (FP32) of the SMs.
+// With fewer, a block's rows and ring decide, not rates: M = 12, N = 99, K = 5832 (16 units) 8.1 us, by the rates of many rows 10.8; M = 35, N =
+// 205, K = 5744 (75) 8.3 and 10.9; but M = 10, N = 871, K = 7248 (126) 14.4 and 13.3.  M = 4, N = 97, K = 8552 with FP32 weights (7) 11.4 and
+// 14.9, but M = 7, N = 1081, K = 4112 (78) 13.2 and 11.3, M = 36, N = 388, K = 8976 (140) 26.4 and 21.1.
 // Of 195 shapes of 16-bit weights none is then slower by more than 1.5 % than by the rates of many rows, of 144 of FP32 weights in long
 // segments none by more than 2.5 %.
 struct TilingRates {
@@ -155,8 +158,14 @@ bool decode_config_for(int64_t M, int64_t N, int64_t K, int S, int wfmt, int var
     if (variant == 0) {
         const bool fp32 = wfmt == DET_WEIGHT_FP32;
         choose(fp32 ? kRatesFp32Short : kRatesFewRows);
-        const TilingRates* better = fp32 ? (decode_segment(K, S) > 256 ? &kRatesFp32 : nullptr) : M > 8 && K >= 2560 ? &kRatesManyRows : nullptr;
-        if (better && pick >= 0 && tiling_units(class_table(wfmt, pick_cls)->entries[pick].cfg, M, N) > sms / 2) choose(*better);
+        if (pick >= 0) {
+            const int64_t units = tiling_units(class_table(wfmt, pick_cls)->entries[pick].cfg, M, N), seg = decode_segment(K, S);
+            if (!fp32) {
+                if (M > 8 && K >= 2560 && 3 * units > 2 * sms) choose(kRatesManyRows);
+            } else if ((seg > 256 && units > sms / 2) || (seg == 256 && units > sms / 2 && units <= sms) || units > 7 * sms) {
+                choose(kRatesFp32);
+            }
+        }
     } else {
         int seen = 0;
         for (int ci = 0; ci < n_classes && pick < 0; ++ci) {

@@ -10,7 +10,7 @@ from tests.gpu_util import KERNEL_DECODE, assert_bits_equal, decode_tilings, ora
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("M,N,K", [(3, 61, 128), (4, 85, 132), (5, 30, 260), (8, 113, 1156), (13, 57, 1028), (16, 225, 900), (33, 90, 516), (64, 29, 2048),
-                                   (3, 61, 4100), (8, 113, 1540), (13, 57, 1284), (16, 225, 2564), (33, 90, 1156), (12, 16400, 772)])
+                                   (3, 61, 4100), (8, 113, 1540), (13, 57, 1284), (16, 225, 2564), (33, 90, 1156), (12, 16400, 772), (20, 16400, 264)])
 def test_every_tiling(M, N, K):
     x, W, b = inputs.make_case_w(M, N, K, "fp32")
     want = oracle_y(x, W, b)

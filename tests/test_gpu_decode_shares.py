@@ -40,7 +40,7 @@ def every_tiling(M, N, K, wfmt):
 
 # one wave of at most a block an SM: small blocks
 @pytest.mark.gpu
-@pytest.mark.parametrize("M,N,K,wfmt", [(12, 99, 5832, "bf16"), (42, 89, 4416, "fp16"), (24, 246, 6112, "bf16"), (17, 59, 2704, "fp16")])
+@pytest.mark.parametrize("M,N,K,wfmt", [(12, 99, 5832, "bf16"), (42, 89, 4416, "fp16"), (24, 246, 6112, "bf16"), (35, 205, 5744, "bf16"), (17, 59, 2704, "fp16")])
 def test_tilings_of_few_units(M, N, K, wfmt):
     plan = B.det_linear_plan_w(M, N, K, wfmt)
     t = B.det_linear_plan_describe(plan)["decode_tiling"]
