@@ -18,8 +18,8 @@
 //   * a small layer is one wave of warps that wait for their own instructions: batch blocks of fewer rows and a warp per segment
 //     spread them over the SMs (decode_any_layout.cpp).
 // Measured on B200, us a call in a chain (in brackets a warp per row that walks it chunk by chunk, for every batch row again): M = 6, N =
-// 1333, K = 1001 4.7 (15.8); M = 3, N = K = 4097 14.3 (49.6); M = 64, N = 8192, K = 4097 218 (1705; 27 % of the FP32 peak: line-up and
-// widening of every weight in every batch block, one-word loads); M = 64, N = 300, K = 333 4.6 (68).
+// 1333, K = 1001 4.1 (15.8); M = 3, N = K = 4097 13.1 (49.6); M = 64, N = 8192, K = 4097 214 (1705; 27 % of the FP32 peak: line-up and
+// widening of every weight in every batch block, one-word loads); M = 64, N = 300, K = 333 4.1 (68).
 #include "internal.h"
 #include "device_utils.cuh"
 

@@ -55,8 +55,8 @@ static double layout_cost(const AnyLayout& l, int64_t M, int64_t N, int64_t K, i
 }
 
 // Fewer batch rows a warp than there are, where the layer leaves SMs idle otherwise (the weights then come from L2 for the other batch
-// blocks): M = 6, N = 1333, K = 1001 6.1 -> 4.7 us, M = 7, N = 250, K = 3001 with FP32 weights 10.1 -> 5.8; a warp a segment: M = 8, N = 64,
-// K = 4095 19.5 -> 6.8.  The largest batch block with one, two or four rows by the number of warps, the rule without this, keeps the calls
+// blocks): M = 6, N = 1333, K = 1001 6.4 -> 4.1 us, M = 7, N = 250, K = 3001 with FP32 weights 10.9 -> 5.3; a warp a segment: M = 8, N = 64,
+// K = 4095 19.7 -> 6.7.  The largest batch block with one, two or four rows by the number of warps, the rule without this, keeps the calls
 // that would not gain 3 %.
 AnyLayout any_layout_for(int64_t M, int64_t N, int64_t K, int S, int wfmt, int sms)
 {
